@@ -49,7 +49,7 @@ struct Shape {
 };
 
 // Launch shapes measured fastest on GB300 at 2^27-2^28 keys (insert with
-// dynamic chunk claims; load factors near each scheme's working range).
+// chunk claims; load factors near each scheme's working range).
 // Finds read 16-pair buckets fastest with two queries in flight per lane
 // and 32-pair buckets with one; builds the other way round, except the
 // keys-only set, fastest with one key per lane for both. BCHT reads a
@@ -396,19 +396,18 @@ struct ght_table {
 
 namespace {
 
-// Insert n pairs. The warps claim runs of 32-pair chunks from the control
-// block's work cursor, which must be zero at launch (the fill clears it), so
-// that the warps finish together however long the eviction chains of their
-// keys are; a static slice per warp left a slow tail of 15-30 % at 2^28 keys.
+// Insert n pairs (shares per warp: claim_plan). The control block's work
+// cursor must be zero at launch (the fill clears it). ordered: the pairs are
+// grouped, so the warps advance through them together.
 // past_first: the keys are the overflow of a first-choice placement, whose
 // H_0 buckets are full (the placement counted that visit), so a BCHT insert
 // starts them at H_1 instead of reading H_0 again and exchanging there.
 cudaError_t launch_insert(const ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n,
-                          bool past_first = false) {
+                          bool past_first = false, bool ordered = false) {
   ght::TableView tv = t->view();
   if (past_first && tv.h > 1 && (t->shape.scheme == GHT_BCHT || t->shape.scheme == GHT_BCHT_SET)) tv.first = 1;
   ght::LaunchOpts o = t->build_opts();
-  o.dynamic = true;
+  o.ordered = ordered;
   if (t->shape.scheme == GHT_BCHT) return ght::launch_insert_bcht(t->shape.b, tv, k, v, n, o, t->stream);
   if (t->shape.scheme == GHT_BCHT_SET) return ght::launch_insert_set(tv, k, v ? v : k, n, o, t->stream);
   return ght::launch_insert_other(t->shape.scheme, t->shape.b, tv, k, v, n, o, t->stream);
@@ -863,7 +862,7 @@ int build_device(ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n,
       cudaEventRecord(t->tev[2], t->stream);
     }
     if (in > 0) {
-      e = launch_insert(t, ik, iv, in, this_ranked);
+      e = launch_insert(t, ik, iv, in, this_ranked, grouped && !this_ranked);
       if (e != cudaSuccess) { rc = cuda_fail(e, "launching insert"); break; }
     }
     cudaEventRecord(t->tev[3], t->stream);

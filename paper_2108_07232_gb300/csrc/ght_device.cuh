@@ -33,7 +33,7 @@ struct Ctrl {
   unsigned long long find_probes;
   unsigned long long find_queries;
   unsigned long long longest_chain;
-  unsigned long long work_cursor;  // next input index claimed by a dynamic-chunk build
+  unsigned long long work_cursor;  // next input index claimed by an insert
   unsigned long long reserved[24];
 };
 static_assert(sizeof(Ctrl) == 256, "control block is 256 bytes");
@@ -88,6 +88,11 @@ __host__ __device__ __forceinline__ uint32_t select4(const uint32_t (&x)[4], int
 __host__ __device__ __forceinline__ uint32_t bucket_of(const HashFamily &hf, int i, uint32_t k) {
   return fastmod(mod_prime((uint64_t)select4(hf.a, i) * k + select4(hf.c, i)), hf.mod);
 }
+
+// Shares of an insert's input per warp (see claim_plan).
+struct ClaimPlan {
+  uint32_t first, claim;
+};
 
 // Everything a kernel needs to address a table; passed by value.
 struct TableView {

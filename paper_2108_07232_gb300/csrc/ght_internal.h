@@ -18,7 +18,7 @@ struct LaunchOpts {
   int keys_per_lane = 2;
   int blocks_per_sm = 0;
   bool count = false;    // probe counters
-  bool dynamic = false;  // build: warps claim 32-pair chunks from a global cursor
+  bool ordered = false;  // insert: the warps advance through the input together
   bool async_find = false;  // find: bucket parts staged in shared memory (BCHT, b = 16, 4-lane tiles)
 };
 
@@ -105,6 +105,37 @@ inline cudaError_t grid_for_smem(K kernel, int threads, size_t smem, uint64_t n,
 inline uint64_t per_warp_of(uint64_t n, int blocks) {
   const uint64_t warps = (uint64_t)blocks * (kThreads / 32);
   return (n + warps - 1) / warps;
+}
+
+// How the warps of an insert share its input of n pairs, in 32-pair chunks:
+// `first` chunks each, and what is left in runs of `claim` chunks claimed from
+// a global cursor (zero at launch), so that the warps finish together however
+// long the eviction chains of their keys are.
+//  * Up to 32 chunks a warp: an even share and no claims. Claims of 1024
+//    pairs, whatever n, gave 2^20 keys to 1024 warps of 3648 and 20,000 keys to
+//    20: BCHT at LF 0.9 took 137 us for 2^20 keys (now 85) and at LF 0.95 139
+//    us for 20,000 (now 67); at 2^21 keys the even share takes 116 us against
+//    159 with claims.
+//  * Beyond: three quarters shared evenly, the rest in about eight runs a warp
+//    (each claim is one atomic on one address, ~3 ns apart): 2^24 keys 747 ->
+//    712 us for BCHT at LF 0.95, 1191 -> 1091 for P2BHT and 1073 -> 922 for IHT
+//    at LF 0.8. (Half shared evenly and four runs: 817, 1165, 1040.)
+//  * ordered: the input order is a locality order (a grouped input, or a batch
+//    whose tables follow one another), so all warps advance together: claims
+//    only.
+inline ClaimPlan claim_plan(uint64_t n, int blocks, bool ordered) {
+  const uint64_t warps = (uint64_t)blocks * (kThreads / 32);
+  const uint64_t chunks = (n + 31) / 32;
+  ClaimPlan p;
+  if (chunks <= 32 * warps && !ordered) {
+    p.first = (uint32_t)((chunks + warps - 1) / warps);
+    p.claim = 1;
+  } else {
+    p.first = ordered ? 0u : (uint32_t)(chunks / warps * 3 / 4);
+    const uint64_t share = (chunks - p.first * warps) / (warps * 8);
+    p.claim = (uint32_t)(share < 1 ? 1 : (share > 32 ? 32 : share));
+  }
+  return p;
 }
 
 // Scratch of a two-phase (ranked placement) build: one arrival counter per

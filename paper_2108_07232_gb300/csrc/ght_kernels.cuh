@@ -19,48 +19,40 @@ namespace ght {
 
 // ----------------------------------------------------------------------------
 // Key and value streams of a build, read like StreamQueue, 32 pairs at a
-// time, two chunks ahead. Chunks are either consecutive pieces of the warp's
-// static slice, or (dynamic mode) claimed from a global cursor so that all
-// warps advance through the input together -- which keeps the in-flight
-// inserts of a grouped build inside a small window of the table.
+// time, two chunks ahead. A warp's chunks are first its own share of the
+// input (ClaimPlan::first chunks), then runs claimed from a global cursor.
 struct PairQueue {
   uint64_t ba, bb, bc;  // input index of entry 0 of chunks a, b, c (warp-uniform)
-  uint64_t claim_next;  // dynamic mode: next chunk of the warp's current claim
-  uint32_t claim_left;  // chunks left in that claim
+  uint64_t claim_next;  // next chunk of the warp's current run
+  uint32_t claim_left;  // chunks left in that run
   int head;             // next unused entry of chunk a
   uint32_t ka, kb, kc, va, vb, vc;
 };
 
-// Dynamic mode: a warp claims kClaimChunks consecutive 32-pair chunks at a
-// time from the global cursor (one atomic per claim, not per chunk).
-constexpr uint32_t kClaimChunks = 32;
-
-__device__ __forceinline__ uint64_t claim_chunk(PairQueue &q, Ctrl *ctrl, int lane) {
-  if (q.claim_left == 0) {
+// The next 32-pair chunk of this warp, past the end once the input is spent.
+// Chunks from `shared` on are claimed from `cursor`, relative to `shared`.
+__device__ __forceinline__ uint64_t claim_chunk(uint64_t &next, uint32_t &left, const ClaimPlan &plan,
+                                                uint64_t shared, uint64_t end, unsigned long long *cursor, int lane) {
+  if (left == 0) {
     unsigned long long x = 0ull;
-    if (lane == 0) x = atomicAdd(&ctrl->work_cursor, 32ull * kClaimChunks);
-    q.claim_next = __shfl_sync(kFull, x, 0);
-    q.claim_left = kClaimChunks;
+    if (lane == 0 && shared < end) x = atomicAdd(cursor, 32ull * plan.claim);
+    next = shared + __shfl_sync(kFull, x, 0);
+    left = plan.claim;
   }
-  const uint64_t at = q.claim_next;
-  q.claim_next += 32;
-  q.claim_left--;
+  const uint64_t at = next;
+  next += 32;
+  left--;
   return at;
 }
 
 __device__ __forceinline__ void pair_init(PairQueue &q, const uint32_t *__restrict__ k, const uint32_t *__restrict__ v,
-                                          uint64_t beg, uint64_t end, bool dynamic, Ctrl *ctrl, int lane) {
-  q.claim_next = 0;
-  q.claim_left = 0;
-  if (dynamic) {
-    q.ba = claim_chunk(q, ctrl, lane);
-    q.bb = claim_chunk(q, ctrl, lane);
-    q.bc = claim_chunk(q, ctrl, lane);
-  } else {
-    q.ba = beg;
-    q.bb = beg + 32;
-    q.bc = beg + 64;
-  }
+                                          const ClaimPlan &plan, uint64_t warp, uint64_t shared, uint64_t end,
+                                          Ctrl *ctrl, int lane) {
+  q.claim_next = warp * plan.first * 32ull;
+  q.claim_left = plan.first;
+  q.ba = claim_chunk(q.claim_next, q.claim_left, plan, shared, end, &ctrl->work_cursor, lane);
+  q.bb = claim_chunk(q.claim_next, q.claim_left, plan, shared, end, &ctrl->work_cursor, lane);
+  q.bc = claim_chunk(q.claim_next, q.claim_left, plan, shared, end, &ctrl->work_cursor, lane);
   q.head = 0;
   q.ka = stream_load(k, q.ba + lane, end);
   q.kb = stream_load(k, q.bb + lane, end);
@@ -73,8 +65,8 @@ __device__ __forceinline__ void pair_init(PairQueue &q, const uint32_t *__restri
 __device__ __forceinline__ bool pair_exhausted(const PairQueue &q, uint64_t end) { return q.ba + q.head >= end; }
 
 __device__ __forceinline__ uint64_t pair_take(PairQueue &q, const uint32_t *__restrict__ k,
-                                              const uint32_t *__restrict__ v, uint64_t end, bool dynamic,
-                                              Ctrl *ctrl, unsigned need, unsigned below, int lane,
+                                              const uint32_t *__restrict__ v, const ClaimPlan &plan,
+                                              uint64_t shared, uint64_t end, Ctrl *ctrl, unsigned need, unsigned below, int lane,
                                               uint32_t &key, uint32_t &val) {
   const int pos = q.head + __popc(need & below);
   const uint32_t ka = __shfl_sync(kFull, q.ka, pos & 31), kb = __shfl_sync(kFull, q.kb, pos & 31);
@@ -87,7 +79,7 @@ __device__ __forceinline__ uint64_t pair_take(PairQueue &q, const uint32_t *__re
     q.head -= 32;
     q.ba = q.bb;
     q.bb = q.bc;
-    q.bc = dynamic ? claim_chunk(q, ctrl, lane) : q.bc + 32;
+    q.bc = claim_chunk(q.claim_next, q.claim_left, plan, shared, end, &ctrl->work_cursor, lane);
     q.ka = q.kb;
     q.kb = q.kc;
     q.va = q.vb;
@@ -120,7 +112,7 @@ __device__ __forceinline__ uint64_t pair_take(PairQueue &q, const uint32_t *__re
 //
 // Each lane runs KPL independent slots. A slot's atomic result is inspected
 // only on the slot's next turn, so with KPL = 2 its latency is hidden behind
-// the other slot's bucket reads. per_warp = 0 selects dynamic chunks.
+// the other slot's bucket reads.
 //
 // Minimum resident blocks per SM the insert is compiled for (0: the
 // compiler's choice). The insert is latency-bound, so resident warps matter:
@@ -137,7 +129,7 @@ constexpr int insert_min_blocks() {
 template <int SCHEME, int B, int G, int KPL, bool COUNT, typename S = PairSlot>
 __global__ void __launch_bounds__(256, insert_min_blocks<B, G, KPL, COUNT>())
 bucketed_insert_kernel(TableView tv, const uint32_t *__restrict__ keys,
-                       const uint32_t *__restrict__ values, uint64_t n, uint64_t per_warp) {
+                       const uint32_t *__restrict__ values, uint64_t n, ClaimPlan plan) {
   using T = typename S::T;
   constexpr int PPL = B / G;
   T *slots = reinterpret_cast<T *>(tv.slots);
@@ -148,16 +140,15 @@ bucketed_insert_kernel(TableView tv, const uint32_t *__restrict__ keys,
   const unsigned tmask = (G == 32 ? kFull : ((1u << G) - 1u)) << tbase;
   const uint64_t gtid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const uint64_t warp = gtid >> 5;
-  const bool dynamic = per_warp == 0;
-  const uint64_t beg = dynamic ? 0 : warp * per_warp;
-  if (beg >= n) return;  // whole warp
-  const uint64_t end = dynamic ? n : (beg + per_warp < n ? beg + per_warp : n);
+  const uint64_t end = n;
+  // input from here on is claimed chunk by chunk
+  const uint64_t shared = (uint64_t)gridDim.x * (blockDim.x >> 5) * plan.first * 32ull;
   const unsigned below = lanemask_lt();
   const int h = tv.h;
 
   uint32_t rng = lane_seed(tv.rng_seed, gtid);
   PairQueue pq;
-  pair_init(pq, keys, values, beg, end, dynamic, tv.ctrl, lane);
+  pair_init(pq, keys, values, plan, warp, shared, end, tv.ctrl, lane);
   // per-slot state
   bool active[KPL], retrying[KPL];
   T pair[KPL], old[KPL];
@@ -235,7 +226,7 @@ bucketed_insert_kernel(TableView tv, const uint32_t *__restrict__ keys,
       const unsigned need = __ballot_sync(kFull, !active[s]);
       if (need != 0u && !pair_exhausted(pq, end)) {
         uint32_t k, val;
-        const uint64_t at = pair_take(pq, keys, values, end, dynamic, tv.ctrl, need, below, lane, k, val);
+        const uint64_t at = pair_take(pq, keys, values, plan, shared, end, tv.ctrl, need, below, lane, k, val);
         if (at < end) {
           if (k == kEmptyKey) {
             atomicOr(&tv.ctrl->status, kStatusSentinel);

@@ -94,9 +94,8 @@ __device__ __forceinline__ void bq_init(BatchQueue &q, const uint32_t *__restric
 }
 
 // Key/value stream of the batched insert: 32-pair chunks claimed from the
-// batch's work cursor (runs of kClaimChunks chunks per claim, as in the
-// single-table insert), each with the table of its first pair, kept two
-// chunks ahead of use.
+// batch's work cursor (all warps stay on the few tables the cursor is in),
+// each with the table of its first pair, kept two chunks ahead of use.
 struct BatchClaimQueue {
   uint64_t ba, bb, bc;  // index of entry 0 of chunks a, b, c (warp-uniform)
   uint64_t claim_next;  // next chunk of the warp's current claim
@@ -106,28 +105,16 @@ struct BatchClaimQueue {
   uint32_t ka, kb, kc, va, vb, vc;
 };
 
-__device__ __forceinline__ uint64_t bc_claim(BatchClaimQueue &q, Ctrl *ctrl, uint64_t lo, int lane) {
-  if (q.claim_left == 0) {
-    unsigned long long x = 0ull;
-    if (lane == 0) x = atomicAdd(&ctrl->work_cursor, 32ull * kClaimChunks);
-    q.claim_next = lo + __shfl_sync(kFull, x, 0);
-    q.claim_left = kClaimChunks;
-  }
-  const uint64_t at = q.claim_next;
-  q.claim_next += 32;
-  q.claim_left--;
-  return at;
-}
-
 __device__ __forceinline__ void bc_init(BatchClaimQueue &q, const uint32_t *__restrict__ keys,
-                                        const uint32_t *__restrict__ vals, uint64_t lo, uint64_t hi,
-                                        const BatchView &bv, const uint64_t *__restrict__ offs, int lane) {
-  q.claim_next = 0;
-  q.claim_left = 0;
+                                        const uint32_t *__restrict__ vals, const ClaimPlan &plan, uint64_t warp,
+                                        uint64_t lo, uint64_t shared, uint64_t hi, const BatchView &bv,
+                                        const uint64_t *__restrict__ offs, int lane) {
+  q.claim_next = lo + warp * plan.first * 32ull;
+  q.claim_left = plan.first;
   q.head = 0;
-  q.ba = bc_claim(q, bv.ctrl, lo, lane);
-  q.bb = bc_claim(q, bv.ctrl, lo, lane);
-  q.bc = bc_claim(q, bv.ctrl, lo, lane);
+  q.ba = claim_chunk(q.claim_next, q.claim_left, plan, shared, hi, &bv.ctrl->work_cursor, lane);
+  q.bb = claim_chunk(q.claim_next, q.claim_left, plan, shared, hi, &bv.ctrl->work_cursor, lane);
+  q.bc = claim_chunk(q.claim_next, q.claim_left, plan, shared, hi, &bv.ctrl->work_cursor, lane);
   bq_load<true>(q.ka, q.va, q.ta, keys, vals, q.ba, hi, bv, offs, lane);
   bq_load<true>(q.kb, q.vb, q.tb, keys, vals, q.bb, hi, bv, offs, lane);
   bq_load<true>(q.kc, q.vc, q.tc, keys, vals, q.bc, hi, bv, offs, lane);
@@ -136,9 +123,10 @@ __device__ __forceinline__ void bc_init(BatchClaimQueue &q, const uint32_t *__re
 // Hand the next popc(need) pairs to the lanes in `need`; returns the pair's
 // index (~0 for lanes without one) and its table.
 __device__ __forceinline__ uint64_t bc_take(BatchClaimQueue &q, const uint32_t *__restrict__ keys,
-                                            const uint32_t *__restrict__ vals, uint64_t lo, uint64_t hi,
-                                            const BatchView &bv, const uint64_t *__restrict__ offs, unsigned need,
-                                            unsigned below, int lane, uint32_t &key, uint32_t &val, uint32_t &table) {
+                                            const uint32_t *__restrict__ vals, const ClaimPlan &plan, uint64_t shared,
+                                            uint64_t hi, const BatchView &bv, const uint64_t *__restrict__ offs,
+                                            unsigned need, unsigned below, int lane, uint32_t &key, uint32_t &val,
+                                            uint32_t &table) {
   const int pos = q.head + __popc(need & below);
   const uint32_t ka = __shfl_sync(kFull, q.ka, pos & 31), kb = __shfl_sync(kFull, q.kb, pos & 31);
   const uint32_t va = __shfl_sync(kFull, q.va, pos & 31), vb = __shfl_sync(kFull, q.vb, pos & 31);
@@ -151,7 +139,7 @@ __device__ __forceinline__ uint64_t bc_take(BatchClaimQueue &q, const uint32_t *
     q.head -= 32;
     q.ba = q.bb;
     q.bb = q.bc;
-    q.bc = bc_claim(q, bv.ctrl, lo, lane);
+    q.bc = claim_chunk(q.claim_next, q.claim_left, plan, shared, hi, &bv.ctrl->work_cursor, lane);
     q.ka = q.kb;
     q.kb = q.kc;
     q.va = q.vb;
@@ -182,7 +170,8 @@ __global__ void __launch_bounds__(256) batch_fill_kernel(BatchView bv, uint4 *__
 // key-word gathers and register bound of the single-table insert kernel.
 template <int G, int KPL, bool COUNT>
 __global__ void __launch_bounds__(256, insert_min_blocks<16, G, KPL, COUNT>())
-batch_insert_kernel(BatchView bv, const uint32_t *__restrict__ keys, const uint32_t *__restrict__ values) {
+batch_insert_kernel(BatchView bv, const uint32_t *__restrict__ keys, const uint32_t *__restrict__ values,
+                    ClaimPlan plan) {
   constexpr int B = 16;
   constexpr int PPL = B / G;
   static_assert(B % G == 0 && 32 % G == 0 && (KPL == 1 || KPL == 2), "tile shape");
@@ -196,9 +185,11 @@ batch_insert_kernel(BatchView bv, const uint32_t *__restrict__ keys, const uint3
   const unsigned below = lanemask_lt();
   const int h = bv.h;
 
+  const uint64_t shared = lo + (uint64_t)gridDim.x * (blockDim.x >> 5) * plan.first * 32ull;
+
   uint32_t rng = lane_seed(bv.rng_seed, gtid);
   BatchClaimQueue q;
-  bc_init(q, keys, values, lo, hi, bv, offs, lane);
+  bc_init(q, keys, values, plan, gtid >> 5, lo, shared, hi, bv, offs, lane);
   bool active[KPL], retrying[KPL];
   uint64_t pair[KPL], old[KPL];
   uint32_t cur[KPL], chain[KPL], steps[KPL], tab[KPL];
@@ -245,7 +236,7 @@ batch_insert_kernel(BatchView bv, const uint32_t *__restrict__ keys, const uint3
       const unsigned need = __ballot_sync(kFull, !active[s]);
       if (need != 0u && q.ba + q.head < hi) {
         uint32_t k, val, tb;
-        const uint64_t at = bc_take(q, keys, values, lo, hi, bv, offs, need, below, lane, k, val, tb);
+        const uint64_t at = bc_take(q, keys, values, plan, shared, hi, bv, offs, need, below, lane, k, val, tb);
         if (at != ~0ull) {
           if (k == kEmptyKey) {
             atomicOr(&bv.tables[tb].status, kStatusSentinel);
@@ -647,7 +638,7 @@ static cudaError_t insert_cfg(const BatchView &bv, const uint32_t *k, const uint
   int blocks = 0;
   cudaError_t e = grid_for(kern, items, o.blocks_per_sm, &blocks);
   if (e != cudaSuccess) return e;
-  kern<<<blocks, kThreads, 0, s>>>(bv, k, v);  // claims from bv.ctrl->work_cursor, zeroed by the fill
+  kern<<<blocks, kThreads, 0, s>>>(bv, k, v, claim_plan(items, blocks, true));  // the fill zeroed the claim cursor
   return cudaGetLastError();
 }
 

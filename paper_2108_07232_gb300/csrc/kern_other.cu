@@ -37,7 +37,7 @@ static cudaError_t insert_kpl(const TableView &tv, const uint32_t *k, const uint
   int blocks = 0;
   cudaError_t e = grid_for(kern, n, o.blocks_per_sm, &blocks);
   if (e != cudaSuccess) return e;
-  kern<<<blocks, kThreads, 0, s>>>(tv, k, v, n, o.dynamic ? 0 : per_warp_of(n, blocks));
+  kern<<<blocks, kThreads, 0, s>>>(tv, k, v, n, claim_plan(n, blocks, o.ordered));
   return cudaGetLastError();
 }
 
