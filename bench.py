@@ -161,7 +161,7 @@ class ClockSampler:
 # identified by a hash of the find kernel's headers; after any change to them
 # the traffic is reported as null.
 FIND_TRAFFIC = {"bytes_per_launch": 60460572544, "source_sha256_16": "d0a797b09e952b68",
-               "kernel": "bcht_find_async_kernel"}
+               "kernel": "bcht_find_async_kernel"}  # --find-async 1
 
 
 def build_kernels(st: dict) -> list[str]:
@@ -178,20 +178,23 @@ def build_kernels(st: dict) -> list[str]:
     return ks + ["bucketed_insert_kernel"]
 
 
-def find_kernels(st: dict) -> list[str]:
-    """The library kernels one find launches, from the table's stats."""
+def find_kernels(st: dict, line: bool = False) -> list[str]:
+    """The library kernels one find launches, from the table's stats; line: the
+    table's config names no find shape (tile_lanes, keys_per_lane, find_async)."""
     if st["last_find_grouped"]:  # per round: two groupings and the lookup; then the return to query order
         rnd = ["region_cursors_kernel", "group_scatter_kernel", "region_cursors_kernel", "group_scatter_kernel",
                "grouped_lookup_kernel"]
         return rnd * st["num_hashes"] + ["grouped_spill_kernel"] + ["region_cursors_kernel", "group_scatter_kernel"] * 2 \
             + ["window_write_kernel"]
+    if line:
+        return ["line_find_kernel"]
     return ["bcht_find_async_kernel" if st["find_staged"] else "bucketed_find_kernel"]
 
 
 def kernel_source_hash() -> str:
     import hashlib
     h = hashlib.sha256()
-    for f in ("ght_find.cuh", "ght_find_async.cuh", "ght_device.cuh"):
+    for f in ("ght_find.cuh", "ght_find_line.cuh", "ght_device.cuh"):
         with open(os.path.join(ROOT, "paper_2108_07232_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -354,6 +357,9 @@ def run_ours(args, world, rank, local):
     phase_ms = {f"{op}@{lf}": [] for lf in LFS
                 for op in ("fill", "group", "split", "place", "insert", "find_pos", "find_neg")}
 
+    # the config names no other find shape than BCHT's default
+    line_find = not args.find_async and args.tile_lanes in (0, 4) and args.keys_per_lane in (0, 2)
+
     def step(record: bool):
         for lf in LFS:
             t = tables[lf]
@@ -368,7 +374,7 @@ def run_ours(args, world, rank, local):
             e1.record()
             t.find(neg, out)
             e2.record()
-            launches[0] += 2 * len(find_kernels(t.stats()))
+            launches[0] += 2 * len(find_kernels(t.stats(), line_find))
             if record:
                 phase_ms[f"fill@{lf}"].append(st["last_fill_ms"])
                 phase_ms[f"group@{lf}"].append(max(st["last_group_ms"], 0.0))
@@ -489,7 +495,7 @@ def run_ours(args, world, rank, local):
     st0 = st_dev
     bks = build_kernels(st0)
     has_fill = "fill_kernel" in bks  # else the placement writes every line: no fill to rate
-    find_name = "+".join(dict.fromkeys(find_kernels(st0)))
+    find_name = "+".join(dict.fromkeys(find_kernels(st0, line_find)))
     for lf in LFS:
         # a build's work after the fill: the grouping (one or two levels) and
         # the ranked placement (when the build does them) and the cuckoo

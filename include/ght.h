@@ -89,8 +89,12 @@ typedef struct {
   /* Launch shapes (0 = tuned default). Find: lanes that read one bucket
    * together (4, 8 or 16; 8 or 16 for 32-pair buckets; 8 for schemes other
    * than BCHT; 4 for the staged find, see find_async), queries each lane
-   * keeps in flight (1 or 2; 2..8 for the staged find), blocks per SM.
-   * Build: the same three for the insert kernel. */
+   * keeps in flight (1 or 2; 2..8 for the staged find), blocks per SM. With
+   * find_async 0 and tile_lanes and keys_per_lane 0 or as
+   * ght_default_config gives them, 128-byte buckets are read by the line find
+   * (32-byte loads, one query per lane, queries that need another bucket
+   * refill the warp), which is faster at every size; other values select the
+   * register or staged find. Build: the same three for the insert kernel. */
   int32_t tile_lanes;
   int32_t blocks_per_sm;
   int32_t keys_per_lane;
@@ -181,7 +185,8 @@ typedef struct {
   int32_t last_build_ranked;   /* 1 if the last build was two-phase (ranked placement first) */
   double last_place_ms;        /* device time of its ranked placement (-1 if not two-phase) */
   uint64_t place_overflow;     /* keys the ranked placement left to the cuckoo insert */
-  int32_t find_staged;         /* 1 if finds stage bucket parts in shared memory (find_async) */
+  int32_t find_staged;         /* find_async as resolved: 1 if tile_lanes and keys_per_lane are the staged find's
+                                  (which runs where the config names them, the line find where it does not) */
   int32_t last_build_split;    /* 1 if the last build split its groups into 64 KB sub-groups and placed
                                   each whole in shared memory (block placement, no table fill) */
   /* host-to-device copies of the last ght_build_host / ght_find_host call:

@@ -41,6 +41,7 @@ struct Shape {
   int group_build;  // 1: group the input by first-choice bucket range before inserting
   int ranked_build;  // 1: two-phase build (ranked first-choice placement, then cuckoo insert)
   int find_async;    // 1: finds stage bucket parts in shared memory (BCHT b = 16, the set)
+  int find_line;     // 1: the config names no find shape of its own: the line find
   int check_dups;    // 1: a successful build checks that no key is stored twice
   int slot_bytes;   // 8 (key/value pair) or 4 (keys-only set)
   uint32_t max_steps;  // per-key step bound of the insert kernels (0: derived)
@@ -196,6 +197,13 @@ int resolve(int scheme, uint64_t capacity, double lf, const ght_config *user, Sh
   s->ranked_build = (scheme == GHT_BCHT || scheme == GHT_BCHT_SET) ? d.ranked_build : -1;
   s->slot_bytes = (int)slot_bytes;
   s->find_async = async_find ? 1 : 0;
+  // the line find, unless the config names another find shape than the scheme's default
+  ght_config shape0;
+  memset(&shape0, 0, sizeof shape0);
+  default_shape(scheme, b, &shape0);
+  const bool named = d.find_async != 0 || (user_tile && user->tile_lanes != shape0.tile_lanes) ||
+                     (kpl_given && user->keys_per_lane != shape0.keys_per_lane);
+  s->find_line = (uint64_t)b * slot_bytes == 128 && !named ? 1 : 0;
   s->check_dups = d.check_duplicates > 0 ? 1 : 0;
   s->max_steps = d.max_steps;
   s->find_grouped = grouped_shape ? d.find_grouped : -1;
@@ -698,6 +706,17 @@ cudaError_t launch_find(const ght_table *t, const uint32_t *q, uint32_t *out, ui
     }
   }
   const ght::TableView tv = t->view();
+  if (t->shape.find_line) {
+    ght::LaunchOpts o = t->find_opts();
+    // Three blocks (24 warps) per SM on tables from 1.5x the L2, whose finds
+    // DRAM's random lines bound and more warps only crowd (2^26 keys at LF 0.9
+    // 1990 us against 2160 with four, 2^28 present 9250 / 9530); as many as fit
+    // (four) below, where latency counts (2^24 keys, 141 MB: 312 us against 345
+    // with three).
+    if (o.blocks_per_sm == 0 && 2 * t->storage_bytes >= 3 * device_l2_bytes()) o.blocks_per_sm = 3;
+    const bool early = t->shape.scheme == GHT_BCHT || t->shape.scheme == GHT_BCHT_SET;
+    return ght::launch_find_line(t->shape.slot_bytes == 4, tv, q, out, n, early, o, t->stream);
+  }
   if (t->shape.scheme == GHT_BCHT) {
     const ght::LaunchOpts o = t->find_opts();
     return o.async_find ? ght::launch_find_bcht_async(t->shape.b, tv, q, out, n, o, t->stream)

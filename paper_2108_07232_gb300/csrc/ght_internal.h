@@ -121,13 +121,14 @@ inline uint64_t per_warp_of(uint64_t n, int blocks) {
 //    712 us for BCHT at LF 0.95, 1191 -> 1091 for P2BHT and 1073 -> 922 for IHT
 //    at LF 0.8. (Half shared evenly and four runs: 817, 1165, 1040.)
 //  * ordered: the input order is a locality order (a grouped input, or a batch
-//    whose tables follow one another), so all warps advance together: claims
-//    only.
+//    whose tables follow one another), so beyond 8 chunks a warp (0.9 M pairs,
+//    whose buckets the L2 holds in any order) all warps advance together:
+//    claims only.
 inline ClaimPlan claim_plan(uint64_t n, int blocks, bool ordered) {
   const uint64_t warps = (uint64_t)blocks * (kThreads / 32);
   const uint64_t chunks = (n + 31) / 32;
   ClaimPlan p;
-  if (chunks <= 32 * warps && !ordered) {
+  if (chunks <= (ordered ? 8 : 32) * warps) {
     p.first = (uint32_t)((chunks + warps - 1) / warps);
     p.claim = 1;
   } else {
@@ -169,6 +170,9 @@ cudaError_t launch_find_bcht_async(int B, const TableView &tv, const uint32_t *q
                                    const LaunchOpts &o, cudaStream_t s, bool early_exit = true);
 cudaError_t launch_find_set_async(const TableView &tv, const uint32_t *q, uint32_t *out, uint64_t n,
                                   const LaunchOpts &o, cudaStream_t s);
+// kern_find.cu: the find with 32-byte loads (128-byte buckets of any scheme; see ght_find_line.cuh)
+cudaError_t launch_find_line(bool key_slots, const TableView &tv, const uint32_t *q, uint32_t *out, uint64_t n,
+                             bool early_exit, const LaunchOpts &o, cudaStream_t s);
 bool bcht_shape_supported(int B, int G);
 
 // kern_set.cu (keys-only BCHT, 32 four-byte keys per bucket)

@@ -46,3 +46,29 @@ def _check(G, scheme, n, lf, seed, n_queries=None, **cfg):
                                          ("iht", 0.8, 3735553), ("p2bht", 0.75, 5000011)])
 def test_insert_shares(G, scheme, lf, n):
     _check(G, scheme, n, lf, seed=n & 0xFFFF)
+
+
+# around a chunk of 32 queries, a block's 256, and past one chunk per resident warp (4864 x 32)
+@pytest.mark.parametrize("nq", [1, 31, 32, 33, 257, 155648, 155649, 700001])
+@pytest.mark.parametrize("scheme,b,lf", [("bcht", 16, 0.99), ("p2bht", 16, 0.8), ("iht", 16, 0.8),
+                                         ("bcht_lb", 16, 0.9), ("bcht_set", 32, 0.99)])
+def test_line_find(G, scheme, b, lf, nq):
+    """The default find: answers, sentinel queries and exact probe counts."""
+    n = 20011
+    keys, vals = W.make_keys(n, 7), W.make_values(n, 7)
+    t = G.HashTable(scheme, n, lf, seed=11, count_probes=1, bucket_size=b)
+    t.build(keys.cuda(), None if scheme == "bcht_set" else vals.cuda())
+    q = W.make_queries(keys, nq, 0.5, seed=nq)
+    q[nq // 2::97] = -1
+    t.reset_counters()
+    got = O._u32(t.find(q.cuda()).cpu())
+    want = O.lookup(keys, vals, q)
+    if scheme == "bcht_set":
+        want = (want != O.EMPTY).astype(want.dtype)
+    assert (got == want).all()
+    st = t.stats()
+    assert st["find_queries"] == nq
+    if scheme != "bcht_set":
+        T = O.Table(G.SCHEMES[scheme], n, lf, b=b, m=st["num_buckets"])
+        T.set_constants(st["hash_a"], st["hash_c"])
+        assert st["find_probes"] == T.find(q, slots=t.export())[2]
