@@ -442,7 +442,8 @@ int ght_batch_run(ght_batch *b, const uint32_t *d_keys, const uint32_t *d_values
 
 /* Choose the insert and find launch shapes by timing each candidate on
  * these arrays: first the tile shape (lanes per bucket tile, keys per lane;
- * for finds also 4-lane tiles with 6 query sets per lane, the staged find
+ * for finds 4 lanes and one query per lane is the line find, the default, and
+ * 4-lane tiles with 6 query sets per lane the staged find
  * whose bucket parts wait in shared memory), then the grid (1-4 resident
  * blocks per SM, or as many as fit) of the best shape; keeps the fastest.
  * The tables are rebuilt as a side effect. */

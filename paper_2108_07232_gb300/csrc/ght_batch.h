@@ -27,8 +27,9 @@ struct BatchView {
 };
 
 bool batch_shape_supported(int tile_lanes, int keys_per_lane);
-// Find shapes: the above, and 4-lane tiles with 6 query sets per lane (the
-// staged find: bucket parts in shared memory).
+// Find shapes: the above, of which 4-lane tiles with one query per lane are the
+// line find (32-byte loads, the default), and 4-lane tiles with 6 query sets
+// per lane (the staged find: bucket parts in shared memory).
 bool batch_find_shape_supported(int tile_lanes, int keys_per_lane);
 
 // Describe a built single BCHT table (b = 16) as a batch descriptor (ght_api.cu).

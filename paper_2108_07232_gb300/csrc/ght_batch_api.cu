@@ -180,7 +180,7 @@ ght_batch *ght_batch_create(uint32_t num_tables, const uint64_t *h_capacities, c
   b->T = num_tables;
   b->seed = seed;
   b->find_o.tile_lanes = 4;
-  b->find_o.keys_per_lane = 2;
+  b->find_o.keys_per_lane = 1;  // the line find
   b->build_o.tile_lanes = 16;
   b->build_o.keys_per_lane = 1;
   if (cfg) {
@@ -396,7 +396,7 @@ int ght_batch_autotune(ght_batch *b, const uint32_t *d_keys, const uint32_t *d_v
   // tile shapes (lanes per bucket, keys per lane), then the grid (resident
   // blocks per SM; 0 = as many as fit) of the chosen shape
   static const int kBuild[][2] = {{16, 1}, {8, 1}, {8, 2}, {4, 2}};
-  static const int kFind[][2] = {{4, 2}, {4, 1}, {8, 2}, {8, 1}, {16, 1}, {4, 6}};  // {4, 6}: the staged find
+  static const int kFind[][2] = {{4, 1}, {4, 2}, {8, 2}, {8, 1}, {16, 1}, {4, 6}};  // the line find first; {4, 6}: staged
   static const int kGrid[] = {0, 1, 2, 3, 4};
   if (b->build_o.blocks_per_sm < 0 || b->find_o.blocks_per_sm < 0) return fail(GHT_ERR_INVALID_ARG, "negative grid");
   auto time_between = [&](float *out_ms) -> int {

@@ -9,6 +9,7 @@
 // uniform binary search per 32 items) and reads that table's descriptor.
 #include "ght_batch.h"
 #include "ght_find_async.cuh"
+#include "ght_find_line.cuh"
 #include "ght_kernels.cuh"
 
 namespace ght {
@@ -446,6 +447,125 @@ batch_find_kernel(BatchView bv, const uint32_t *__restrict__ queries, uint32_t *
 }
 
 // ----------------------------------------------------------------------------
+constexpr int kBatchTableBits = 30;  // a waiting query's table, below its next probe (h <= 4)
+
+// As table_of for an index a little beyond table tb's first: steps double from tb.
+__device__ __forceinline__ uint32_t seek_table(const uint64_t *__restrict__ offs, uint32_t tb, uint32_t t_hi,
+                                               uint64_t i) {
+  uint32_t step = 1;
+  while (tb + step < t_hi && __ldg(offs + tb + step) <= i) {
+    tb += step;
+    step *= 2;
+  }
+  return table_of(offs, tb, min(tb + step, t_hi), i);
+}
+
+// The same find with 32-byte loads (the line find, ght_find_line.cuh): 32
+// queries per step, those that need another bucket wait in shared memory with
+// their table. A step's queries are consecutive, so their tables are found by
+// walking on from the last step's first table, and the descriptors come from
+// L1.
+//
+// The warps take the chunks of 32 queries in turn, so that all of them are in
+// the same few tables, whose lines then stay in the L2; a slice of the batch
+// per warp, as the register find has, keeps every table in use at once (and
+// the reads in DRAM). Find of 512 tables of 2^10..2^20 keys (85 M keys, 171 M
+// queries, half present): 13.5 ms (register find, two queries per lane; one:
+// 11.2) -> 2.5 ms; 64 tables of 2^12..2^22 keys (87 M queries) 6.5 -> 1.3 ms;
+// 512 tables of 2^10..2^14 keys (6 M queries, all in the L2) 0.30 -> 0.12 ms.
+template <bool COUNT>
+__global__ void __launch_bounds__(kLineFindThreads, 4)
+batch_line_find_kernel(BatchView bv, const uint32_t *__restrict__ queries, uint32_t *__restrict__ out,
+                       uint32_t n) {
+  __shared__ uint2 s_wait[kLineFindWarps][kLineFindWaiting];
+  __shared__ uint32_t s_table[kLineFindWarps][kLineFindWaiting];
+  const uint64_t *offs = bv.query_offs;
+  const int lane = threadIdx.x & 31;
+  const int r = lane & (kLineFindLanes - 1);
+  const int tbase = lane - r;
+  const unsigned below = lanemask_lt();
+  uint2 *wait = s_wait[threadIdx.x >> 5];
+  uint32_t *wait_table = s_table[threadIdx.x >> 5];
+  const uint32_t step = gridDim.x * kLineFindThreads;
+  const uint32_t start = blockIdx.x * kLineFindThreads + (threadIdx.x & ~31u);
+  if (start >= n) return;  // whole warp
+  const uint64_t lo = __ldg(offs + bv.t_lo);
+  queries += lo;
+  out += lo;
+  int waiting = 0;
+  unsigned long long probes = 0, answered = 0;
+  uint32_t first = table_of(offs, bv.t_lo, bv.t_hi, lo + start);  // table of the next step's first query
+  uint32_t next = __ldg(queries + min(start + lane, n - 1u));
+  for (uint32_t c = start;;) {
+    uint32_t k, at, tb;
+    int probe;
+    bool valid;
+    if (waiting >= 32 || c >= n) {
+      if (waiting == 0) break;
+      const int take = min(waiting, 32);
+      waiting -= take;
+      const uint2 e = wait[waiting + min(lane, take - 1)];
+      const uint32_t tp = wait_table[waiting + min(lane, take - 1)];
+      k = e.x;
+      at = e.y;
+      tb = tp & ((1u << kBatchTableBits) - 1u);
+      probe = (int)(tp >> kBatchTableBits);
+      valid = lane < take;
+      __syncwarp();  // read before the step's own entries go there
+    } else {
+      k = next;
+      at = c + lane;
+      probe = 0;
+      tb = advance_table(offs, first, bv.t_hi, lo + min(at, n - 1u));
+      if (c < n - min(n, step)) {
+        c += step;
+        next = __ldg(queries + min(c + lane, n - 1u));
+        first = seek_table(offs, first, bv.t_hi, lo + c);
+      } else {
+        c = n;
+      }
+      valid = at < n && k != kEmptyKey;
+      if (COUNT && at < n) answered++;
+      if (at < n && k == kEmptyKey) out[at] = kEmptyKey;  // the sentinel is never a key
+    }
+    const BatchTable &d = bv.tables[tb];
+    FastMod mod;
+    mod.M = __ldg(reinterpret_cast<const unsigned long long *>(&d.mod.M));
+    mod.d = __ldg(&d.mod.d);
+    const uint32_t b = fastmod(mod_prime((uint64_t)__ldg(&d.a[probe]) * k + __ldg(&d.c[probe])), mod);
+    const uint64_t bucket =
+        __ldg(reinterpret_cast<const unsigned long long *>(&d.slots)) + (uint64_t)b * (16u * sizeof(uint64_t));
+    bool hit, empty;
+    uint32_t value;
+    line_probe<PairSlot, true>(
+        k, r, tbase, lane,
+        [&](int j, uint32_t(&x)[8]) {
+          load32_ro(reinterpret_cast<const char *>(__shfl_sync(kFull, bucket, tbase + j)) + r * 32, x);
+        },
+        hit, empty, value);
+    if (COUNT && valid) probes++;
+    const bool more = valid && !hit && !empty && probe + 1 < bv.h;
+    if (valid && !more) out[at] = hit ? value : kEmptyKey;
+    const unsigned mb = __ballot_sync(kFull, more);
+    if (more) {
+      const int i = waiting + __popc(mb & below);
+      wait[i] = make_uint2(k, at);
+      wait_table[i] = tb | ((uint32_t)(probe + 1) << kBatchTableBits);
+    }
+    waiting += __popc(mb);
+    __syncwarp();
+  }
+  if (COUNT) {
+    probes = warp_sum(probes);
+    answered = warp_sum(answered);
+    if (lane == 0) {
+      atomicAdd(&bv.ctrl->find_probes, probes);
+      atomicAdd(&bv.ctrl->find_queries, answered);
+    }
+  }
+}
+
+// ----------------------------------------------------------------------------
 // The same find with the bucket parts staged in shared memory (the staged
 // find of the single-table path, ght_find_async.cuh): 4-lane tiles, KPL
 // query sets per lane in flight, each set's buckets copied by cp.async (two
@@ -724,6 +844,17 @@ static cudaError_t find_staged(const BatchView &bv, const uint32_t *q, uint32_t 
   return cudaGetLastError();
 }
 
+static cudaError_t find_lines(const BatchView &bv, const uint32_t *q, uint32_t *out, uint64_t items,
+                              const LaunchOpts &o, cudaStream_t s) {
+  if (items > 0xFFFF0000ull) return find_cfg<4, 2>(bv, q, out, items, o, s);  // 32-bit places
+  auto kern = o.count ? batch_line_find_kernel<true> : batch_line_find_kernel<false>;
+  int blocks = 0;
+  const cudaError_t e = grid_for(kern, items, o.blocks_per_sm, &blocks);
+  if (e != cudaSuccess) return e;
+  kern<<<blocks, kLineFindThreads, 0, s>>>(bv, q, out, (uint32_t)items);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_batch_insert(const BatchView &bv, const uint32_t *k, const uint32_t *v, uint64_t items,
                                 const LaunchOpts &o, cudaStream_t s) {
   if (items == 0) return cudaSuccess;
@@ -741,7 +872,7 @@ cudaError_t launch_batch_find(const BatchView &bv, const uint32_t *q, uint32_t *
   if (g == 16) return kpl == 1 ? find_cfg<16, 1>(bv, q, out, items, o, s) : find_cfg<16, 2>(bv, q, out, items, o, s);
   if (g == 8) return kpl == 1 ? find_cfg<8, 1>(bv, q, out, items, o, s) : find_cfg<8, 2>(bv, q, out, items, o, s);
   if (g == 4 && kpl == 6) return find_staged(bv, q, out, items, o, s);
-  if (g == 4) return kpl == 1 ? find_cfg<4, 1>(bv, q, out, items, o, s) : find_cfg<4, 2>(bv, q, out, items, o, s);
+  if (g == 4) return kpl == 1 ? find_lines(bv, q, out, items, o, s) : find_cfg<4, 2>(bv, q, out, items, o, s);
   return cudaErrorInvalidValue;
 }
 

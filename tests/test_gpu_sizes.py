@@ -1,6 +1,7 @@
 """Builds and finds at the sizes where the kernels' splits of the work change:
 around a warp's chunk, around one share per warp, and past it."""
 
+import numpy as np
 import pytest
 import torch
 
@@ -72,3 +73,22 @@ def test_line_find(G, scheme, b, lf, nq):
         T = O.Table(G.SCHEMES[scheme], n, lf, b=b, m=st["num_buckets"])
         T.set_constants(st["hash_a"], st["hash_c"])
         assert st["find_probes"] == T.find(q, slots=t.export())[2]
+
+
+@pytest.mark.parametrize("tables,most", [(1, 5), (3, 70), (700, 9), (300, 3000)])
+def test_batch_line_find_over_uneven_segments(G, tables, most):
+    """Tables without keys or queries between others, query segments shorter than a chunk and
+    across many of them, sentinel queries: every segment answered from its own table."""
+    r = np.random.default_rng(tables)
+    nk, nq = r.integers(0, most, tables), r.integers(0, 2 * most, tables) * r.integers(0, 2, tables)
+    nq[-1] = 0 if tables > 1 else 7
+    ko, qo = (np.concatenate([[0], np.cumsum(x)]).astype(np.uint64) for x in (nk, nq))
+    keys, vals = W.make_keys(int(ko[-1]) + 1, 5), W.make_values(int(ko[-1]) + 1, 5)
+    q = torch.cat([W.make_queries(keys, int(qo[-1]), 0.8, seed=3), keys[:0]])
+    q[3::41] = -1
+    b = G.Batch(np.maximum(nk, 1), np.full(tables, 0.9), seed=2)
+    b.set_layout(ko, qo)
+    got = O._u32(b.run(keys.cuda(), vals.cuda(), q.cuda()).cpu())
+    for t in range(tables):
+        k0, k1, q0, q1 = (int(x) for x in (ko[t], ko[t + 1], qo[t], qo[t + 1]))
+        assert (got[q0:q1] == O.lookup(keys[k0:k1], vals[k0:k1], q[q0:q1])).all(), t
