@@ -21,10 +21,14 @@ struct BatchView {
   const uint64_t *key_offs;    // num_tables + 1 prefix offsets into the key/value arrays
   const uint64_t *query_offs;  // num_tables + 1 prefix offsets into the query/result arrays
   Ctrl *ctrl;                  // batch-wide probe counters
+  const uint32_t *const *src;  // finds, if set: each segment's queries and answers in arrays of its own
+  uint32_t *const *dst;        // (the line find alone reads them: 4 lanes, one query per lane)
   uint32_t t_lo, t_hi;         // tables this launch covers
   int32_t h;
   uint32_t max_chain, max_steps, rng_seed;
 };
+
+constexpr uint64_t kLineFindMost = 0xFFFF0000ull;  // queries of one batched line find (32-bit places)
 
 bool batch_shape_supported(int tile_lanes, int keys_per_lane);
 // Find shapes: the above, of which 4-lane tiles with one query per lane are the

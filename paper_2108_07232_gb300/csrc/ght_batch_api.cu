@@ -58,6 +58,8 @@ struct ght_batch {
     v.key_offs = d_key_offs;
     v.query_offs = d_query_offs;
     v.ctrl = d_ctrl;
+    v.src = nullptr;
+    v.dst = nullptr;
     v.t_lo = lo;
     v.t_hi = hi;
     v.h = h;

@@ -6,8 +6,9 @@
 //   * the find scheduler keeps up to two batched launches in flight. Whenever
 //     one completes it packs every pending find request whose table is ready
 //     (oldest first, up to a query cap) into the next launch: one upload of
-//     per-request descriptors, a gather of the requests' queries into one
-//     array, one batched find, a scatter of the answers. Requests that arrive
+//     per-request descriptors and one batched find that reads and answers each
+//     request in its own arrays (find shapes other than the line find: a gather
+//     of the queries before it, a scatter after it). Requests that arrive
 //     while launches run join the next launch (continuous batching).
 //   * the build worker admits build requests in arrival order when the table
 //     fits in the HBM budget, allocates its storage from the library pool and
@@ -158,7 +159,10 @@ int ght_pool::launch_finds(Slot &sl, std::vector<uint64_t> &batch) {
   uint64_t *d_offs = reinterpret_cast<uint64_t *>(d + R * sizeof(ght::BatchTable));
   const uint32_t *const *d_src = reinterpret_cast<const uint32_t *const *>(d_offs + R + 1);
   uint32_t *const *d_dst = reinterpret_cast<uint32_t *const *>(d_offs + R + 1 + R);
-  const uint64_t need = 2ull * total * sizeof(uint32_t) + 512;
+  // The line find reads and answers each request in its own arrays; the other
+  // find shapes take one array, gathered and scattered around them.
+  const bool direct = find_o.tile_lanes == 4 && find_o.keys_per_lane == 1 && total <= ght::kLineFindMost;
+  const uint64_t need = direct ? 0 : 2ull * total * sizeof(uint32_t) + 512;
   if (sl.staging_bytes < need) {
     if (sl.staging) cudaFreeAsync(sl.staging, find_stream);
     sl.staging = nullptr;
@@ -169,9 +173,9 @@ int ght_pool::launch_finds(Slot &sl, std::vector<uint64_t> &batch) {
     sl.staging_bytes = want;
   }
   uint32_t *q = static_cast<uint32_t *>(sl.staging);
-  uint32_t *o = q + ((total + 63) & ~63ull);
+  uint32_t *o = direct ? nullptr : q + ((total + 63) & ~63ull);
   cudaError_t e = cudaMemcpyAsync(sl.dev, sl.pinned, layout, cudaMemcpyHostToDevice, find_stream);
-  if (e == cudaSuccess) e = ght::launch_segment_gather(d_src, d_offs, R, q, total, find_stream);
+  if (e == cudaSuccess && !direct) e = ght::launch_segment_gather(d_src, d_offs, R, q, total, find_stream);
   if (e == cudaSuccess) {
     ght::BatchView bv;
     memset(&bv, 0, sizeof bv);
@@ -179,12 +183,14 @@ int ght_pool::launch_finds(Slot &sl, std::vector<uint64_t> &batch) {
     bv.key_offs = d_offs;
     bv.query_offs = d_offs;
     bv.ctrl = nullptr;
+    bv.src = direct ? d_src : nullptr;
+    bv.dst = direct ? d_dst : nullptr;
     bv.t_lo = 0;
     bv.t_hi = R;
     bv.h = 3;
     e = ght::launch_batch_find(bv, q, o, total, find_o, find_stream);
   }
-  if (e == cudaSuccess) e = ght::launch_segment_scatter(o, d_dst, d_offs, R, total, find_stream);
+  if (e == cudaSuccess && !direct) e = ght::launch_segment_scatter(o, d_dst, d_offs, R, total, find_stream);
   if (e == cudaSuccess) e = cudaEventRecord(sl.ev, find_stream);
   if (e != cudaSuccess) return cuda_fail(e, "launching pooled finds");
   sl.busy = true;
@@ -375,6 +381,8 @@ ght_pool *ght_pool_create(uint64_t hbm_budget_bytes, const ght_config *cfg) {
   }
   p->find_o.tile_lanes = p->cfg.tile_lanes;
   p->find_o.keys_per_lane = p->cfg.keys_per_lane;
+  // a config that names no other find shape than the default: the line find
+  if (p->find_o.tile_lanes == 4 && p->find_o.keys_per_lane == 2) p->find_o.keys_per_lane = 1;
   if (!ght::batch_find_shape_supported(p->find_o.tile_lanes, p->find_o.keys_per_lane)) {
     fail(GHT_ERR_INVALID_ARG, "unsupported find shape");
     delete p;

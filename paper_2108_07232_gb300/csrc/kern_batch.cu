@@ -473,7 +473,14 @@ __device__ __forceinline__ uint32_t seek_table(const uint64_t *__restrict__ offs
 // queries, half present): 13.5 ms (register find, two queries per lane; one:
 // 11.2) -> 2.5 ms; 64 tables of 2^12..2^22 keys (87 M queries) 6.5 -> 1.3 ms;
 // 512 tables of 2^10..2^14 keys (6 M queries, all in the L2) 0.30 -> 0.12 ms.
-template <bool COUNT>
+//
+// SEG: segment t's queries are read from bv.src[t] and its answers go to
+// bv.dst[t] (the requests of a pool, each with arrays of its own), instead of
+// one array each; `queries` and `out` are not used. A burst of 128 requests
+// (9.6 M queries, 32 tables of 2^16..2^22 keys), submit to last answer: 1040 us
+// with the register find between a gather and a scatter, 534 us now (most of
+// it the host's submits and waits).
+template <bool COUNT, bool SEG>
 __global__ void __launch_bounds__(kLineFindThreads, 4)
 batch_line_find_kernel(BatchView bv, const uint32_t *__restrict__ queries, uint32_t *__restrict__ out,
                        uint32_t n) {
@@ -490,12 +497,23 @@ batch_line_find_kernel(BatchView bv, const uint32_t *__restrict__ queries, uint3
   const uint32_t start = blockIdx.x * kLineFindThreads + (threadIdx.x & ~31u);
   if (start >= n) return;  // whole warp
   const uint64_t lo = __ldg(offs + bv.t_lo);
-  queries += lo;
-  out += lo;
+  queries += SEG ? 0 : lo;
+  out += SEG ? 0 : lo;
+  auto query = [&](uint32_t i, uint32_t t) {
+    // (a request may be answered in place: each query is read once, before its answer is written)
+    if constexpr (SEG) return bv.src[t][lo + i - __ldg(offs + t)];
+    else return __ldg(queries + i);
+  };
+  auto answer = [&](uint32_t i, uint32_t t, uint32_t v) {
+    if constexpr (SEG) bv.dst[t][lo + i - __ldg(offs + t)] = v;
+    else out[i] = v;
+  };
   int waiting = 0;
   unsigned long long probes = 0, answered = 0;
-  uint32_t first = table_of(offs, bv.t_lo, bv.t_hi, lo + start);  // table of the next step's first query
-  uint32_t next = __ldg(queries + min(start + lane, n - 1u));
+  // the next step's queries and their tables
+  uint32_t first = table_of(offs, bv.t_lo, bv.t_hi, lo + start);
+  uint32_t next_table = advance_table(offs, first, bv.t_hi, lo + min(start + lane, n - 1u));
+  uint32_t next = query(min(start + lane, n - 1u), next_table);
   for (uint32_t c = start;;) {
     uint32_t k, at, tb;
     int probe;
@@ -516,17 +534,19 @@ batch_line_find_kernel(BatchView bv, const uint32_t *__restrict__ queries, uint3
       k = next;
       at = c + lane;
       probe = 0;
-      tb = advance_table(offs, first, bv.t_hi, lo + min(at, n - 1u));
+      tb = next_table;
       if (c < n - min(n, step)) {
         c += step;
-        next = __ldg(queries + min(c + lane, n - 1u));
+        const uint32_t i = min(c + lane, n - 1u);
         first = seek_table(offs, first, bv.t_hi, lo + c);
+        next_table = advance_table(offs, first, bv.t_hi, lo + i);
+        next = query(i, next_table);
       } else {
         c = n;
       }
       valid = at < n && k != kEmptyKey;
       if (COUNT && at < n) answered++;
-      if (at < n && k == kEmptyKey) out[at] = kEmptyKey;  // the sentinel is never a key
+      if (at < n && k == kEmptyKey) answer(at, tb, kEmptyKey);  // the sentinel is never a key
     }
     const BatchTable &d = bv.tables[tb];
     FastMod mod;
@@ -545,7 +565,7 @@ batch_line_find_kernel(BatchView bv, const uint32_t *__restrict__ queries, uint3
         hit, empty, value);
     if (COUNT && valid) probes++;
     const bool more = valid && !hit && !empty && probe + 1 < bv.h;
-    if (valid && !more) out[at] = hit ? value : kEmptyKey;
+    if (valid && !more) answer(at, tb, hit ? value : kEmptyKey);
     const unsigned mb = __ballot_sync(kFull, more);
     if (more) {
       const int i = waiting + __popc(mb & below);
@@ -846,8 +866,10 @@ static cudaError_t find_staged(const BatchView &bv, const uint32_t *q, uint32_t 
 
 static cudaError_t find_lines(const BatchView &bv, const uint32_t *q, uint32_t *out, uint64_t items,
                               const LaunchOpts &o, cudaStream_t s) {
-  if (items > 0xFFFF0000ull) return find_cfg<4, 2>(bv, q, out, items, o, s);  // 32-bit places
-  auto kern = o.count ? batch_line_find_kernel<true> : batch_line_find_kernel<false>;
+  if (items > kLineFindMost) return find_cfg<4, 2>(bv, q, out, items, o, s);  // 32-bit places
+  auto kern = bv.src    ? (o.count ? batch_line_find_kernel<true, true> : batch_line_find_kernel<false, true>)
+              : o.count ? batch_line_find_kernel<true, false>
+                        : batch_line_find_kernel<false, false>;
   int blocks = 0;
   const cudaError_t e = grid_for(kern, items, o.blocks_per_sm, &blocks);
   if (e != cudaSuccess) return e;
@@ -869,6 +891,7 @@ cudaError_t launch_batch_find(const BatchView &bv, const uint32_t *q, uint32_t *
                               const LaunchOpts &o, cudaStream_t s) {
   if (items == 0) return cudaSuccess;
   const int g = o.tile_lanes, kpl = o.keys_per_lane;
+  if (bv.src && !(g == 4 && kpl == 1 && items <= kLineFindMost)) return cudaErrorInvalidValue;
   if (g == 16) return kpl == 1 ? find_cfg<16, 1>(bv, q, out, items, o, s) : find_cfg<16, 2>(bv, q, out, items, o, s);
   if (g == 8) return kpl == 1 ? find_cfg<8, 1>(bv, q, out, items, o, s) : find_cfg<8, 2>(bv, q, out, items, o, s);
   if (g == 4 && kpl == 6) return find_staged(bv, q, out, items, o, s);

@@ -92,3 +92,27 @@ def test_batch_line_find_over_uneven_segments(G, tables, most):
     for t in range(tables):
         k0, k1, q0, q1 = (int(x) for x in (ko[t], ko[t + 1], qo[t], qo[t + 1]))
         assert (got[q0:q1] == O.lookup(keys[k0:k1], vals[k0:k1], q[q0:q1])).all(), t
+
+
+@pytest.mark.parametrize("cfg", [{}, {"tile_lanes": 8}])
+def test_pool_requests_of_all_sizes(G, cfg):
+    """Requests from one query to several chunks against two tables, a request answered in place,
+    sentinel queries; through the direct find and through the gathered one."""
+    n = 30000
+    pool = G.Pool(1 << 28, **cfg)
+    sets = [(W.make_keys(n, s), W.make_values(n, s)) for s in (1, 2)]
+    ids = []
+    for s, (k, v) in enumerate(sets):
+        ticket, table = pool.submit_build(n, 0.95, s, k.cuda(), v.cuda())
+        assert pool.wait(ticket)["status"] == 0
+        ids.append(table)
+    qs = [W.make_queries(sets[i & 1][0], nq, 0.6, seed=i) for i, nq in enumerate([1, 31, 32, 33, 5000, 1, 100003, 64])]
+    qs[4][::13] = -1
+    ins = [q.cuda() for q in qs]
+    outs = [ins[i] if i == 6 else torch.empty_like(q) for i, q in enumerate(ins)]
+    torch.cuda.synchronize()
+    for ticket in [pool.submit_find(ids[i & 1], q, o) for i, (q, o) in enumerate(zip(ins, outs))]:
+        assert pool.wait(ticket)["status"] == 0
+    for i, (q, o) in enumerate(zip(qs, outs)):
+        assert (O._u32(o.cpu()) == O.lookup(*sets[i & 1], q)).all(), i
+    pool.close()
