@@ -104,17 +104,18 @@ typedef struct {
   /* Grouped build: the pairs are first regrouped by first-choice bucket
    * range (H_0(k) >> s), so the build's concurrent stores and atomics stay in
    * a few MB of the table at a time. 1 = on, -1 = off, 0 = default: on for
-   * BCHT and BCHT_SET tables of at least 4x the device's L2 size. Needs
+   * two-phase builds of tables of at least the device's L2 size. Needs
    * scratch (ght_build_scratch_bytes) and 16-byte aligned key and value
    * arrays, else the build runs in input order. */
   int32_t group_build;
-  /* Two-phase build of BCHT and BCHT_SET: every key that arrives at its
-   * first-choice bucket while it has room is stored at its arrival rank
-   * without reading the bucket, the rest are inserted by the cuckoo insert
-   * (the same BCHT, Sec. III-A, with those keys inserted first). 1 = on,
-   * -1 = off, 0 = default: on when the build is grouped. Needs scratch
-   * (ght_build_scratch_bytes), else the build runs the cuckoo insert for
-   * every key. */
+  /* Two-phase build of BCHT, BCHT_SET and IHT: every key that arrives at its
+   * first-choice bucket while it has room (IHT: while it holds fewer than
+   * threshold - 1 keys) is stored at its arrival rank without reading the
+   * bucket, the rest are inserted by the scheme's insert (the same table,
+   * Sec. III-A and III-C, with those keys inserted first). 1 = on, -1 = off, 0 =
+   * default: on where it pays (IHT: while few keys are expected beyond the
+   * threshold; without grouping: tables below twice the L2). Needs scratch
+   * (ght_build_scratch_bytes), else the build inserts every key. */
   int32_t ranked_build;
   /* Finds of 128-byte buckets (16 pairs: BCHT with 4-lane tiles, P2BHT, IHT
    * and the load-balanced BCHT, whose find tiles then have 4 lanes; the
@@ -250,8 +251,8 @@ int ght_find(const ght_table *t, const uint32_t *d_queries, uint32_t *d_out, uin
  * or the results are in h_out. Pinned host memory copies fastest. A build
  * from page-locked keys and values (allocated or registered with the CUDA
  * runtime) that requests neither grouping nor the two-phase build
- * (group_build and ranked_build <= 0, the host-buffer defaults) copies
- * nothing: its input-order insert reads them in place (last_h2d_ms -1); they
+ * (group_build and ranked_build <= 0) copies nothing: its placement or insert
+ * reads them in place, ungrouped (last_h2d_ms -1); they
  * must stay unchanged until the call returns. If the bounded wait for the
  * device runs out (GHT_ERR_DEVICE_TIMEOUT, see GHT_WAIT_TIMEOUT_S), copies
  * or kernels already queued may still read h_keys/h_values or write h_out

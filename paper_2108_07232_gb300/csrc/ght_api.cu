@@ -179,6 +179,13 @@ int resolve(int scheme, uint64_t capacity, double lf, const ght_config *user, Sh
   const bool grouped_shape = scheme != GHT_CUCKOO1 && scheme != GHT_BCHT_SET && b == 16;
   if (d.find_grouped > 0 && !grouped_shape)
     return fail(GHT_ERR_INVALID_ARG, "the grouped find is for tables of 16-pair buckets");
+  // the line find, unless the config names another find shape than the scheme's default
+  ght_config shape0;
+  memset(&shape0, 0, sizeof shape0);
+  default_shape(scheme, b, &shape0);
+  const bool named = d.find_async != 0 || (user_tile && user->tile_lanes != shape0.tile_lanes) ||
+                     (kpl_given && user->keys_per_lane != shape0.keys_per_lane);
+  s->find_line = (uint64_t)b * slot_bytes == 128 && !named ? 1 : 0;
   s->scheme = scheme;
   s->b = b;
   s->h = h;
@@ -193,17 +200,10 @@ int resolve(int scheme, uint64_t capacity, double lf, const ght_config *user, Sh
   s->build_blocks_per_sm = d.build_blocks_per_sm;
   s->build_keys_per_lane = d.build_keys_per_lane;
   s->group_build = d.group_build;
-  // ranked placement applies to the cuckoo tables with buckets (BCHT and the set)
-  s->ranked_build = (scheme == GHT_BCHT || scheme == GHT_BCHT_SET) ? d.ranked_build : -1;
+  // ranked placement applies to the cuckoo tables with buckets (BCHT and the set) and to IHT's primaries
+  s->ranked_build = (scheme == GHT_BCHT || scheme == GHT_BCHT_SET || scheme == GHT_IHT) ? d.ranked_build : -1;
   s->slot_bytes = (int)slot_bytes;
   s->find_async = async_find ? 1 : 0;
-  // the line find, unless the config names another find shape than the scheme's default
-  ght_config shape0;
-  memset(&shape0, 0, sizeof shape0);
-  default_shape(scheme, b, &shape0);
-  const bool named = d.find_async != 0 || (user_tile && user->tile_lanes != shape0.tile_lanes) ||
-                     (kpl_given && user->keys_per_lane != shape0.keys_per_lane);
-  s->find_line = (uint64_t)b * slot_bytes == 128 && !named ? 1 : 0;
   s->check_dups = d.check_duplicates > 0 ? 1 : 0;
   s->max_steps = d.max_steps;
   s->find_grouped = grouped_shape ? d.find_grouped : -1;
@@ -258,8 +258,9 @@ uint64_t place_scratch_bytes(uint64_t m, uint64_t n) {
   return align256(m * sizeof(uint32_t)) + 2 * align256(place_cap(n) * sizeof(uint32_t));
 }
 
-ght::PlaceBuffers place_buffers(char *scr, uint64_t m, uint64_t n) {
+ght::PlaceBuffers place_buffers(char *scr, uint64_t m, uint64_t n, uint32_t limit) {
   ght::PlaceBuffers pb;
+  pb.limit = limit;
   pb.counters = reinterpret_cast<uint32_t *>(scr);
   pb.cap = place_cap(n);
   pb.ovf_k = reinterpret_cast<uint32_t *>(scr + align256(m * sizeof(uint32_t)));
@@ -407,18 +408,31 @@ namespace {
 // Insert n pairs (shares per warp: claim_plan). The control block's work
 // cursor must be zero at launch (the fill clears it). ordered: the pairs are
 // grouped, so the warps advance through them together.
-// past_first: the keys are the overflow of a first-choice placement, whose
-// H_0 buckets are full (the placement counted that visit), so a BCHT insert
-// starts them at H_1 instead of reading H_0 again and exchanging there.
-cudaError_t launch_insert(const ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n,
-                          bool past_first = false, bool ordered = false) {
-  ght::TableView tv = t->view();
-  if (past_first && tv.h > 1 && (t->shape.scheme == GHT_BCHT || t->shape.scheme == GHT_BCHT_SET)) tv.first = 1;
-  ght::LaunchOpts o = t->build_opts();
-  o.ordered = ordered;
+cudaError_t launch_insert_opts(const ght_table *t, const ght::TableView &tv, const uint32_t *k, const uint32_t *v,
+                               uint64_t n, const ght::LaunchOpts &o) {
   if (t->shape.scheme == GHT_BCHT) return ght::launch_insert_bcht(t->shape.b, tv, k, v, n, o, t->stream);
   if (t->shape.scheme == GHT_BCHT_SET) return ght::launch_insert_set(tv, k, v ? v : k, n, o, t->stream);
   return ght::launch_insert_other(t->shape.scheme, t->shape.b, tv, k, v, n, o, t->stream);
+}
+
+cudaError_t launch_insert(const ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n,
+                          bool ordered = false) {
+  ght::LaunchOpts o = t->build_opts();
+  o.ordered = ordered;
+  return launch_insert_opts(t, t->view(), k, v, n, o);
+}
+
+// Insert a placement's overflow list of at most pb.cap pairs, whose length the
+// device reads from the control block (no host wait in between). Their
+// first-choice buckets are full (IHT: hold the threshold less one), and the
+// placement counted that visit, so they start at H_1 instead of reading H_0
+// again.
+cudaError_t launch_insert_overflow(const ght_table *t, const ght::PlaceBuffers &pb) {
+  ght::TableView tv = t->view();
+  if (tv.h > 1) tv.first = 1;
+  ght::LaunchOpts o = t->build_opts();
+  o.overflow = true;
+  return launch_insert_opts(t, tv, pb.ovf_k, pb.ovf_v, pb.cap, o);
 }
 
 // L2 size of the current device (bytes; cached per device).
@@ -442,26 +456,66 @@ uint64_t device_l2_bytes() {
   return cache[dev];
 }
 
-// Whether a build of n keys groups its input first by first-choice bucket
-// range (config group_build: 1 on, -1 off, 0 by table size); it also needs
-// scratch (caller-set, or the library pool when the library owns the table
-// storage), else the build runs in input order.
-bool wants_grouping(const ght_table *t, uint64_t n) {
-  if (t->shape.scheme == GHT_CUCKOO1 || n == 0 || n > 0xFFFFFFFFull) return false;
-  if (t->shape.group_build != 0) return t->shape.group_build > 0;
-  // default: cuckoo tables with buckets far larger than the L2, where the
-  // grouped two-phase build measured 1.3-1.4x faster than the insert of
-  // every key in input order (2^28 keys); at 2^20-2^24 keys it was slower
-  if (t->shape.scheme != GHT_BCHT && t->shape.scheme != GHT_BCHT_SET) return false;
-  return t->storage_bytes >= 4ull * device_l2_bytes();
+// Pairs a bucket takes in the ranked placement: all its slots, or in IHT the
+// keys that find fewer than the threshold with them (Sec. III-C); 0 for the
+// schemes that place by their candidates' loads.
+uint32_t place_limit(const Shape &s) {
+  if (s.scheme == GHT_BCHT || s.scheme == GHT_BCHT_SET) return (uint32_t)s.b;
+  if (s.scheme == GHT_IHT) return (uint32_t)std::min(s.b, s.t - 1);
+  return 0;
+}
+
+// Share of n keys beyond their first-choice bucket's `limit` under a random
+// hash (Poisson arrivals).
+double expected_overflow(uint64_t n, uint64_t m, uint32_t limit) {
+  const double mean = (double)n / (double)m;
+  double p = std::exp(-mean), below = 0.0, cdf = 0.0;  // sum of k p_k and of p_k, k <= limit
+  for (uint32_t k = 0; k <= limit; ++k) {
+    below += k * p;
+    cdf += p;
+    p *= mean / (k + 1);
+  }
+  return mean > 0.0 ? (mean - below - limit * (1.0 - cdf)) / mean : 0.0;
 }
 
 // Whether a build of n keys runs in two phases (ranked first-choice
-// placement, then the cuckoo insert of the overflow).
+// placement, then the insert of the overflow; config ranked_build: 1 on, -1
+// off, 0 always where it applies). It costs no bucket read for the keys that
+// find room at once, so it won at every size measured (whole builds, us,
+// input order -> two phases, BCHT at LF 0.9): 2^14 keys 94 -> 81, 2^17 97 ->
+// 85, 2^20 126 -> 105, 2^22 259 -> 154, 2^24 657 -> 411; IHT at LF 0.8: 2^17
+// 120 -> 94, 2^20 181 -> 125, 2^24 1157 -> 550; set at LF 0.95: 2^17 169 ->
+// 100, 50 M keys 2920 -> 1115. IHT's overflow, the keys beyond its threshold,
+// has to fit the overflow list: above 0.22 of the keys it builds in input
+// order (low thresholds, or load factors where it rarely succeeds).
+// Ungrouped, the placement's stores and counters go to DRAM one sector each on
+// tables beyond the L2: above twice its size (where 2^28 keys took 17.6 ms
+// against 16.8 in input order) only on request.
+bool places_ungrouped(const ght_table *t) {
+  return t->shape.ranked_build > 0 || t->storage_bytes < 2ull * device_l2_bytes();
+}
+
 bool wants_ranked(const ght_table *t, uint64_t n) {
-  if (t->shape.ranked_build < 0 || n == 0 || n > 0xFFFFFFFFull) return false;
-  // default: with the grouping, whose order keeps the placement's stores in L2
-  return t->shape.ranked_build > 0 || wants_grouping(t, n);
+
+  const uint32_t limit = place_limit(t->shape);
+  if (!limit || t->shape.ranked_build < 0 || n == 0 || n > 0xFFFFFFFFull) return false;
+  if (t->shape.group_build < 0 && !places_ungrouped(t)) return false;
+  return t->shape.scheme != GHT_IHT || expected_overflow(n, t->shape.m, limit) <= 0.22;
+}
+
+// Whether a build of n keys groups its input first by first-choice bucket
+// range (config group_build: 1 on, -1 off, 0 by table size). Like the
+// placement it needs scratch (caller-set, or the library pool when the library
+// owns the table storage), else the build runs in input order. Default: the
+// two-phase builds of tables from the L2's size up. Inside the L2 the
+// placement's scattered stores and counters are cheaper than the two grouping
+// passes (BCHT, 112 MB 360 us ungrouped, 381 grouped; 2^22 keys 154 / 191; set
+// of 2^24 keys, 70 MB, 372 / 437); beyond it they go to DRAM (BCHT 2^24 keys,
+// 149 MB, 534 / 411).
+bool wants_grouping(const ght_table *t, uint64_t n) {
+  if (t->shape.scheme == GHT_CUCKOO1 || n == 0 || n > 0xFFFFFFFFull) return false;
+  if (t->shape.group_build != 0) return t->shape.group_build > 0;
+  return wants_ranked(t, n) && t->storage_bytes >= device_l2_bytes();
 }
 
 // Second-level split of a two-phase grouped build (the block placement):
@@ -488,31 +542,44 @@ bool sub_shape(const Shape &s, uint64_t n, int shift, uint32_t region1, SubShape
   return true;
 }
 
-// Entries of the regrouped arrays of a build of n pairs (the groups' regions
-// when the build places by rank, else n).
-uint64_t grouped_len(const ght_table *t, uint64_t n) {
+// Grouping of a build of n keys: groups of 2^shift first-choice buckets, each
+// in a region of `region` pairs when the build places by rank (0: exact
+// offsets, `len` = n entries); split: the groups are split into sub-groups,
+// which are placed by one block each in shared memory.
+struct GroupPlan {
   int shift = 0;
-  uint32_t groups = 1;
-  group_shape(t->shape.m, &shift, &groups);
-  const uint32_t region = wants_ranked(t, n) ? group_region(n, groups) : 0u;
-  return region ? (uint64_t)groups * region : n;
+  uint32_t groups = 1, region = 0;
+  uint64_t len = 0;
+  bool split = false;
+  SubShape sub;
+};
+
+GroupPlan group_plan(const ght_table *t, uint64_t n) {
+  GroupPlan g;
+  const uint64_t m = t->shape.m;
+  group_shape(m, &g.shift, &g.groups);
+  g.len = n;
+  if (!wants_ranked(t, n)) return g;
+  g.region = group_region(n, g.groups);
+  g.split = g.region && sub_shape(t->shape, n, g.shift, g.region, &g.sub);
+  if (g.region) g.len = (uint64_t)g.groups * g.region;
+  return g;
 }
 
 // Scratch of the second-level split: the split pairs and one cursor per
 // sub-group (0 where the build does not use it).
-uint64_t sub_scratch_bytes(const ght_table *t, uint64_t n) {
-  if (!wants_grouping(t, n) || !wants_ranked(t, n)) return 0;
-  int shift = 0;
-  uint32_t groups = 1;
-  group_shape(t->shape.m, &shift, &groups);
-  SubShape sh;
-  if (!sub_shape(t->shape, n, shift, group_region(n, groups), &sh)) return 0;
-  return 2 * align256((uint64_t)sh.bins * sh.region2 * sizeof(uint32_t)) + align256(sh.bins * sizeof(uint32_t));
+uint64_t sub_scratch_bytes(const GroupPlan &g) {
+  if (!g.split) return 0;
+  return 2 * align256((uint64_t)g.sub.bins * g.sub.region2 * sizeof(uint32_t)) + align256(g.sub.bins * sizeof(uint32_t));
 }
 
 uint64_t build_scratch_need(const ght_table *t, uint64_t n) {
-  return (wants_grouping(t, n) ? group_scratch_bytes(grouped_len(t, n)) : 0) +
-         (wants_ranked(t, n) ? place_scratch_bytes(t->shape.m, n) : 0) + sub_scratch_bytes(t, n);
+  uint64_t need = wants_ranked(t, n) ? place_scratch_bytes(t->shape.m, n) : 0;
+  if (wants_grouping(t, n)) {
+    const GroupPlan g = group_plan(t, n);
+    need += group_scratch_bytes(g.len) + sub_scratch_bytes(g);
+  }
+  return need;
 }
 
 // Scratch of a two- or grouped-phase build: the caller's, else (for tables on
@@ -530,7 +597,7 @@ cudaError_t launch_place(const ght_table *t, const uint32_t *k, const uint32_t *
                          const ght::PlaceBuffers &pb) {
   const bool count = t->shape.count_probes != 0;
   if (t->shape.scheme == GHT_BCHT_SET) return ght::launch_place_set(t->view(), k, n, pb, count, t->stream);
-  return ght::launch_place_bcht(t->shape.b, t->view(), k, v, n, pb, count, t->stream);
+  return ght::launch_place_pairs(t->shape.b, t->view(), k, v, n, pb, count, t->stream);
 }
 
 // Grouped find (kern_gfind.cu): shape of the two grouping levels of each
@@ -754,18 +821,42 @@ bool device_view(const void *h, const void **d) {
   return true;
 }
 
-// One build from device-resident keys: fill, (group,) insert, status; retry
-// with the next attempt's constants on failure.
+// Take over an attempt's control block (just read): GHT_OK if it built the
+// table, GHT_ERR_BUILD_FAILED if another attempt may.
+int finish_attempt(ght_table *t, uint64_t n, uint32_t attempt, bool grouped, bool split, bool ranked) {
+  const uint32_t st = t->h_ctrl->status;
+  t->last_grouped = grouped;
+  t->last_split = split;
+  t->last_ranked = ranked;
+  t->attempts = attempt + 1;
+  t->insert_probes = t->h_ctrl->insert_probes;
+  t->insert_retries = t->h_ctrl->insert_retries;
+  t->insert_evictions = t->h_ctrl->insert_evictions;
+  t->longest_chain = t->h_ctrl->longest_chain;
+  if (st == 0u) {
+    t->built = true;
+    t->n_stored = n;
+    return GHT_OK;
+  }
+  if (st & ght::kStatusSentinel) return fail(GHT_ERR_SENTINEL_KEY, "an input key is the sentinel 0xFFFFFFFF");
+  if (st & ght::kStatusTimeout) return fail(GHT_ERR_DEVICE_TIMEOUT, "a key exceeded the per-key step bound");
+  if (st & ght::kStatusCorrupt) return fail(GHT_ERR_CUDA, "table corrupt: an evicted key did not hash to its bucket");
+  return fail(GHT_ERR_BUILD_FAILED, "build failed in %u attempts (chain bound or full buckets)", t->shape.max_attempts);
+}
+
+// One build from keys the device can read (host_input: page-locked host
+// memory): fill, (group, place,) insert, status; retry with the next attempt's
+// constants on failure.
 int build_device(ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n, uint32_t first_attempt,
-                 bool input_order = false) {
+                 bool host_input = false) {
   t->built = false;
   t->n_stored = 0;
-  bool ranked = !input_order && wants_ranked(t, n);
-  bool grouped = !input_order && wants_grouping(t, n);
-  if (grouped && ((reinterpret_cast<uintptr_t>(k) | reinterpret_cast<uintptr_t>(v ? v : k)) & 15u)) {
-    // the grouping copies 16-byte pieces of the input: unaligned arrays build ungrouped
+  bool ranked = wants_ranked(t, n);
+  bool grouped = wants_grouping(t, n);
+  if (grouped && (host_input || ((reinterpret_cast<uintptr_t>(k) | reinterpret_cast<uintptr_t>(v ? v : k)) & 15u))) {
+    // the grouping makes bulk copies of 16-byte pieces of device memory: other input builds ungrouped
     grouped = false;
-    ranked = t->shape.ranked_build > 0;
+    ranked = ranked && places_ungrouped(t);
   }
   void *pool_buf = nullptr;
   char *scr = nullptr;
@@ -773,26 +864,20 @@ int build_device(ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n,
     scr = build_scratch(t, build_scratch_need(t, n), &pool_buf);
     if (!scr) ranked = grouped = false;  // no scratch: the cuckoo insert of every key in input order
   }
-  int shift = 0;
-  uint32_t groups = 1;
-  group_shape(t->shape.m, &shift, &groups);
-  // grouped pairs in per-group regions when placed by rank (no count pass)
-  const uint64_t glen = grouped ? grouped_len(t, n) : n;
-  uint32_t region = grouped && ranked && glen != n ? group_region(n, groups) : 0u;
+  GroupPlan g;
+  if (grouped) g = group_plan(t, n);
+  // scratch layout: [grouping: counts, cursors, keys, values][ranked placement][sub-group keys, values, cursors]
   uint32_t *counts = reinterpret_cast<uint32_t *>(scr);
   uint32_t *cursors = counts + ght::kMaxGroups;
   uint32_t *gk = reinterpret_cast<uint32_t *>(scr + 2ull * ght::kMaxGroups * sizeof(uint32_t));
-  uint32_t *gv = gk + align256(glen * sizeof(uint32_t)) / sizeof(uint32_t);
-  // scratch layout: [grouping: counts, cursors, keys, values][ranked placement]
+  uint32_t *gv = gk + align256(g.len * sizeof(uint32_t)) / sizeof(uint32_t);
+  char *place_scr = grouped ? scr + group_scratch_bytes(g.len) : scr;
   const ght::PlaceBuffers pb =
-      ranked ? place_buffers(scr + (grouped ? group_scratch_bytes(glen) : 0), t->shape.m, n) : ght::PlaceBuffers();
-  // second-level split and block placement: [sub-group keys, values, cursors] after the placement scratch
-  SubShape sub;
-  bool two_level = region && sub_shape(t->shape, n, shift, region, &sub) && sub_scratch_bytes(t, n) > 0;
+      ranked ? place_buffers(place_scr, t->shape.m, n, place_limit(t->shape)) : ght::PlaceBuffers();
   uint32_t *sk = nullptr, *sv = nullptr, *scur = nullptr;
-  if (two_level) {
-    char *p = scr + group_scratch_bytes(glen) + place_scratch_bytes(t->shape.m, n);
-    const uint64_t arr = align256((uint64_t)sub.bins * sub.region2 * sizeof(uint32_t));
+  if (g.split) {
+    char *p = place_scr + place_scratch_bytes(t->shape.m, n);
+    const uint64_t arr = align256((uint64_t)g.sub.bins * g.sub.region2 * sizeof(uint32_t));
     sk = reinterpret_cast<uint32_t *>(p);
     sv = reinterpret_cast<uint32_t *>(p + arr);
     scur = reinterpret_cast<uint32_t *>(p + 2 * arr);
@@ -804,25 +889,25 @@ int build_device(ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n,
     const ght::TableView tv = t->view();
     cudaEventRecord(t->tev[0], t->stream);
     // the block placement writes every table line: only the control block is reset
-    cudaError_t e = two_level ? cudaMemsetAsync(t->ctrl, 0, kCtrlBytes, t->stream) : ght::launch_fill(tv, t->words(), t->stream);
+    cudaError_t e = g.split ? cudaMemsetAsync(t->ctrl, 0, kCtrlBytes, t->stream)
+                            : ght::launch_fill(tv, t->words(), t->stream, ranked ? pb.counters : nullptr, t->shape.m);
     if (e != cudaSuccess) { rc = cuda_fail(e, "launching fill"); break; }
     cudaEventRecord(t->tev[1], t->stream);
-    const uint32_t *ik = k, *iv = v;  // what the cuckoo insert takes
-    uint64_t in = n;
-    bool this_ranked = false;
+    const uint32_t *ik = k, *iv = v;  // what an insert of every key takes
+    bool this_ranked = ranked;
     t->place_overflow = 0;
     if (grouped) {
-      e = ght::launch_group(tv, k, v ? v : k, n, shift, groups, counts, cursors, gk, gv, t->stream, region);
-      if (e == cudaSuccess && two_level) {
-        cudaEventRecord(t->tev[9], t->stream);
+      e = ght::launch_group(tv, k, v ? v : k, n, g.shift, g.groups, counts, cursors, gk, gv, t->stream, g.region);
+      if (g.split) cudaEventRecord(t->tev[9], t->stream);
+      if (e == cudaSuccess && g.split) {
         ght::SubSplit ss;
         ss.ends1 = cursors;
-        ss.region1 = region;
-        ss.region1_M = ght::make_fastmod(region).M;
-        ss.fine_shift = sub.fine_shift;
-        ss.subs_log2 = sub.subs_log2;
-        ss.groups = groups;
-        e = ght::launch_subgroup(tv, gk, gv, (uint64_t)groups * region, ss, sub.bins, scur, sub.region2, sk, sv,
+        ss.region1 = g.region;
+        ss.region1_M = ght::make_fastmod(g.region).M;
+        ss.fine_shift = g.sub.fine_shift;
+        ss.subs_log2 = g.sub.subs_log2;
+        ss.groups = g.groups;
+        e = ght::launch_subgroup(tv, gk, gv, (uint64_t)g.groups * g.region, ss, g.sub.bins, scur, g.sub.region2, sk, sv,
                                  t->stream);
       }
       if (e != cudaSuccess) { rc = cuda_fail(e, "launching grouping"); break; }
@@ -832,81 +917,61 @@ int build_device(ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n,
     }
     if (ranked) {
       // phase 1: ranked first-choice placement (of the grouped pairs, when
-      // grouped: the stores then stay in a few MB of the table, whose lines
-      // fill up in L2); its overflow goes to phase 2
-      ght::PlaceBuffers pa = pb;
-      if (region) {  // the pairs of group g are [g * region, cursors[g])
-        pa.ends = cursors;
-        pa.region = region;
-        pa.region_M = ght::make_fastmod(region).M;
-      }
-      if (two_level) {
-        e = ght::launch_block_place(t->shape.b, t->shape.scheme == GHT_BCHT_SET, tv, sk, sv, scur, sub.region2,
-                                    sub.bins, sub.fine_shift, pb, t->shape.count_probes != 0, t->stream);
-      } else if ((e = cudaMemsetAsync(pb.counters, 0, t->shape.m * sizeof(uint32_t), t->stream)) == cudaSuccess) {
-        e = launch_place(t, ik, iv, region ? (uint64_t)groups * region : n, pa);
+      // grouped: by blocks in shared memory, or with the stores in a few MB of
+      // the table, whose lines fill up in L2); phase 2: its overflow
+      const bool set = t->shape.scheme == GHT_BCHT_SET, count = t->shape.count_probes != 0;
+      if (g.split) {
+        e = ght::launch_block_place(t->shape.b, set, tv, sk, sv, scur, g.sub.region2, g.sub.bins, g.sub.fine_shift, pb,
+                                    count, t->stream);
+      } else {
+        ght::PlaceBuffers pa = pb;
+        if (g.region) {  // the pairs of group g are [g * region, cursors[g])
+          pa.ends = cursors;
+          pa.region = g.region;
+          pa.region_M = ght::make_fastmod(g.region).M;
+        }
+        e = launch_place(t, ik, iv, g.region ? (uint64_t)g.groups * g.region : n, pa);
       }
       if (e != cudaSuccess) {
         rc = cuda_fail(e, "launching the ranked placement");
         break;
       }
       cudaEventRecord(t->tev[2], t->stream);
-      if ((rc = read_ctrl(t)) != GHT_OK) break;
-      if (region && ((t->h_ctrl->status & ght::kStatusGroupRegion) || t->h_ctrl->reserved[0] > pb.cap)) {
+      e = launch_insert_overflow(t, pb);
+    } else {
+      cudaEventRecord(t->tev[2], t->stream);
+      e = n > 0 ? launch_insert(t, ik, iv, n, grouped) : cudaSuccess;
+    }
+    if (e != cudaSuccess) { rc = cuda_fail(e, "launching insert"); break; }
+    cudaEventRecord(t->tev[3], t->stream);
+    t->timed_build = true;
+    if ((rc = read_ctrl(t)) != GHT_OK) break;
+    if (ranked) {
+      const uint64_t ovf = t->h_ctrl->reserved[0];
+      if (g.region && ((t->h_ctrl->status & ght::kStatusGroupRegion) || ovf > pb.cap)) {
         // a group outgrew its region, or the overflow outgrew its list: this
         // attempt again with exact group offsets and the filled table of the
         // global-counter placement (its fallback reads dense arrays)
-        region = 0;
-        two_level = false;
+        g.region = 0;
+        g.split = false;
         --attempt;
         continue;
       }
-      if (t->h_ctrl->status & ght::kStatusSentinel) { rc = fail(GHT_ERR_SENTINEL_KEY, "an input key is the sentinel 0xFFFFFFFF"); break; }
-      const uint64_t ovf = t->h_ctrl->reserved[0];
       t->place_overflow = ovf;
-      if (ovf <= pb.cap) {
-        this_ranked = true;
-        ik = pb.ovf_k;
-        iv = pb.ovf_v;
-        in = ovf;
-      } else {
+      if (ovf > pb.cap && !(t->h_ctrl->status & ght::kStatusSentinel)) {
         // too many keys share first-choice buckets for the overflow list:
         // start over and insert every key (grouped, if it was) with the cuckoo insert
+        this_ranked = false;
         cudaEventRecord(t->tev[0], t->stream);
         if ((e = ght::launch_fill(tv, t->words(), t->stream)) != cudaSuccess) { rc = cuda_fail(e, "launching fill"); break; }
         cudaEventRecord(t->tev[1], t->stream);
         cudaEventRecord(t->tev[2], t->stream);
+        if ((e = launch_insert(t, ik, iv, n, grouped)) != cudaSuccess) { rc = cuda_fail(e, "launching insert"); break; }
+        cudaEventRecord(t->tev[3], t->stream);
+        if ((rc = read_ctrl(t)) != GHT_OK) break;
       }
-    } else {
-      cudaEventRecord(t->tev[2], t->stream);
     }
-    if (in > 0) {
-      e = launch_insert(t, ik, iv, in, this_ranked, grouped && !this_ranked);
-      if (e != cudaSuccess) { rc = cuda_fail(e, "launching insert"); break; }
-    }
-    cudaEventRecord(t->tev[3], t->stream);
-    t->timed_build = true;
-    t->last_grouped = grouped;
-    t->last_split = this_ranked && two_level;
-    t->last_ranked = this_ranked;
-    rc = read_ctrl(t);
-    if (rc) break;
-    const uint32_t st = t->h_ctrl->status;
-    t->attempts = attempt + 1;
-    t->insert_probes = t->h_ctrl->insert_probes;
-    t->insert_retries = t->h_ctrl->insert_retries;
-    t->insert_evictions = t->h_ctrl->insert_evictions;
-    t->longest_chain = t->h_ctrl->longest_chain;
-    if (st == 0u) {
-      t->built = true;
-      t->n_stored = n;
-      rc = GHT_OK;
-      break;
-    }
-    if (st & ght::kStatusSentinel) { rc = fail(GHT_ERR_SENTINEL_KEY, "an input key is the sentinel 0xFFFFFFFF"); break; }
-    if (st & ght::kStatusTimeout) { rc = fail(GHT_ERR_DEVICE_TIMEOUT, "a key exceeded the per-key step bound"); break; }
-    if (st & ght::kStatusCorrupt) { rc = fail(GHT_ERR_CUDA, "table corrupt: an evicted key did not hash to its bucket"); break; }
-    rc = fail(GHT_ERR_BUILD_FAILED, "build failed in %u attempts (chain bound or full buckets)", t->shape.max_attempts);
+    if ((rc = finish_attempt(t, n, attempt, grouped, this_ranked && g.split, this_ranked)) != GHT_ERR_BUILD_FAILED) break;
   }
   if (pool_buf) cudaFreeAsync(pool_buf, t->stream);
   return rc;
@@ -1087,11 +1152,11 @@ int ght_build_host(ght_table *t, const uint32_t *h_keys, const uint32_t *h_value
     return fail(GHT_ERR_INVALID_ARG, "keys or values is NULL");
   if (n == 0) return build_device(t, nullptr, nullptr, 0, 0);
   if (!h_values) h_values = h_keys;  // a set ignores values
-  // Pinned host arrays the device can address: the input-order insert reads
-  // them in place, in one launch (the host link's rate is the same for the
-  // kernel's reads as for copies, and the copies' chunk pipeline -- its first
-  // chunk's wait and one insert launch tail per chunk -- goes away). A
-  // requested grouped or two-phase build still stages the pairs.
+  // Pinned host arrays the device can address: the ranked placement or the
+  // input-order insert reads them in place, in one launch (the host link's rate
+  // is the same for the kernel's reads as for copies, and the copies' chunk
+  // pipeline -- its first chunk's wait and one insert launch tail per chunk --
+  // goes away). A requested grouped or two-phase build still stages the pairs.
   const void *dk_in = nullptr, *dv_in = nullptr;
   if (t->shape.group_build <= 0 && t->shape.ranked_build <= 0 && device_view(h_keys, &dk_in) &&
       device_view(h_values, &dv_in)) {
@@ -1131,7 +1196,7 @@ int ght_build_host(ght_table *t, const uint32_t *h_keys, const uint32_t *h_value
     void *place_pool = nullptr;
     char *scr = ranked_wanted ? build_scratch(t, place_scratch_bytes(t->shape.m, n), &place_pool) : nullptr;
     const bool ranked = scr != nullptr;
-    const ght::PlaceBuffers pb = ranked ? place_buffers(scr, t->shape.m, n) : ght::PlaceBuffers();
+    const ght::PlaceBuffers pb = ranked ? place_buffers(scr, t->shape.m, n, place_limit(t->shape)) : ght::PlaceBuffers();
     cudaStream_t copy = nullptr;
     cudaEvent_t landed[2] = {nullptr, nullptr};
     if ((e = cudaStreamCreateWithFlags(&copy, cudaStreamNonBlocking)) != cudaSuccess ||
@@ -1149,11 +1214,8 @@ int ght_build_host(ght_table *t, const uint32_t *h_keys, const uint32_t *h_value
       t->derive(0);
       const ght::TableView tv = t->view();
       cudaEventRecord(t->tev[0], t->stream);
-      if ((e = ght::launch_fill(tv, t->words(), t->stream)) != cudaSuccess)
+      if ((e = ght::launch_fill(tv, t->words(), t->stream, ranked ? pb.counters : nullptr, t->shape.m)) != cudaSuccess)
         rc = cuda_fail(e, "launching fill");
-      if (rc == GHT_OK && ranked &&
-          (e = cudaMemsetAsync(pb.counters, 0, t->shape.m * sizeof(uint32_t), t->stream)) != cudaSuccess)
-        rc = cuda_fail(e, "clearing the arrival counters");
       cudaEventRecord(t->tev[1], t->stream);
       if (!ranked) cudaEventRecord(t->tev[2], t->stream);
       cudaEventRecord(t->tev[7], copy);
@@ -1187,7 +1249,7 @@ int ght_build_host(ght_table *t, const uint32_t *h_keys, const uint32_t *h_value
           const uint64_t ovf = t->h_ctrl->reserved[0];
           t->place_overflow = ovf;
           if (ovf > pb.cap) retry_staged = true;  // overflow list too small: build_device falls back
-          else if (ovf > 0 && (e = launch_insert(t, pb.ovf_k, pb.ovf_v, ovf, true)) != cudaSuccess)
+          else if (ovf > 0 && (e = launch_insert_overflow(t, pb)) != cudaSuccess)
             rc = cuda_fail(e, "launching insert");
         }
       }

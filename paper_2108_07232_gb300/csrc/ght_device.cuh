@@ -94,6 +94,37 @@ struct ClaimPlan {
   uint32_t first, claim;
 };
 
+// How the warps of an insert share its input of n pairs, in 32-pair chunks:
+// `first` chunks each, and what is left in runs of `claim` chunks claimed from
+// a global cursor (zero at launch), so that the warps finish together however
+// long the eviction chains of their keys are.
+//  * Up to 32 chunks a warp: an even share and no claims. Claims of 1024
+//    pairs, whatever n, gave 2^20 keys to 1024 warps of 3648 and 20,000 keys to
+//    20: BCHT at LF 0.9 took 137 us for 2^20 keys (now 85) and at LF 0.95 139
+//    us for 20,000 (now 67); at 2^21 keys the even share takes 116 us against
+//    159 with claims.
+//  * Beyond: three quarters shared evenly, the rest in about eight runs a warp
+//    (each claim is one atomic on one address, ~3 ns apart): 2^24 keys 747 ->
+//    712 us for BCHT at LF 0.95, 1191 -> 1091 for P2BHT and 1073 -> 922 for IHT
+//    at LF 0.8. (Half shared evenly and four runs: 817, 1165, 1040.)
+//  * ordered: the input order is a locality order (a grouped input, or a batch
+//    whose tables follow one another), so beyond 8 chunks a warp (0.9 M pairs,
+//    whose buckets the L2 holds in any order) all warps advance together:
+//    claims only.
+__host__ __device__ inline ClaimPlan claim_plan(uint64_t n, uint64_t warps, bool ordered) {
+  const uint64_t chunks = (n + 31) / 32;
+  ClaimPlan p;
+  if (chunks <= (ordered ? 8 : 32) * warps) {
+    p.first = (uint32_t)((chunks + warps - 1) / warps);
+    p.claim = 1;
+  } else {
+    p.first = ordered ? 0u : (uint32_t)(chunks / warps * 3 / 4);
+    const uint64_t share = (chunks - p.first * warps) / (warps * 8);
+    p.claim = (uint32_t)(share < 1 ? 1 : (share > 32 ? 32 : share));
+  }
+  return p;
+}
+
 // Everything a kernel needs to address a table; passed by value.
 struct TableView {
   uint64_t *slots;     // m * b pairs, bucket-major
@@ -105,7 +136,7 @@ struct TableView {
   uint32_t max_chain;  // cuckoo exchanges per insert
   uint32_t rng_seed;   // eviction xorshift seed
   uint32_t max_steps;  // per-key bound on build rounds (timeout)
-  int32_t first;       // BCHT: hash index a new key starts at (1 for keys whose H_0 is known to be full)
+  int32_t first;       // BCHT and IHT: hash index a new key starts at (1 for keys whose H_0 is known to be full)
 };
 
 __device__ __forceinline__ uint32_t pair_key(uint64_t p) { return (uint32_t)p; }

@@ -19,6 +19,7 @@ struct LaunchOpts {
   int blocks_per_sm = 0;
   bool count = false;    // probe counters
   bool ordered = false;  // insert: the warps advance through the input together
+  bool overflow = false;  // insert: the pairs are a placement's overflow, counted in the control block
   bool async_find = false;  // find: bucket parts staged in shared memory (BCHT, b = 16, 4-lane tiles)
 };
 
@@ -80,7 +81,8 @@ inline cudaError_t grid_for_smem(K kernel, int threads, size_t smem, uint64_t n,
   PerDevice &d = devices[dev];
   if (d.sms == 0 && (e = cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   const void *key = (const void *)kernel;
-  if (smem > 48 * 1024 && d.limit[key] < smem) {
+  // (the 48 KB a kernel may have without asking include its static shared memory)
+  if (d.limit[key] < smem) {
     if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
       return e;
     d.limit[key] = smem;
@@ -107,38 +109,6 @@ inline uint64_t per_warp_of(uint64_t n, int blocks) {
   return (n + warps - 1) / warps;
 }
 
-// How the warps of an insert share its input of n pairs, in 32-pair chunks:
-// `first` chunks each, and what is left in runs of `claim` chunks claimed from
-// a global cursor (zero at launch), so that the warps finish together however
-// long the eviction chains of their keys are.
-//  * Up to 32 chunks a warp: an even share and no claims. Claims of 1024
-//    pairs, whatever n, gave 2^20 keys to 1024 warps of 3648 and 20,000 keys to
-//    20: BCHT at LF 0.9 took 137 us for 2^20 keys (now 85) and at LF 0.95 139
-//    us for 20,000 (now 67); at 2^21 keys the even share takes 116 us against
-//    159 with claims.
-//  * Beyond: three quarters shared evenly, the rest in about eight runs a warp
-//    (each claim is one atomic on one address, ~3 ns apart): 2^24 keys 747 ->
-//    712 us for BCHT at LF 0.95, 1191 -> 1091 for P2BHT and 1073 -> 922 for IHT
-//    at LF 0.8. (Half shared evenly and four runs: 817, 1165, 1040.)
-//  * ordered: the input order is a locality order (a grouped input, or a batch
-//    whose tables follow one another), so beyond 8 chunks a warp (0.9 M pairs,
-//    whose buckets the L2 holds in any order) all warps advance together:
-//    claims only.
-inline ClaimPlan claim_plan(uint64_t n, int blocks, bool ordered) {
-  const uint64_t warps = (uint64_t)blocks * (kThreads / 32);
-  const uint64_t chunks = (n + 31) / 32;
-  ClaimPlan p;
-  if (chunks <= (ordered ? 8 : 32) * warps) {
-    p.first = (uint32_t)((chunks + warps - 1) / warps);
-    p.claim = 1;
-  } else {
-    p.first = ordered ? 0u : (uint32_t)(chunks / warps * 3 / 4);
-    const uint64_t share = (chunks - p.first * warps) / (warps * 8);
-    p.claim = (uint32_t)(share < 1 ? 1 : (share > 32 ? 32 : share));
-  }
-  return p;
-}
-
 // Scratch of a two-phase (ranked placement) build: one arrival counter per
 // bucket and an overflow list of `cap` pairs (see rank_place_kernel).
 struct PlaceBuffers {
@@ -146,6 +116,7 @@ struct PlaceBuffers {
   uint32_t *ovf_k = nullptr;
   uint32_t *ovf_v = nullptr;
   uint64_t cap = 0;
+  uint32_t limit = 0;  // pairs a bucket takes in the placement (its slots, IHT: fewer than its threshold)
   // Grouped input in regions of `region` items per group (0: a dense input):
   // group g's pairs are [g * region, ends[g]); the rest of its region is unused.
   const uint32_t *ends = nullptr;
@@ -158,7 +129,7 @@ struct PlaceBuffers {
 constexpr uint32_t kStatusGroupRegion = 32u;
 
 // kern_bcht.cu
-cudaError_t launch_place_bcht(int B, const TableView &tv, const uint32_t *k, const uint32_t *v, uint64_t n,
+cudaError_t launch_place_pairs(int B, const TableView &tv, const uint32_t *k, const uint32_t *v, uint64_t n,
                               const PlaceBuffers &pb, bool count, cudaStream_t s);
 cudaError_t launch_insert_bcht(int B, const TableView &tv, const uint32_t *k, const uint32_t *v,
                                uint64_t n, const LaunchOpts &o, cudaStream_t s);
@@ -190,7 +161,9 @@ cudaError_t launch_insert_other(int scheme, int B, const TableView &tv, const ui
 cudaError_t launch_find_other(int scheme, int B, const TableView &tv, const uint32_t *q,
                               uint32_t *out, uint64_t n, const LaunchOpts &o, cudaStream_t s);
 bool other_shape_supported(int scheme, int B, int G);
-cudaError_t launch_fill(const TableView &tv, uint64_t num_slots, cudaStream_t s);
+// fills the table, resets its control block and, where given, zeroes the m arrival counters
+cudaError_t launch_fill(const TableView &tv, uint64_t num_slots, cudaStream_t s, uint32_t *counters = nullptr,
+                        uint64_t m = 0);
 cudaError_t launch_dup_check(const TableView &tv, int B, bool key_slots, const uint32_t *keys, uint64_t n,
                              cudaStream_t s);
 cudaError_t launch_hash(const TableView &tv, const uint32_t *k, uint32_t *out, uint64_t n,

@@ -129,10 +129,18 @@ constexpr int insert_min_blocks() {
 template <int SCHEME, int B, int G, int KPL, bool COUNT, typename S = PairSlot>
 __global__ void __launch_bounds__(256, insert_min_blocks<B, G, KPL, COUNT>())
 bucketed_insert_kernel(TableView tv, const uint32_t *__restrict__ keys,
-                       const uint32_t *__restrict__ values, uint64_t n, ClaimPlan plan) {
+                       const uint32_t *__restrict__ values, uint64_t n, bool ordered, bool overflow) {
   using T = typename S::T;
   constexpr int PPL = B / G;
   T *slots = reinterpret_cast<T *>(tv.slots);
+  if (overflow) {
+    // the list of the placement before: its length is on the device; nothing
+    // to insert where the placement gave up or the list is short of it
+    const unsigned long long listed = tv.ctrl->reserved[0];
+    if (load_status(tv.ctrl) != 0u || listed > n) return;
+    n = listed;
+  }
+  const ClaimPlan plan = claim_plan(n, (uint64_t)gridDim.x * (blockDim.x >> 5), ordered);
   static_assert(B % G == 0 && 32 % G == 0 && PPL >= 1 && (KPL == 1 || KPL == 2), "tile shape");
   const int lane = threadIdx.x & 31;
   const int r = lane & (G - 1);
@@ -239,7 +247,11 @@ bucketed_insert_kernel(TableView tv, const uint32_t *__restrict__ keys,
             phase[s] = 0;
             b_b[s] = 0xFFFFFFFFu;
             l_a[s] = B + 1;
-            cur[s] = bucket_of(tv.hf, SCHEME == kBCHT ? tv.first : 0, k);
+            if (SCHEME == kIHT && tv.first) {  // the primary holds its share: its load is read if it is needed
+              phase[s] = 1;
+              l_a[s] = -1;
+            }
+            cur[s] = bucket_of(tv.hf, SCHEME == kBCHT || SCHEME == kIHT ? tv.first : 0, k);
           }
         }
       }
@@ -320,10 +332,20 @@ bucketed_insert_kernel(TableView tv, const uint32_t *__restrict__ keys,
             l_b[s] = load; s_b[s] = my_slot; b_b[s] = cur[s];
             phase[s] = 2;
             cur[s] = bucket_of(tv.hf, 2, k);
+          } else if (phase[s] == 3) {  // both secondaries are full, the primary's load was not known
+            if (load < B) {
+              op[s] = 1;
+              target = slots + (uint64_t)cur[s] * B + my_slot;
+            } else {
+              fail = true;
+            }
           } else if (l_b[s] < B || load < B) {
             op[s] = 1;
             target = (l_b[s] <= load) ? slots + (uint64_t)b_b[s] * B + s_b[s]
                                       : slots + (uint64_t)cur[s] * B + my_slot;
+          } else if (l_a[s] < 0) {
+            phase[s] = 3;
+            cur[s] = bucket_of(tv.hf, 0, k);
           } else if (l_a[s] < B) {
             op[s] = 1;
             target = slots + (uint64_t)b_a[s] * B + s_a[s];
@@ -383,7 +405,8 @@ bucketed_insert_kernel(TableView tv, const uint32_t *__restrict__ keys,
 }
 
 // ----------------------------------------------------------------------------
-// Ranked first-choice placement: phase 1 of a two-phase BCHT build.
+// Ranked first-choice placement: phase 1 of a two-phase build (BCHT; IHT's
+// primaries, with `limit` = t - 1 in place of the bucket's slots).
 //
 // Sequential BCHT (Sec. III-A) may insert the keys in any order. Take the
 // order in which, first, every key that arrives at its first-choice bucket
@@ -416,7 +439,7 @@ __global__ void __launch_bounds__(256)
 rank_place_kernel(TableView tv, const uint32_t *__restrict__ keys, const uint32_t *__restrict__ values,
                   uint64_t n, uint32_t *__restrict__ counters, uint32_t *__restrict__ ovf_k,
                   uint32_t *__restrict__ ovf_v, uint64_t cap, const uint32_t *__restrict__ ends, uint32_t region,
-                  uint64_t region_M) {
+                  uint64_t region_M, uint32_t limit) {
   using T = typename S::T;
   T *slots = reinterpret_cast<T *>(tv.slots);
   unsigned long long *ovf_count = &tv.ctrl->reserved[0];
@@ -461,7 +484,7 @@ rank_place_kernel(TableView tv, const uint32_t *__restrict__ keys, const uint32_
     }
 #pragma unroll
     for (int u = 0; u < kPlacePerThread; ++u) {
-      const bool fits = ok[u] && r[u] < (uint32_t)B;
+      const bool fits = ok[u] && r[u] < limit;
       if (fits) slots[(uint64_t)b[u] * B + r[u]] = S::make(k[u], v[u]);
       if (COUNT && ok[u]) placed++;  // a visit of H_0, stored or not (the overflow insert starts at H_1)
       // overflow: one shared reservation per warp (< 2 * kPlaceTile entries

@@ -778,7 +778,7 @@ static cudaError_t insert_cfg(const BatchView &bv, const uint32_t *k, const uint
   int blocks = 0;
   cudaError_t e = grid_for(kern, items, o.blocks_per_sm, &blocks);
   if (e != cudaSuccess) return e;
-  kern<<<blocks, kThreads, 0, s>>>(bv, k, v, claim_plan(items, blocks, true));  // the fill zeroed the claim cursor
+  kern<<<blocks, kThreads, 0, s>>>(bv, k, v, claim_plan(items, (uint64_t)blocks * (kThreads / 32), true));  // the fill zeroed the claim cursor
   return cudaGetLastError();
 }
 

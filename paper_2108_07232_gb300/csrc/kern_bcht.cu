@@ -13,7 +13,7 @@ static cudaError_t insert_kpl(const TableView &tv, const uint32_t *k, const uint
   int blocks = 0;
   cudaError_t e = grid_for(kern, n, o.blocks_per_sm, &blocks);
   if (e != cudaSuccess) return e;
-  kern<<<blocks, kThreads, 0, s>>>(tv, k, v, n, claim_plan(n, blocks, o.ordered));
+  kern<<<blocks, kThreads, 0, s>>>(tv, k, v, n, o.ordered, o.overflow);
   return cudaGetLastError();
 }
 
@@ -48,11 +48,11 @@ static cudaError_t place_b(const TableView &tv, const uint32_t *k, const uint32_
   cudaError_t e = grid_for(kern, (n + kPlacePerThread - 1) / kPlacePerThread, 0, &blocks);
   if (e != cudaSuccess) return e;
   kern<<<blocks, kThreads, 0, s>>>(tv, k, v, n, pb.counters, pb.ovf_k, pb.ovf_v, pb.cap, pb.ends, pb.region,
-                                       pb.region_M);
+                                       pb.region_M, pb.limit);
   return cudaGetLastError();
 }
 
-cudaError_t launch_place_bcht(int B, const TableView &tv, const uint32_t *k, const uint32_t *v, uint64_t n,
+cudaError_t launch_place_pairs(int B, const TableView &tv, const uint32_t *k, const uint32_t *v, uint64_t n,
                               const PlaceBuffers &pb, bool count, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   if (B == 16) return place_b<16>(tv, k, v, n, pb, count, s);

@@ -9,11 +9,12 @@ namespace ght {
 // Fill (Sec. III-A: initialise all buckets to empty) and reset the control
 // block. slots16 covers the 16-byte aligned body; tail8 the last odd pair.
 __global__ void fill_kernel(uint4 *__restrict__ slots16, uint64_t n16, uint64_t *__restrict__ tail8,
-                            Ctrl *__restrict__ ctrl) {
+                            Ctrl *__restrict__ ctrl, uint32_t *__restrict__ counters, uint64_t m) {
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   const uint4 e = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += stride)
     slots16[i] = e;
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += stride) counters[i] = 0u;
   if (blockIdx.x == 0) {
     if (threadIdx.x == 0 && tail8) *tail8 = kEmptyPair;
     if (threadIdx.x < sizeof(Ctrl) / 8) reinterpret_cast<unsigned long long *>(ctrl)[threadIdx.x] = 0ull;
@@ -37,7 +38,7 @@ static cudaError_t insert_kpl(const TableView &tv, const uint32_t *k, const uint
   int blocks = 0;
   cudaError_t e = grid_for(kern, n, o.blocks_per_sm, &blocks);
   if (e != cudaSuccess) return e;
-  kern<<<blocks, kThreads, 0, s>>>(tv, k, v, n, claim_plan(n, blocks, o.ordered));
+  kern<<<blocks, kThreads, 0, s>>>(tv, k, v, n, o.ordered, o.overflow);
   return cudaGetLastError();
 }
 
@@ -145,13 +146,14 @@ cudaError_t launch_dup_check(const TableView &tv, int B, bool key_slots, const u
   return cudaGetLastError();
 }
 
-cudaError_t launch_fill(const TableView &tv, uint64_t num_slots, cudaStream_t s) {
+cudaError_t launch_fill(const TableView &tv, uint64_t num_slots, cudaStream_t s, uint32_t *counters, uint64_t m) {
   const uint64_t n16 = num_slots / 2;  // slots start 256-byte aligned
   uint64_t *tail = (num_slots & 1) ? tv.slots + (num_slots - 1) : nullptr;
   int blocks = 0;
   cudaError_t e = grid_for(fill_kernel, n16 > 0 ? n16 : 1, 0, &blocks);
   if (e != cudaSuccess) return e;
-  fill_kernel<<<blocks, kThreads, 0, s>>>(reinterpret_cast<uint4 *>(tv.slots), n16, tail, tv.ctrl);
+  fill_kernel<<<blocks, kThreads, 0, s>>>(reinterpret_cast<uint4 *>(tv.slots), n16, tail, tv.ctrl,
+                                      counters, counters ? m : 0);
   return cudaGetLastError();
 }
 

@@ -1,6 +1,7 @@
-// kern_place.cu -- first-choice placement of a two-phase bucketed cuckoo
-// build, one thread block per sub-group of consecutive first-choice buckets
-// (phase 1 of the build; the overflow is inserted by the cuckoo insert).
+// kern_place.cu -- first-choice placement of a two-phase build (BCHT, the set,
+// and IHT's primaries up to t - 1 keys), one thread block per sub-group of
+// consecutive first-choice buckets (phase 1 of the build; the overflow is
+// inserted by the scheme's insert).
 //
 // What it computes is the ranked placement of reading R18 (Sec. III-A with
 // the keys that reach their first-choice bucket H_0 while it has room
@@ -37,7 +38,7 @@ template <typename S, int B, bool COUNT>
 __global__ void __launch_bounds__(kBPThreads, 2)
 block_place_kernel(TableView tv, const uint32_t *__restrict__ pk, const uint32_t *__restrict__ pv,
                    const uint32_t *__restrict__ ends, uint32_t region, uint32_t bins, int fine_shift,
-                   uint32_t *__restrict__ ovf_k, uint32_t *__restrict__ ovf_v, uint64_t cap) {
+                   uint32_t *__restrict__ ovf_k, uint32_t *__restrict__ ovf_v, uint64_t cap, uint32_t limit) {
   using T = typename S::T;
   constexpr int kMaxBuckets = (int)(kBPImageBytes / (B * sizeof(T)));
   constexpr int kVecB = (int)(B * sizeof(T) / 16);  // 16-byte vectors per bucket
@@ -98,7 +99,7 @@ block_place_kernel(TableView tv, const uint32_t *__restrict__ pk, const uint32_t
         const uint32_t lb = bucket_of(tv.hf, 0, k[u]) - b0;
         const uint32_t r = atomicAdd(&bcnt[lb], 1u);
         if (COUNT) placed++;  // a visit of H_0, stored or not (the overflow insert starts at H_1)
-        if (r < (uint32_t)B) {
+        if (r < limit) {
           img[lb * B + r] = S::make(k[u], v[u]);
         } else {
           const uint32_t at = atomicAdd(&s_novf, 1u);
@@ -144,10 +145,11 @@ static cudaError_t place_blocks(const TableView &tv, const uint32_t *pk, const u
                                 cudaStream_t s) {
   auto kern = count ? block_place_kernel<S, B, true> : block_place_kernel<S, B, false>;
   int blocks = 0;
-  cudaError_t e = grid_for_smem(kern, kBPThreads, kBPImageBytes, (uint64_t)bins * kBPThreads, 0, &blocks);
+  const size_t image = ((size_t)B * sizeof(typename S::T)) << fine_shift;
+  cudaError_t e = grid_for_smem(kern, kBPThreads, image, (uint64_t)bins * kBPThreads, 0, &blocks);
   if (e != cudaSuccess) return e;
-  kern<<<blocks, kBPThreads, kBPImageBytes, s>>>(tv, pk, pv, ends, region, bins, fine_shift, pb.ovf_k, pb.ovf_v,
-                                                 pb.cap);
+  kern<<<blocks, kBPThreads, image, s>>>(tv, pk, pv, ends, region, bins, fine_shift, pb.ovf_k, pb.ovf_v, pb.cap,
+                                         pb.limit);
   return cudaGetLastError();
 }
 

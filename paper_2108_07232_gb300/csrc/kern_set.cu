@@ -16,7 +16,7 @@ static cudaError_t set_insert(const TableView &tv, const uint32_t *k, const uint
   int blocks = 0;
   cudaError_t e = grid_for(kern, n, o.blocks_per_sm, &blocks);
   if (e != cudaSuccess) return e;
-  kern<<<blocks, kThreads, 0, s>>>(tv, k, v, n, claim_plan(n, blocks, o.ordered));
+  kern<<<blocks, kThreads, 0, s>>>(tv, k, v, n, o.ordered, o.overflow);
   return cudaGetLastError();
 }
 
@@ -43,7 +43,7 @@ cudaError_t launch_place_set(const TableView &tv, const uint32_t *k, uint64_t n,
   if (e != cudaSuccess) return e;
   // a set has no values: the key array stands in for them and is ignored
   kern<<<blocks, kThreads, 0, s>>>(tv, k, k, n, pb.counters, pb.ovf_k, pb.ovf_v, pb.cap, pb.ends, pb.region,
-                                       pb.region_M);
+                                       pb.region_M, pb.limit);
   return cudaGetLastError();
 }
 

@@ -44,7 +44,8 @@ def _check(G, scheme, n, lf, seed, n_queries=None, **cfg):
 # 3,735,552 pairs: 32 chunks of 32 pairs for each of 152 x 3 x 8 warps
 @pytest.mark.parametrize("scheme,lf,n", [("bcht", 0.9, 31), ("bcht", 0.9, 33), ("p2bht", 0.7, 4097),
                                          ("bcht", 0.95, 116736), ("bcht", 0.95, 116737), ("bcht", 0.99, 3735551),
-                                         ("iht", 0.8, 3735553), ("p2bht", 0.75, 5000011)])
+                                         ("iht", 0.8, 3735553), ("p2bht", 0.75, 5000011),
+                                         ("iht", 0.8, (1 << 24) + 3)])
 def test_insert_shares(G, scheme, lf, n):
     _check(G, scheme, n, lf, seed=n & 0xFFFF)
 
