@@ -380,6 +380,7 @@ struct ght_table {
     const uint64_t steps = ((uint64_t)shape.max_chain + 2ull) * (uint64_t)shape.h * ((uint64_t)shape.b + 2ull) + 64ull;
     v.max_steps = shape.max_steps ? shape.max_steps : (uint32_t)std::min<uint64_t>(steps, 0xFFFFFFF0ull);
     v.first = 0;
+    v.look = shape.m < (1u << 13) ? 4u : 24u;
     return v;
   }
 

@@ -136,6 +136,7 @@ struct TableView {
   uint32_t max_chain;  // cuckoo exchanges per insert
   uint32_t rng_seed;   // eviction xorshift seed
   uint32_t max_steps;  // per-key bound on build rounds (timeout)
+  uint32_t look;       // BCHT: exchanges of one insert from which victims are chosen (see choose_victims)
   int32_t first;       // BCHT and IHT: hash index a new key starts at (1 for keys whose H_0 is known to be full)
 };
 

@@ -126,6 +126,63 @@ constexpr int insert_min_blocks() {
   return B == 16 && G == 16 && KPL == 1 && !COUNT ? 3 : 0;
 }
 
+// Victims for the BCHT owners in `look`, whose buckets are full: the slot of a
+// key whose next bucket still has room (its last slot is empty, the one an
+// insert fills last), or -1. A tile serves its owners one after the other:
+// each lane reads its part of the bucket's keys and peeks at the last slot of
+// each key's next bucket. The exchange itself stays as it was: it takes
+// whichever pair is in the slot by then.
+//
+// This ends the long chains, which are what a build inside the L2 waits for:
+// each exchange is a read and an atomic, ~1.7 us, and at LF 0.99 the longest of
+// 4 M inserts made 161 of them (now 32). It is not for every eviction: a look
+// reads up to 16 more sectors, and from the first exchange on it took the
+// overflow insert of 2^28 keys from 4.8 to 8.8 ms. Used from the 25th exchange
+// of one insert (the average insert probes stay the random walk's, 1.39
+// against 1.42 at LF 0.99): 2^20 keys LF 0.99 insert 234 -> 96 us, 2^22 LF 0.95
+// 88 -> 80, 2^28 LF 0.99 4740 -> 4670. Tables below 8192 buckets use it from the
+// 5th: 20,000 keys LF 0.95 61 -> 50 us.
+template <int B, int G, typename S>
+__device__ __noinline__ int choose_victims(const TableView &tv, unsigned look, uint32_t cur, int tbase, unsigned tmask,
+                                           int r, int lane, uint32_t rng) {
+  using T = typename S::T;
+  constexpr int PPL = B / G;
+  const T *slots = reinterpret_cast<const T *>(tv.slots);
+  int victim = -1;
+  while (look != 0u) {
+    const unsigned mine = look & tmask;
+    const int o = mine ? __ffs(mine) - 1 : lane;
+    const uint32_t at = __shfl_sync(kFull, cur, o);
+    int mv = -1;  // a movable key of this lane's part
+    if (mine) {
+      uint32_t k[PPL];
+      load_keys_rw<PPL>(slots + (uint64_t)at * B, r, k);
+#pragma unroll
+      for (int p = 0; p < PPL; ++p) {
+        int i = tv.h;  // hash index the key is stored under
+        for (int f = tv.h - 1; f >= 0; --f)
+          if (bucket_of(tv.hf, f, k[p]) == at) i = f;
+        if (i + 1 < tv.h) {  // (from the last hash a key returns to H_0, which is full)
+          const T *last = slots + (uint64_t)bucket_of(tv.hf, i + 1, k[p]) * B + (B - 1);
+          uint32_t x;
+          asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(x) : "l"(last) : "memory");
+          if (x == kEmptyKey) mv = p;
+        }
+      }
+    }
+    const unsigned can = (__ballot_sync(kFull, mv >= 0) & tmask) >> tbase;
+    if (can != 0u) {  // the first movable lane from a random one on
+      const int from = (int)(__shfl_sync(tmask, rng, o) >> 8) & (G - 1);
+      const unsigned turned = ((can >> from) | (can << (G - from))) & ((1u << G) - 1u);
+      const int src = (__ffs(turned) - 1 + from) & (G - 1);
+      const int slot = src * PPL + __shfl_sync(tmask, mv, tbase + src);
+      if (lane == o) victim = slot;
+    }
+    look &= ~__ballot_sync(kFull, mine != 0u && lane == o);
+  }
+  return victim;
+}
+
 template <int SCHEME, int B, int G, int KPL, bool COUNT, typename S = PairSlot>
 __global__ void __launch_bounds__(256, insert_min_blocks<B, G, KPL, COUNT>())
 bucketed_insert_kernel(TableView tv, const uint32_t *__restrict__ keys,
@@ -283,6 +340,15 @@ bucketed_insert_kernel(TableView tv, const uint32_t *__restrict__ keys,
         }
       }
 
+      int victim = -1;
+      if (SCHEME == kBCHT) {
+        const unsigned look = __ballot_sync(kFull, active[s] && my_empty == 0 && chain[s] >= tv.look && chain[s] < tv.max_chain);
+        if (look != 0u) {
+          xorshift32(rng);
+          victim = choose_victims<B, G, S>(tv, look, cur[s], tbase, tmask, r, lane, rng);
+        }
+      }
+
       // -- decide and issue this slot's atomic
       T *target = nullptr;
       if (active[s]) {
@@ -304,7 +370,7 @@ bucketed_insert_kernel(TableView tv, const uint32_t *__restrict__ keys,
             fail = true;
           } else {
             op[s] = 2;
-            target = slots + (uint64_t)cur[s] * B + (xorshift32(rng) % B);
+            target = slots + (uint64_t)cur[s] * B + (victim >= 0 ? (uint32_t)victim : xorshift32(rng) % B);
           }
         } else if (SCHEME == kP2BHT) {
           if (phase[s] == 0) {
