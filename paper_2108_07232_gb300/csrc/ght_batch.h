@@ -30,6 +30,15 @@ struct BatchView {
 
 constexpr uint64_t kLineFindMost = 0xFFFF0000ull;  // queries of one batched line find (32-bit places)
 
+// Scratch of a batch's ranked placement: an arrival counter per bucket of the
+// whole slot array, and the overflow list.
+struct BatchPlace {
+  uint64_t *slots = nullptr;  // first slot of the batch
+  uint32_t *counters = nullptr;
+  uint32_t *k = nullptr, *v = nullptr, *table = nullptr;
+  uint64_t cap = 0;
+};
+
 bool batch_shape_supported(int tile_lanes, int keys_per_lane);
 // Find shapes: the above, of which 4-lane tiles with one query per lane are the
 // line find (32-byte loads, the default), and 4-lane tiles with 6 query sets
@@ -46,7 +55,13 @@ cudaError_t launch_segment_gather(const uint32_t *const *src, const uint64_t *of
                                   uint64_t n, cudaStream_t s);
 cudaError_t launch_segment_scatter(const uint32_t *src, uint32_t *const *dst, const uint64_t *offs, uint32_t segs,
                                    uint64_t n, cudaStream_t s);
-cudaError_t launch_batch_fill(const BatchView &bv, uint64_t *slots, uint64_t num_slots, cudaStream_t s);
+// counters: zeroed too where given, the first of them that of slots' first bucket
+cudaError_t launch_batch_fill(const BatchView &bv, uint64_t *slots, uint64_t num_slots, uint32_t *counters,
+                              cudaStream_t s);
+// Two-phase build of the filled tables: ranked placement, then the insert of
+// its overflow (16 lanes, one key per lane).
+cudaError_t launch_batch_place(const BatchView &bv, const BatchPlace &bl, const uint32_t *k, const uint32_t *v,
+                               uint64_t items, const LaunchOpts &o, cudaStream_t s);
 cudaError_t launch_batch_insert(const BatchView &bv, const uint32_t *k, const uint32_t *v, uint64_t items,
                                 const LaunchOpts &o, cudaStream_t s);
 cudaError_t launch_batch_find(const BatchView &bv, const uint32_t *q, uint32_t *out, uint64_t items,

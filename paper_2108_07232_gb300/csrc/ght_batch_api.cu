@@ -25,6 +25,8 @@ struct ght_batch {
   cudaStream_t capture_stream = nullptr;  // private stream the graph is captured on
   // device memory: slots of all tables, then descriptors, offsets, control block
   void *slots_mem = nullptr, *meta_mem = nullptr;
+  void *place_mem = nullptr;  // scratch of the two-phase build
+  ght::BatchPlace place;
   uint64_t total_slots = 0, slot_bytes = 0;
   ght::BatchTable *d_tables = nullptr;
   uint64_t *d_key_offs = nullptr, *d_query_offs = nullptr;
@@ -103,14 +105,23 @@ int download_tables(ght_batch *b, uint32_t lo, uint32_t hi) {
   return wait_event(b->done);
 }
 
-// Fill + insert of tables [lo, hi) (no wait).
-int launch_build(ght_batch *b, uint32_t lo, uint32_t hi, const uint32_t *k, const uint32_t *v) {
+// Overflow list of a two-phase batch build of n keys, as for one table.
+uint64_t place_cap(uint64_t n) { return std::min<uint64_t>(n, n / 4 + 1024); }
+
+// Fill + insert of tables [lo, hi) (no wait): in two phases with the default
+// insert shape, unless `plain` (a rebuild, whatever made the first attempt fail).
+int launch_build(ght_batch *b, uint32_t lo, uint32_t hi, const uint32_t *k, const uint32_t *v, bool plain = false) {
   const ght::BatchView bv = b->view(lo, hi);
+  const uint64_t items = b->key_offs[hi] - b->key_offs[lo];
+  const bool two = !plain && b->place.cap > 0 && b->build_o.tile_lanes == 16 && b->build_o.keys_per_lane == 1 &&
+                   items <= 0xFFFF0000ull;
   uint64_t *slots = static_cast<uint64_t *>(b->slots_mem) + b->slot_off[lo];
   const uint64_t nslots = b->slot_off[hi] - b->slot_off[lo];
-  cudaError_t e = ght::launch_batch_fill(bv, slots, nslots, b->stream);
+  cudaError_t e = ght::launch_batch_fill(bv, slots, nslots, two ? b->place.counters + b->slot_off[lo] / 16 : nullptr,
+                                         b->stream);
   if (e != cudaSuccess) return cuda_fail(e, "launching batch fill");
-  e = ght::launch_batch_insert(bv, k, v, b->key_offs[hi] - b->key_offs[lo], b->build_o, b->stream);
+  e = two ? ght::launch_batch_place(bv, b->place, k, v, items, b->build_o, b->stream)
+          : ght::launch_batch_insert(bv, k, v, items, b->build_o, b->stream);
   return e == cudaSuccess ? GHT_OK : cuda_fail(e, "launching batch insert");
 }
 
@@ -134,7 +145,7 @@ int repair(ght_batch *b, const uint32_t *k, const uint32_t *v, const uint32_t *q
       b->set_constants(t, b->attempt[t] + 1);
       b->rebuilds++;
       int rc = upload_tables(b, t, t + 1);
-      if (!rc) rc = launch_build(b, t, t + 1, k, v);
+      if (!rc) rc = launch_build(b, t, t + 1, k, v, true);
       if (!rc) rc = download_tables(b, t, t + 1);
       if (rc) return rc;
       st = b->h_tables[t].status;
@@ -250,6 +261,19 @@ ght_batch *ght_batch_create(uint32_t num_tables, const uint64_t *h_capacities, c
     ght_batch_destroy(b);
     return nullptr;
   }
+  // scratch of the two-phase build; without it (no memory) builds insert every key
+  uint64_t keys_most = 0;
+  for (uint32_t t = 0; t < num_tables; ++t) keys_most += h_capacities[t];
+  const uint64_t cap = place_cap(keys_most), counters = b->total_slots / 16;
+  if (keys_most > 0 && cudaMalloc(&b->place_mem, (counters + 3 * cap) * sizeof(uint32_t)) == cudaSuccess) {
+    b->place.slots = static_cast<uint64_t *>(b->slots_mem);
+    b->place.counters = static_cast<uint32_t *>(b->place_mem);
+    b->place.k = b->place.counters + counters;
+    b->place.v = b->place.k + cap;
+    b->place.table = b->place.v + cap;
+    b->place.cap = cap;
+  }
+  cudaGetLastError();
   char *p = static_cast<char *>(b->meta_mem);
   b->d_tables = reinterpret_cast<ght::BatchTable *>(p);
   p += num_tables * sizeof(ght::BatchTable);
@@ -549,6 +573,7 @@ void ght_batch_destroy(ght_batch *b) {
   cudaStreamSynchronize(b->stream);
   if (b->slots_mem) cudaFree(b->slots_mem);
   if (b->meta_mem) cudaFree(b->meta_mem);
+  if (b->place_mem) cudaFree(b->place_mem);
   if (b->h_tables) cudaFreeHost(b->h_tables);
   if (b->done) cudaEventDestroy(b->done);
   if (b->ev0) cudaEventDestroy(b->ev0);

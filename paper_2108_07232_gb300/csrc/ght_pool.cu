@@ -336,7 +336,19 @@ void ght_pool::build_loop() {
       if (!t) rc = GHT_ERR_INVALID_ARG;
     }
     if (rc == GHT_OK) rc = ght_set_stream(t, build_stream);
+    // scratch of a two-phase build, for this build only (without it the build inserts every key)
+    void *scratch = nullptr;
+    const uint64_t need = rc == GHT_OK ? ght_build_scratch_bytes(t, r.n) : 0;
+    if (need && ght::host::pool_alloc(&scratch, need, build_stream) != cudaSuccess) {
+      cudaGetLastError();
+      scratch = nullptr;
+    }
+    if (scratch) ght_set_build_scratch(t, scratch, need);
     if (rc == GHT_OK) rc = ght_build(t, r.values ? r.in : nullptr, r.values, r.n);
+    if (scratch) {
+      ght_set_build_scratch(t, nullptr, 0);
+      cudaFreeAsync(scratch, build_stream);
+    }
     std::lock_guard<std::mutex> lock(mu);
     pt.t = t;
     pt.storage = storage;

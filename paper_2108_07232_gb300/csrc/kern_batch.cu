@@ -7,6 +7,8 @@
 // range. Work is split over warps exactly as in the single-table kernels; a
 // lane finds the table of the item it takes from a per-chunk hint (one
 // uniform binary search per 32 items) and reads that table's descriptor.
+#include <algorithm>
+
 #include "ght_batch.h"
 #include "ght_find_async.cuh"
 #include "ght_find_line.cuh"
@@ -31,6 +33,17 @@ __device__ __forceinline__ uint32_t advance_table(const uint64_t *__restrict__ o
   return tb;
 }
 
+// As table_of for an index a little beyond table tb's first: steps double from tb.
+__device__ __forceinline__ uint32_t seek_table(const uint64_t *__restrict__ offs, uint32_t tb, uint32_t t_hi,
+                                               uint64_t i) {
+  uint32_t step = 1;
+  while (tb + step < t_hi && __ldg(offs + tb + step) <= i) {
+    tb += step;
+    step *= 2;
+  }
+  return table_of(offs, tb, min(tb + step, t_hi), i);
+}
+
 __device__ __forceinline__ uint32_t batch_bucket(const BatchTable &d, int i, uint32_t k) {
   return fastmod(mod_prime((uint64_t)select4(d.a, i) * k + select4(d.c, i)), d.mod);
 }
@@ -49,7 +62,7 @@ __device__ __forceinline__ void bq_load(uint32_t &k, uint32_t &v, uint32_t &t, c
                                         const BatchView &bv, const uint64_t *__restrict__ offs, int lane) {
   k = stream_load(keys, at + lane, end);
   if (PAIRS) v = stream_load(vals, at + lane, end);
-  t = at < end ? table_of(offs, bv.t_lo, bv.t_hi, at) : bv.t_lo;
+  t = offs && at < end ? table_of(offs, bv.t_lo, bv.t_hi, at) : bv.t_lo;  // (an overflow list has no offsets)
 }
 
 template <bool PAIRS>
@@ -150,39 +163,148 @@ __device__ __forceinline__ uint64_t bc_take(BatchClaimQueue &q, const uint32_t *
     bq_load<true>(q.kc, q.vc, q.tc, keys, vals, q.bc, hi, bv, offs, lane);
   }
   if (!((need >> lane) & 1u) || at >= hi) return ~0ull;
-  table = advance_table(offs, table, bv.t_hi, at);
+  if (offs) table = advance_table(offs, table, bv.t_hi, at);
   return at;
 }
 
 // ----------------------------------------------------------------------------
 // Fill the slots of tables [t_lo, t_hi) and clear their status words.
-__global__ void __launch_bounds__(256) batch_fill_kernel(BatchView bv, uint4 *__restrict__ slots16, uint64_t n16) {
+__global__ void __launch_bounds__(256)
+batch_fill_kernel(BatchView bv, uint4 *__restrict__ slots16, uint64_t n16, uint32_t *__restrict__ counters) {
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   const uint4 e = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += stride) slots16[i] = e;
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += stride) {
+    slots16[i] = e;
+    if (counters && (i & 7u) == 0u) counters[i >> 3] = 0u;  // one per bucket of 8 pieces
+  }
   for (uint64_t t = bv.t_lo + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < bv.t_hi; t += stride)
     bv.tables[t].status = 0u;
-  if (blockIdx.x == 0 && threadIdx.x == 0) bv.ctrl->work_cursor = 0ull;  // the insert's claims start at zero
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    bv.ctrl->work_cursor = 0ull;  // the insert's claims start at zero
+    bv.ctrl->reserved[0] = 0ull;  // so does the overflow list
+  }
+}
+
+// ----------------------------------------------------------------------------
+// Ranked first-choice placement of a batch (phase 1 of its build, as
+// rank_place_kernel for one table): a key's arrival number at its bucket H_0
+// comes from the bucket's counter (bl.counters, one per bucket in slot order),
+// numbers below 16 are stored in that slot, the other keys go to the overflow
+// list with their table. A key that no longer fits the list fails its table's
+// attempt (the table is then rebuilt alone). The warps take the chunks of 32
+// pairs in turn, so the stores and counters in flight stay in the few tables
+// that the chunks are in. Build of 512 tables of 2^10..2^20 keys at LF
+// 0.8..0.99 (85 M keys): 3.75 ms with the insert of every key, 2.54 now; 64
+// tables of 2^12..2^22 keys 2.05 -> 1.29; 512 of 2^10..2^14 0.39 -> 0.26.
+template <bool COUNT>
+__global__ void __launch_bounds__(256)
+batch_place_kernel(BatchView bv, BatchPlace bl, const uint32_t *__restrict__ keys,
+                   const uint32_t *__restrict__ values, uint32_t n) {
+  // each warp's overflow, appended 32 keys at a time: one reservation each (a
+  // reservation per key, all on one address, took longer than the placement)
+  __shared__ uint32_t s_over[8][3][64];
+  const uint64_t *offs = bv.key_offs;
+  const int lane = threadIdx.x & 31;
+  uint32_t(*over)[64] = s_over[threadIdx.x >> 5];
+  const unsigned below = lanemask_lt();
+  int waiting = 0;
+  const uint32_t step = gridDim.x * blockDim.x;
+  const uint32_t start = blockIdx.x * blockDim.x + (threadIdx.x & ~31u);
+  if (start >= n) return;  // whole warp
+  auto append = [&](int take) {
+    unsigned long long at = 0ull;
+    if (lane == 0) at = atomicAdd(&bv.ctrl->reserved[0], (unsigned long long)take);
+    at = __shfl_sync(kFull, at, 0) + lane;
+    waiting -= take;
+    if (lane < take) {
+      if (at < bl.cap) {
+        bl.k[at] = over[0][waiting + lane];
+        bl.v[at] = over[1][waiting + lane];
+        bl.table[at] = over[2][waiting + lane];
+      } else {
+        atomicOr(&bv.tables[over[2][waiting + lane]].status, kStatusBuildFailed);
+      }
+    }
+    __syncwarp();
+  };
+  const uint64_t lo = __ldg(offs + bv.t_lo);
+  keys += lo;
+  values += lo;
+  unsigned long long placed = 0;
+  uint32_t first = table_of(offs, bv.t_lo, bv.t_hi, lo + start);
+  uint32_t nk = start + lane < n ? __ldg(keys + start + lane) : 0u;
+  uint32_t nv = start + lane < n ? __ldg(values + start + lane) : 0u;
+  for (uint32_t c = start;;) {
+    const uint32_t i = c + lane, k = nk, v = nv;
+    const bool more = c < n - min(n, step);
+    if (more) {
+      nk = i + step < n ? __ldg(keys + i + step) : 0u;
+      nv = i + step < n ? __ldg(values + i + step) : 0u;
+    }
+    bool overflows = false;
+    uint32_t tb = 0;
+    if (i < n) {
+      tb = advance_table(offs, first, bv.t_hi, lo + i);
+      if (k == kEmptyKey) {
+        atomicOr(&bv.tables[tb].status, kStatusSentinel);
+      } else {
+        const BatchTable &d = bv.tables[tb];
+        const uint32_t b = batch_bucket(d, 0, k);
+        const uint64_t bucket = (uint64_t)(d.slots - bl.slots) / 16u + b;
+        const uint32_t r = atomicAdd(bl.counters + bucket, 1u);
+        if (COUNT) placed++;
+        overflows = r >= 16u;
+        if (!overflows) bl.slots[bucket * 16u + r] = ((uint64_t)v << 32) | k;
+      }
+    }
+    const unsigned om = __ballot_sync(kFull, overflows);
+    if (overflows) {
+      const int x = waiting + __popc(om & below);
+      over[0][x] = k;
+      over[1][x] = v;
+      over[2][x] = tb;
+    }
+    waiting += __popc(om);
+    __syncwarp();
+    if (waiting >= 32) append(32);
+    if (!more) break;
+    c += step;
+    first = seek_table(offs, first, bv.t_hi, lo + c);
+  }
+  if (waiting > 0) append(waiting);
+  if (COUNT) {
+    placed = warp_sum(placed);
+    if (lane == 0) atomicAdd(&bv.ctrl->insert_probes, placed);
+  }
 }
 
 // ----------------------------------------------------------------------------
 // BCHT bulk build of every table in [t_lo, t_hi) (Sec. III-A, V-B), with the
 // turn structure, chunk claims (the batch's work cursor, zeroed by the fill),
 // key-word gathers and register bound of the single-table insert kernel.
-template <int G, int KPL, bool COUNT>
+//
+// LIST: the pairs are the overflow list of the batch's placement (bl), of the
+// length that the control block gives; they start at H_1, H_0 being full.
+template <int G, int KPL, bool COUNT, bool LIST>
 __global__ void __launch_bounds__(256, insert_min_blocks<16, G, KPL, COUNT>())
 batch_insert_kernel(BatchView bv, const uint32_t *__restrict__ keys, const uint32_t *__restrict__ values,
-                    ClaimPlan plan) {
+                    ClaimPlan plan, BatchPlace bl) {
   constexpr int B = 16;
   constexpr int PPL = B / G;
   static_assert(B % G == 0 && 32 % G == 0 && (KPL == 1 || KPL == 2), "tile shape");
-  const uint64_t *offs = bv.key_offs;
+  const uint64_t *offs = LIST ? nullptr : bv.key_offs;
   const int lane = threadIdx.x & 31;
   const int r = lane & (G - 1);
   const int tbase = lane - r;
   const unsigned tmask = (G == 32 ? kFull : ((1u << G) - 1u)) << tbase;
   const uint64_t gtid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const uint64_t lo = __ldg(offs + bv.t_lo), hi = __ldg(offs + bv.t_hi);
+  const uint64_t lo = LIST ? 0ull : __ldg(offs + bv.t_lo);
+  const uint64_t hi = LIST ? min(bv.ctrl->reserved[0], (unsigned long long)bl.cap) : __ldg(offs + bv.t_hi);
+  if (LIST) {
+    keys = bl.k;
+    values = bl.v;
+    plan = claim_plan(hi, (uint64_t)gridDim.x * (blockDim.x >> 5), true);
+  }
   const unsigned below = lanemask_lt();
   const int h = bv.h;
 
@@ -239,6 +361,7 @@ batch_insert_kernel(BatchView bv, const uint32_t *__restrict__ keys, const uint3
         uint32_t k, val, tb;
         const uint64_t at = bc_take(q, keys, values, plan, shared, hi, bv, offs, need, below, lane, k, val, tb);
         if (at != ~0ull) {
+          if (LIST) tb = __ldg(bl.table + at);
           if (k == kEmptyKey) {
             atomicOr(&bv.tables[tb].status, kStatusSentinel);
           } else {
@@ -247,7 +370,7 @@ batch_insert_kernel(BatchView bv, const uint32_t *__restrict__ keys, const uint3
             active[s] = true;
             retrying[s] = false;
             chain[s] = steps[s] = 0;
-            cur[s] = batch_bucket(bv.tables[tb], 0, k);
+            cur[s] = batch_bucket(bv.tables[tb], LIST ? 1 : 0, k);
           }
         }
       }
@@ -448,17 +571,6 @@ batch_find_kernel(BatchView bv, const uint32_t *__restrict__ queries, uint32_t *
 
 // ----------------------------------------------------------------------------
 constexpr int kBatchTableBits = 30;  // a waiting query's table, below its next probe (h <= 4)
-
-// As table_of for an index a little beyond table tb's first: steps double from tb.
-__device__ __forceinline__ uint32_t seek_table(const uint64_t *__restrict__ offs, uint32_t tb, uint32_t t_hi,
-                                               uint64_t i) {
-  uint32_t step = 1;
-  while (tb + step < t_hi && __ldg(offs + tb + step) <= i) {
-    tb += step;
-    step *= 2;
-  }
-  return table_of(offs, tb, min(tb + step, t_hi), i);
-}
 
 // The same find with 32-byte loads (the line find, ght_find_line.cuh): 32
 // queries per step, those that need another bucket wait in shared memory with
@@ -762,23 +874,25 @@ static cudaError_t launch_sliced(K kern, uint64_t items, int blocks_per_sm, cuda
   return cudaSuccess;
 }
 
-cudaError_t launch_batch_fill(const BatchView &bv, uint64_t *slots, uint64_t num_slots, cudaStream_t s) {
+cudaError_t launch_batch_fill(const BatchView &bv, uint64_t *slots, uint64_t num_slots, uint32_t *counters,
+                              cudaStream_t s) {
   const uint64_t n16 = num_slots / 2;  // every table's slot count is even (b = 16)
   int blocks = 0;
   cudaError_t e = grid_for(batch_fill_kernel, n16 > 0 ? n16 : 1, 0, &blocks);
   if (e != cudaSuccess) return e;
-  batch_fill_kernel<<<blocks, kThreads, 0, s>>>(bv, reinterpret_cast<uint4 *>(slots), n16);
+  batch_fill_kernel<<<blocks, kThreads, 0, s>>>(bv, reinterpret_cast<uint4 *>(slots), n16, counters);
   return cudaGetLastError();
 }
 
 template <int G, int KPL>
 static cudaError_t insert_cfg(const BatchView &bv, const uint32_t *k, const uint32_t *v, uint64_t items,
                               const LaunchOpts &o, cudaStream_t s) {
-  auto kern = o.count ? batch_insert_kernel<G, KPL, true> : batch_insert_kernel<G, KPL, false>;
+  auto kern = o.count ? batch_insert_kernel<G, KPL, true, false> : batch_insert_kernel<G, KPL, false, false>;
   int blocks = 0;
   cudaError_t e = grid_for(kern, items, o.blocks_per_sm, &blocks);
   if (e != cudaSuccess) return e;
-  kern<<<blocks, kThreads, 0, s>>>(bv, k, v, claim_plan(items, (uint64_t)blocks * (kThreads / 32), true));  // the fill zeroed the claim cursor
+  kern<<<blocks, kThreads, 0, s>>>(bv, k, v, claim_plan(items, (uint64_t)blocks * (kThreads / 32), true),
+                                   BatchPlace());  // the fill zeroed the claim cursor
   return cudaGetLastError();
 }
 
@@ -885,6 +999,22 @@ cudaError_t launch_batch_insert(const BatchView &bv, const uint32_t *k, const ui
   if (g == 8) return kpl == 1 ? insert_cfg<8, 1>(bv, k, v, items, o, s) : insert_cfg<8, 2>(bv, k, v, items, o, s);
   if (g == 4) return kpl == 1 ? insert_cfg<4, 1>(bv, k, v, items, o, s) : insert_cfg<4, 2>(bv, k, v, items, o, s);
   return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_batch_place(const BatchView &bv, const BatchPlace &bl, const uint32_t *k, const uint32_t *v,
+                               uint64_t items, const LaunchOpts &o, cudaStream_t s) {
+  if (items == 0) return cudaSuccess;
+  if (items > 0xFFFF0000ull) return cudaErrorInvalidValue;  // 32-bit places
+  int blocks = 0;
+  auto place = o.count ? batch_place_kernel<true> : batch_place_kernel<false>;
+  cudaError_t e = grid_for(place, items, 0, &blocks);
+  if (e != cudaSuccess) return e;
+  place<<<blocks, kThreads, 0, s>>>(bv, bl, k, v, (uint32_t)items);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  auto insert = o.count ? batch_insert_kernel<16, 1, true, true> : batch_insert_kernel<16, 1, false, true>;
+  if ((e = grid_for(insert, std::min<uint64_t>(items, bl.cap), o.blocks_per_sm, &blocks)) != cudaSuccess) return e;
+  insert<<<blocks, kThreads, 0, s>>>(bv, nullptr, nullptr, ClaimPlan(), bl);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_batch_find(const BatchView &bv, const uint32_t *q, uint32_t *out, uint64_t items,

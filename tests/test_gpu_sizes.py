@@ -117,3 +117,22 @@ def test_pool_requests_of_all_sizes(G, cfg):
     for i, (q, o) in enumerate(zip(qs, outs)):
         assert (O._u32(o.cpu()) == O.lookup(*sets[i & 1], q)).all(), i
     pool.close()
+
+
+def test_batch_overflow_beyond_the_list_rebuilds_the_table(G):
+    """Every key of one table in one bucket under its first constants: its overflow outgrows the
+    batch's list, and the table is rebuilt alone."""
+    n, seed = 6000, 29
+    m = O.num_buckets(n, 0.5, 16)
+    a, c = O.derive_constants(seed, 0, 3)
+    cand = np.arange(1, 1 << 24, dtype=np.uint64)
+    h0 = ((np.uint64(a[0]) * cand + np.uint64(c[0])) % np.uint64(O.PRIME)) % np.uint64(m)
+    crowd = torch.from_numpy(cand[h0 == h0[0]][:n].astype(np.uint32).view(np.int32).copy())
+    assert crowd.numel() == n
+    other = W.make_keys(500, 3)
+    keys, vals = torch.cat([crowd, other]), W.make_values(n + 500, 8)
+    b = G.Batch([n, 500], [0.5, 0.9], seed=seed)
+    offs = np.array([0, n, n + 500], dtype=np.uint64)
+    b.set_layout(offs, offs)
+    out = O._u32(b.run(keys.cuda(), vals.cuda(), keys.cuda()).cpu())
+    assert (out == O._u32(vals)).all()
