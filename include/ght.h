@@ -112,7 +112,9 @@ typedef struct {
    * first-choice bucket while it has room (IHT: while it holds fewer than
    * threshold - 1 keys) is stored at its arrival rank without reading the
    * bucket, the rest are inserted by the scheme's insert (the same table,
-   * Sec. III-A and III-C, with those keys inserted first). 1 = on, -1 = off, 0 =
+   * Sec. III-A and III-C, with those keys inserted first). P2BHT and BCHT_LB:
+   * keys go to the least loaded candidate by the buckets' counts of arrivals
+   * (ungrouped), the rest of BCHT_LB's by its insert. 1 = on, -1 = off, 0 =
    * default: on where it pays (IHT: while few keys are expected beyond the
    * threshold; without grouping: tables below twice the L2). Needs scratch
    * (ght_build_scratch_bytes), else the build inserts every key. */

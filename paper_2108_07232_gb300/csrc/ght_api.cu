@@ -200,8 +200,7 @@ int resolve(int scheme, uint64_t capacity, double lf, const ght_config *user, Sh
   s->build_blocks_per_sm = d.build_blocks_per_sm;
   s->build_keys_per_lane = d.build_keys_per_lane;
   s->group_build = d.group_build;
-  // ranked placement applies to the cuckoo tables with buckets (BCHT and the set) and to IHT's primaries
-  s->ranked_build = (scheme == GHT_BCHT || scheme == GHT_BCHT_SET || scheme == GHT_IHT) ? d.ranked_build : -1;
+  s->ranked_build = scheme == GHT_CUCKOO1 ? -1 : d.ranked_build;
   s->slot_bytes = (int)slot_bytes;
   s->find_async = async_find ? 1 : 0;
   s->check_dups = d.check_duplicates > 0 ? 1 : 0;
@@ -466,6 +465,10 @@ uint32_t place_limit(const Shape &s) {
   return 0;
 }
 
+// The schemes whose placement counts arrivals at every candidate, not only at
+// the first choice (load_place_kernel).
+bool places_by_load(const Shape &s) { return s.scheme == GHT_P2BHT || s.scheme == GHT_BCHT_LB; }
+
 // Share of n keys beyond their first-choice bucket's `limit` under a random
 // hash (Poisson arrivals).
 double expected_overflow(uint64_t n, uint64_t m, uint32_t limit) {
@@ -499,7 +502,9 @@ bool places_ungrouped(const ght_table *t) {
 bool wants_ranked(const ght_table *t, uint64_t n) {
 
   const uint32_t limit = place_limit(t->shape);
-  if (!limit || t->shape.ranked_build < 0 || n == 0 || n > 0xFFFFFFFFull) return false;
+  if (t->shape.ranked_build < 0 || n == 0 || n > 0xFFFFFFFFull) return false;
+  if (places_by_load(t->shape)) return t->shape.group_build <= 0;  // in input order
+  if (!limit) return false;
   if (t->shape.group_build < 0 && !places_ungrouped(t)) return false;
   return t->shape.scheme != GHT_IHT || expected_overflow(n, t->shape.m, limit) <= 0.22;
 }
@@ -516,7 +521,7 @@ bool wants_ranked(const ght_table *t, uint64_t n) {
 bool wants_grouping(const ght_table *t, uint64_t n) {
   if (t->shape.scheme == GHT_CUCKOO1 || n == 0 || n > 0xFFFFFFFFull) return false;
   if (t->shape.group_build != 0) return t->shape.group_build > 0;
-  return wants_ranked(t, n) && t->storage_bytes >= device_l2_bytes();
+  return wants_ranked(t, n) && !places_by_load(t->shape) && t->storage_bytes >= device_l2_bytes();
 }
 
 // Second-level split of a two-phase grouped build (the block placement):
@@ -598,6 +603,8 @@ cudaError_t launch_place(const ght_table *t, const uint32_t *k, const uint32_t *
                          const ght::PlaceBuffers &pb) {
   const bool count = t->shape.count_probes != 0;
   if (t->shape.scheme == GHT_BCHT_SET) return ght::launch_place_set(t->view(), k, n, pb, count, t->stream);
+  if (places_by_load(t->shape))
+    return ght::launch_place_by_load(t->shape.b, t->view(), k, v, n, pb, t->shape.scheme == GHT_BCHT_LB, count, t->stream);
   return ght::launch_place_pairs(t->shape.b, t->view(), k, v, n, pb, count, t->stream);
 }
 
@@ -938,7 +945,7 @@ int build_device(ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n,
         break;
       }
       cudaEventRecord(t->tev[2], t->stream);
-      e = launch_insert_overflow(t, pb);
+      e = t->shape.scheme == GHT_P2BHT ? cudaSuccess : launch_insert_overflow(t, pb);  // (P2BHT has none)
     } else {
       cudaEventRecord(t->tev[2], t->stream);
       e = n > 0 ? launch_insert(t, ik, iv, n, grouped) : cudaSuccess;

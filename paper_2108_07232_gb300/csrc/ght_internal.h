@@ -160,6 +160,11 @@ cudaError_t launch_insert_other(int scheme, int B, const TableView &tv, const ui
                                 const uint32_t *v, uint64_t n, const LaunchOpts &o, cudaStream_t s);
 cudaError_t launch_find_other(int scheme, int B, const TableView &tv, const uint32_t *q,
                               uint32_t *out, uint64_t n, const LaunchOpts &o, cudaStream_t s);
+// Placement of every key into the least loaded of its h candidates; without
+// evicts a key that finds them all full fails the build, else it goes to pb's
+// overflow list.
+cudaError_t launch_place_by_load(int B, const TableView &tv, const uint32_t *k, const uint32_t *v, uint64_t n,
+                                 const PlaceBuffers &pb, bool evicts, bool count, cudaStream_t s);
 bool other_shape_supported(int scheme, int B, int G);
 // fills the table, resets its control block and, where given, zeroes the m arrival counters
 cudaError_t launch_fill(const TableView &tv, uint64_t num_slots, cudaStream_t s, uint32_t *counters = nullptr,

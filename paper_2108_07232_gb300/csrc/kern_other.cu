@@ -31,6 +31,130 @@ __global__ void hash_kernel(TableView tv, const uint32_t *__restrict__ keys, uin
   }
 }
 
+// ----------------------------------------------------------------------------
+// Placement by load, for the schemes that put a key into the least loaded of
+// its candidates (ties to the lowest hash index): P2BHT (two, Sec. III-B) and
+// the load-balanced BCHT (h, Sec. III-A last paragraph).
+//
+// A bucket's load is its count of arrivals, 4 bytes that stay in L2, instead
+// of 128 bytes of bucket: a key reads its candidates' counts, adds one to the
+// least by a CAS, and stores its pair in the slot of the old count. The CAS
+// fails when the bucket has grown since, and the key looks again: so the
+// choices are as balanced as those of the insert, whose CAS into the first
+// empty slot fails in the same case. (With a plain add, keys in flight choose
+// by old counts, and P2BHT at LF 0.8 failed on tables of up to 2^20 keys.)
+// P2BHT fails when all candidates are full; the load-balanced BCHT's keys then
+// go to the overflow list, whose insert evicts (Sec. III-A takes the keys in any
+// order, so also in this one).
+//
+// The insert that reads the buckets is bound by its random lines (two or three
+// 128-byte reads and a CAS per key); this by the L2's atomics and scattered
+// stores. Insert -> placement, us: P2BHT 2^20 keys LF 0.8 120 -> 60, 2^24 1095 ->
+// 570, 2^26 4830 -> 2790; load-balanced BCHT 2^22 LF 0.95 424 -> 201 with the
+// overflow's insert, 2^24 LF 0.9 1617 -> 644.
+template <bool COUNT>
+__global__ void __launch_bounds__(256)
+load_place_kernel(TableView tv, int B, const uint32_t *__restrict__ keys, const uint32_t *__restrict__ values,
+                  uint64_t n, uint32_t *__restrict__ counters, uint32_t *__restrict__ ovf_k,
+                  uint32_t *__restrict__ ovf_v, uint64_t cap) {
+  constexpr int kPer = 2;
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  const int h = tv.h;
+  unsigned long long probes = 0, retries = 0;
+  for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += stride * kPer) {
+    uint32_t k[kPer], v[kPer], b[kPer], c[kPer];
+    bool open[kPer];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      const uint64_t i = i0 + u * stride;
+      open[u] = i < n;
+      k[u] = open[u] ? __ldg(keys + i) : kEmptyKey;
+      v[u] = open[u] ? __ldg(values + i) : 0u;
+      if (open[u] && k[u] == kEmptyKey) {
+        atomicOr(&tv.ctrl->status, kStatusSentinel);
+        open[u] = false;
+      }
+    }
+    bool first = true;
+    for (uint32_t steps = h;; steps += h) {  // bucket visits of a key, as the inserts count them
+      bool any = false;
+#pragma unroll
+      for (int u = 0; u < kPer; ++u) {
+        c[u] = 0xFFFFFFFFu;
+        any |= open[u];
+        if (!open[u]) continue;
+        if (COUNT) (first ? probes : retries) += h;
+        uint32_t bf[4], cf[4];
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+          if (f >= h) continue;
+          bf[f] = bucket_of(tv.hf, f, k[u]);
+          asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(cf[f]) : "l"(counters + bf[f]) : "memory");
+        }
+#pragma unroll
+        for (int f = 0; f < 4; ++f)
+          if (f < h && cf[f] < c[u]) {
+            c[u] = cf[f];
+            b[u] = bf[f];
+          }
+      }
+      if (!any) break;
+      if (steps > tv.max_steps) {
+        atomicOr(&tv.ctrl->status, kStatusTimeout);
+        break;
+      }
+      uint32_t was[kPer];
+#pragma unroll
+      for (int u = 0; u < kPer; ++u)
+        if (open[u] && c[u] < (uint32_t)B) was[u] = atomicCAS(counters + b[u], c[u], c[u] + 1u);
+#pragma unroll
+      for (int u = 0; u < kPer; ++u) {
+        if (!open[u]) continue;
+        if (c[u] < (uint32_t)B) {
+          if (was[u] == c[u]) {
+            tv.slots[(uint64_t)b[u] * B + c[u]] = PairSlot::make(k[u], v[u]);
+            open[u] = false;
+          }
+        } else {  // every candidate is full
+          open[u] = false;
+          if (ovf_k) {
+            if (COUNT) (first ? probes : retries) -= h;  // the overflow's insert reads them
+            const unsigned long long at = atomicAdd(&tv.ctrl->reserved[0], 1ull);
+            if (at < cap) {
+              ovf_k[at] = k[u];
+              ovf_v[at] = v[u];
+            }
+          } else {
+            atomicOr(&tv.ctrl->status, kStatusBuildFailed);
+          }
+        }
+      }
+      first = false;
+    }
+    if ((load_status(tv.ctrl) & (kStatusBuildFailed | kStatusTimeout)) != 0u) break;
+  }
+  if (COUNT) {
+    probes = warp_sum(probes);
+    retries = warp_sum(retries);
+    if ((threadIdx.x & 31) == 0) {
+      atomicAdd(&tv.ctrl->insert_probes, probes);
+      atomicAdd(&tv.ctrl->insert_retries, retries);
+    }
+  }
+}
+
+cudaError_t launch_place_by_load(int B, const TableView &tv, const uint32_t *k, const uint32_t *v, uint64_t n,
+                                 const PlaceBuffers &pb, bool evicts, bool count, cudaStream_t s) {
+  if (n == 0) return cudaSuccess;
+  auto kern = count ? load_place_kernel<true> : load_place_kernel<false>;
+  int blocks = 0;
+  const cudaError_t e = grid_for(kern, (n + 1) / 2, 0, &blocks);
+  if (e != cudaSuccess) return e;
+  kern<<<blocks, kThreads, 0, s>>>(tv, B, k, v, n, pb.counters, evicts ? pb.ovf_k : nullptr,
+                                   evicts ? pb.ovf_v : nullptr, pb.cap);
+  return cudaGetLastError();
+}
+
 template <int S, int B, int G, int KPL>
 static cudaError_t insert_kpl(const TableView &tv, const uint32_t *k, const uint32_t *v,
                               uint64_t n, const LaunchOpts &o, cudaStream_t s) {

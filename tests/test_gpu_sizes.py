@@ -119,6 +119,14 @@ def test_pool_requests_of_all_sizes(G, cfg):
     pool.close()
 
 
+# placement by load: pairs of keys per thread, odd counts; buckets of 16 and 32, evictions at 0.99
+@pytest.mark.parametrize("scheme,b,lf,n", [("p2bht", 16, 0.8, 40001), ("p2bht", 32, 0.88, 622593), ("bcht_lb", 16, 0.99, 622592),
+                                           ("bcht_lb", 32, 0.99, 70003), ("p2bht", 16, 0.82, 5000011)])
+def test_placement_by_load(G, scheme, b, lf, n):
+    st = _check(G, scheme, n, lf, seed=n & 0xFFF, bucket_size=b)
+    assert st["last_build_ranked"] == 1 and st["last_build_grouped"] == 0
+
+
 def test_batch_overflow_beyond_the_list_rebuilds_the_table(G):
     """Every key of one table in one bucket under its first constants: its overflow outgrows the
     batch's list, and the table is rebuilt alone."""
