@@ -31,7 +31,8 @@
  *     stream once per attempt to read the build status.
  *   - Functions return a ght_status; on error ght_last_error() gives a
  *     thread-local message. No C++ exception crosses this ABI.
- *   - Every host wait for the device polls an event with a deadline: the
+ *   - Every host wait for the device polls (an event, or a number the device
+ *     writes to pinned memory) with a deadline: the
  *     environment variable GHT_WAIT_TIMEOUT_S in seconds (default 300); when
  *     it runs out the call returns GHT_ERR_DEVICE_TIMEOUT.
  *   - The hash family is h_i(k) = ((a_i k + c_i) mod p) mod m, p = 4294967291

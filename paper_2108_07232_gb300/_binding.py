@@ -2,6 +2,7 @@
 
 from __future__ import annotations
 
+import contextlib
 import ctypes as C
 import os
 import threading
@@ -123,6 +124,8 @@ def lib_path() -> str:
 def lib():
     """Load libght.so. Raises if it has not been built (no fallback path)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(_LIB_PATH):
@@ -351,6 +354,7 @@ class HashTable:
         self.load_factor = float(load_factor)
         self.device = torch.device(device) if device is not None else torch.device("cuda", torch.cuda.current_device())
         self._cfg = _config(config) if config else None
+        self._grouped_find = self._cfg is not None and self._cfg.find_grouped > 0
         nbytes = ght_table_bytes(self.scheme, self.capacity, self.load_factor, self._cfg)
         if nbytes == 0:
             raise GhtError(1, ght_last_error())
@@ -447,7 +451,8 @@ class HashTable:
         with _device_of(self.device):
             self._stream()
             if q.is_cuda:
-                self._ensure_find_scratch(q.numel())
+                if self._grouped_find:  # no other find needs scratch
+                    self._ensure_find_scratch(q.numel())
                 ght_find(self._t, q, out, q.numel())
             else:
                 ght_find_host(self._t, q, out, q.numel())
@@ -485,8 +490,14 @@ class HashTable:
         return (out.to(torch.int64) & 0xFFFFFFFF).view(-1, h)
 
 
+_NO_SWITCH = contextlib.nullcontext()
+
+
 def _device_of(dev):
+    """Make `dev` the current CUDA device, doing nothing where it already is."""
     import torch
+    if dev.index is None or dev.index == torch.cuda.current_device():
+        return _NO_SWITCH
     return torch.cuda.device(dev)
 
 

@@ -38,6 +38,23 @@ struct Ctrl {
 };
 static_assert(sizeof(Ctrl) == 256, "control block is 256 bytes");
 
+// Pinned host copy of a control block; the number of the copy is written last.
+struct PublishedCtrl {
+  Ctrl ctrl;
+  unsigned long long published;
+};
+
+// One warp: copy the control block to the host, then its number.
+__device__ __forceinline__ void publish_ctrl(const Ctrl *ctrl, PublishedCtrl *host, unsigned long long number,
+                                             int lane) {
+  const unsigned long long *from = reinterpret_cast<const unsigned long long *>(ctrl);
+  volatile unsigned long long *to = reinterpret_cast<volatile unsigned long long *>(&host->ctrl);
+  to[lane] = from[lane];  // 32 words
+  __threadfence_system();
+  __syncwarp();
+  if (lane == 0) *(volatile unsigned long long *)&host->published = number;
+}
+
 // Remainder by a runtime divisor d in [1, 2^32) without a divide, after
 // Lemire, Kaser and Kurz, "Faster remainder by direct computation" (Software:
 // Practice and Experience, 2019): with M = ceil(2^64 / d), x mod d is the

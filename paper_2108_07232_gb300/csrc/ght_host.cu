@@ -59,9 +59,30 @@ uint32_t derive_rng_seed(uint64_t seed, uint32_t attempt) {
   return (uint32_t)splitmix64(r) | 1u;
 }
 
-int wait_event(cudaEvent_t ev) {
+namespace {
+double wait_limit_s() {
   const char *env = getenv("GHT_WAIT_TIMEOUT_S");
-  const double limit = env && atof(env) > 0.0 ? atof(env) : 300.0;
+  return env && atof(env) > 0.0 ? atof(env) : 300.0;
+}
+}  // namespace
+
+int wait_poll(bool (*done)(const void *), const void *arg, cudaStream_t s) {
+  const double limit = wait_limit_s();
+  const auto t0 = std::chrono::steady_clock::now();
+  for (uint64_t spins = 1;; ++spins) {
+    if (done(arg)) return GHT_OK;
+    if (spins % 512 != 0) continue;
+    const cudaError_t e = cudaStreamQuery(s);
+    if (e != cudaSuccess && e != cudaErrorNotReady) return cuda_fail(e, "waiting for the device");
+    const double waited = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
+    if (waited > limit) return fail(GHT_ERR_DEVICE_TIMEOUT, "device work did not finish within %.0f s", limit);
+    if (waited > 1e-3) std::this_thread::sleep_for(std::chrono::microseconds(20));
+    else std::this_thread::yield();
+  }
+}
+
+int wait_event(cudaEvent_t ev) {
+  const double limit = wait_limit_s();
   const auto t0 = std::chrono::steady_clock::now();
   for (uint64_t spins = 0;; ++spins) {
     const cudaError_t e = cudaEventQuery(ev);

@@ -27,6 +27,14 @@ uint32_t derive_rng_seed(uint64_t seed, uint32_t attempt);
 // Wait for `ev` by polling with a deadline (GHT_WAIT_TIMEOUT_S, default 300 s).
 int wait_event(cudaEvent_t ev);
 
+// Wait until done() by polling it with the same deadline; an error of the
+// stream that is to bring it about ends the wait.
+int wait_poll(bool (*done)(const void *), const void *arg, cudaStream_t s);
+template <typename F>
+int wait_until(F done, cudaStream_t s) {
+  return wait_poll([](const void *f) { return (*static_cast<const F *>(f))(); }, &done, s);
+}
+
 // Stream-ordered allocation from the library's own pool (one per device).
 cudaError_t pool_alloc(void **p, uint64_t bytes, cudaStream_t s);
 

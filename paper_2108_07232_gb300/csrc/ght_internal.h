@@ -235,6 +235,9 @@ cudaError_t launch_block_place(int B, bool key_slots, const TableView &tv, const
                                const uint32_t *ends, uint32_t region, uint32_t bins, int fine_shift,
                                const PlaceBuffers &pb, bool count, cudaStream_t s);
 
+// Copy a control block to pinned host memory, its number last (kern_other.cu).
+cudaError_t launch_publish(const Ctrl *ctrl, PublishedCtrl *host, unsigned long long number, cudaStream_t s);
+
 // region > 0: no count pass; group g's pairs go to [g * region, ...) and
 // cursors[g] ends as the end of its pairs (counts is not written); a group
 // with more than `region` pairs sets kStatusGroupRegion in tv.ctrl.

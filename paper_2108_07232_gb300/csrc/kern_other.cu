@@ -21,6 +21,16 @@ __global__ void fill_kernel(uint4 *__restrict__ slots16, uint64_t n16, uint64_t 
   }
 }
 
+__global__ void __launch_bounds__(32)
+publish_kernel(const Ctrl *__restrict__ ctrl, PublishedCtrl *__restrict__ host, unsigned long long number) {
+  publish_ctrl(ctrl, host, number, (int)threadIdx.x);
+}
+
+cudaError_t launch_publish(const Ctrl *ctrl, PublishedCtrl *host, unsigned long long number, cudaStream_t s) {
+  publish_kernel<<<1, 32, 0, s>>>(ctrl, host, number);
+  return cudaGetLastError();
+}
+
 // Bucket indices under each hash function (diagnostic; out is n x h).
 __global__ void hash_kernel(TableView tv, const uint32_t *__restrict__ keys, uint32_t *__restrict__ out,
                             uint64_t n) {
