@@ -43,6 +43,7 @@ struct Shape {
   int find_async;    // 1: finds stage bucket parts in shared memory (BCHT b = 16, the set)
   int find_line;     // 1: the config names no find shape of its own: the line find
   int check_dups;    // 1: a successful build checks that no key is stored twice
+  int small_build;   // 1: the config names no build path or shape: tables that fit one SM are built there
   int slot_bytes;   // 8 (key/value pair) or 4 (keys-only set)
   uint32_t max_steps;  // per-key step bound of the insert kernels (0: derived)
   int find_grouped;    // 1: grouped find (rounds by bucket range), else per query
@@ -200,6 +201,9 @@ int resolve(int scheme, uint64_t capacity, double lf, const ght_config *user, Sh
   s->build_blocks_per_sm = d.build_blocks_per_sm;
   s->build_keys_per_lane = d.build_keys_per_lane;
   s->group_build = d.group_build;
+  s->small_build = d.group_build == 0 && d.ranked_build == 0 && d.build_blocks_per_sm == 0 &&
+                   !(user && user->build_tile_lanes && user->build_tile_lanes != shape0.build_tile_lanes) &&
+                   !(user && user->build_keys_per_lane && user->build_keys_per_lane != shape0.build_keys_per_lane);
   s->ranked_build = scheme == GHT_CUCKOO1 ? -1 : d.ranked_build;
   s->slot_bytes = (int)slot_bytes;
   s->find_async = async_find ? 1 : 0;
@@ -344,6 +348,7 @@ struct ght_table {
   bool last_grouped = false;
   bool last_split = false;
   bool last_ranked = false;
+  bool last_small = false;  // the last build was one launch (tev[0] to tev[3])
   mutable bool last_find_grouped = false;
   uint64_t place_overflow = 0;
   void *scratch = nullptr;  // caller-owned build scratch (ght_set_build_scratch)
@@ -500,8 +505,29 @@ bool places_ungrouped(const ght_table *t) {
   return t->shape.ranked_build > 0 || t->storage_bytes < 2ull * device_l2_bytes();
 }
 
-bool wants_ranked(const ght_table *t, uint64_t n) {
+// Whether a build of n keys runs in one block (kern_small.cu): where the table
+// fits and one SM is faster than the two phases over all of them. Whole builds,
+// us, one block / two phases: BCHT LF 0.8 1000 keys 28 / 52, 16,000 47 / 60; LF 0.95
+// 4000 keys 42 / 71, 16,000 58 / 74, 20,000 74 / 72; LF 0.99 (long chains) 4000
+// keys 72 / 92, 8000 85 / 95, 12,000 125 / 98. IHT LF 0.8 4000 keys 31 / 78, 24,000
+// 64 / 85; set LF 0.95 4000 34 / 79, 27,000 60 / 86; P2BHT LF 0.75 4000 34 / 64,
+// 20,000 60 / 63; load-balanced LF 0.9 20,000 72 / 81, 24,000 92 / 83; bucket size
+// one (its insert in place of two phases) LF 0.8 1000 51 / 65, 2000 68 / 68, 4000
+// 78 / 67.
+bool wants_small(const ght_table *t, uint64_t n) {
+  const Shape &s = t->shape;
+  if (!s.small_build || !ght::small_build_fits(s.b, s.m, n)) return false;
+  switch (s.scheme) {
+    case GHT_BCHT: return n <= (t->lf <= 0.96 ? 18432u : 8192u);
+    case GHT_CUCKOO1: return n <= 2048u;
+    case GHT_P2BHT:
+    case GHT_BCHT_LB: return n <= 20480u;
+    default: return true;
+  }
+}
 
+bool wants_ranked(const ght_table *t, uint64_t n) {
+  if (wants_small(t, n)) return false;
   const uint32_t limit = place_limit(t->shape);
   if (t->shape.ranked_build < 0 || n == 0 || n > 0xFFFFFFFFull) return false;
   if (places_by_load(t->shape)) return t->shape.group_build <= 0;  // in input order
@@ -869,6 +895,7 @@ int build_device(ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n,
                  bool host_input = false) {
   t->built = false;
   t->n_stored = 0;
+  const bool small = wants_small(t, n);
   bool ranked = wants_ranked(t, n);
   bool grouped = wants_grouping(t, n);
   if (grouped && (host_input || ((reinterpret_cast<uintptr_t>(k) | reinterpret_cast<uintptr_t>(v ? v : k)) & 15u))) {
@@ -906,6 +933,21 @@ int build_device(ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n,
     t->derive(attempt);
     const ght::TableView tv = t->view();
     cudaEventRecord(t->tev[0], t->stream);
+    if (small) {
+      cudaError_t e = ght::launch_small_build(t->shape.scheme == GHT_BCHT_SET ? (int)GHT_BCHT : t->shape.scheme,
+                                              t->shape.b, t->shape.scheme == GHT_BCHT_SET, tv, k, v, n,
+                                              place_limit(t->shape), t->shape.count_probes != 0, t->h_ctrl,
+                                              ++t->published, t->stream);
+      if (e != cudaSuccess) { rc = cuda_fail(e, "launching the one-block build"); break; }
+      cudaEventRecord(t->tev[3], t->stream);
+      t->timed_build = true;
+      t->last_small = true;
+      t->place_overflow = 0;
+      if ((rc = wait_published(t)) != GHT_OK) break;
+      if ((rc = finish_attempt(t, n, attempt, false, false, false)) != GHT_ERR_BUILD_FAILED) break;
+      continue;
+    }
+    t->last_small = false;
     // the block placement writes every table line: only the control block is reset
     cudaError_t e = g.split ? cudaMemsetAsync(t->ctrl, 0, kCtrlBytes, t->stream)
                             : ght::launch_fill(tv, t->words(), t->stream, ranked ? pb.counters : nullptr, t->shape.m);
@@ -1201,7 +1243,7 @@ int ght_build_host(ght_table *t, const uint32_t *h_keys, const uint32_t *h_value
   // inserts chunk by chunk, which a grouped build cannot (the grouping needs
   // every pair); so here grouping and ranked placement run only on request.
   const bool ranked_wanted = t->shape.ranked_build > 0 && wants_ranked(t, n);
-  if (t->shape.group_build > 0 && wants_grouping(t, n)) {
+  if ((t->shape.group_build > 0 && wants_grouping(t, n)) || wants_small(t, n)) {
     cudaEventRecord(t->tev[7], t->stream);
     if ((e = cudaMemcpyAsync(d_k, h_keys, n * 4, cudaMemcpyHostToDevice, t->stream)) != cudaSuccess ||
         (e = cudaMemcpyAsync(d_v, h_values, n * 4, cudaMemcpyHostToDevice, t->stream)) != cudaSuccess)
@@ -1273,6 +1315,7 @@ int ght_build_host(ght_table *t, const uint32_t *h_keys, const uint32_t *h_value
       }
       cudaEventRecord(t->tev[3], t->stream);
       t->timed_build = true;
+      t->last_small = false;
       t->last_grouped = false;
       t->last_split = false;
       t->last_ranked = ranked && !retry_staged;
@@ -1456,10 +1499,14 @@ int ght_stats(const ght_table *t, ght_stats_t *out) {
   out->find_staged = t->shape.find_async;
   out->find_grouped = t->shape.find_grouped;
   out->last_find_grouped = t->last_find_grouped ? 1 : 0;
-  if (t->timed_build && cudaEventQuery(t->tev[3]) == cudaSuccess) {
-    if (cudaEventElapsedTime(&ms, t->tev[0], t->tev[1]) == cudaSuccess) out->last_fill_ms = ms;
+  // (a one-block build returns when it has written the table, a moment before its end event)
+  if (t->timed_build && (t->last_small ? wait_event(t->tev[3]) == GHT_OK : cudaEventQuery(t->tev[3]) == cudaSuccess)) {
+    if (t->last_small) out->last_fill_ms = 0.0;  // part of the one-block build
+    else if (cudaEventElapsedTime(&ms, t->tev[0], t->tev[1]) == cudaSuccess) out->last_fill_ms = ms;
     // between the fill and the cuckoo insert: the grouping and/or the ranked placement
-    if (t->last_grouped && t->last_ranked) {
+    if (t->last_small) {
+      if (cudaEventElapsedTime(&ms, t->tev[0], t->tev[3]) == cudaSuccess) out->last_insert_ms = ms;
+    } else if (t->last_grouped && t->last_ranked) {
       if (t->last_split) {  // first level, then the second level's split
         if (cudaEventElapsedTime(&ms, t->tev[1], t->tev[9]) == cudaSuccess) out->last_group_ms = ms;
         if (cudaEventElapsedTime(&ms, t->tev[9], t->tev[6]) == cudaSuccess) out->last_split_ms = ms;
@@ -1471,7 +1518,7 @@ int ght_stats(const ght_table *t, ght_stats_t *out) {
       if (t->last_ranked) out->last_place_ms = ms;
       else if (t->last_grouped) out->last_group_ms = ms;
     }
-    if (cudaEventElapsedTime(&ms, t->tev[2], t->tev[3]) == cudaSuccess) out->last_insert_ms = ms;
+    if (!t->last_small && cudaEventElapsedTime(&ms, t->tev[2], t->tev[3]) == cudaSuccess) out->last_insert_ms = ms;
   }
   out->last_h2d_ms = -1.0;
   if (t->timed_h2d && cudaEventQuery(t->tev[8]) == cudaSuccess &&

@@ -235,6 +235,13 @@ cudaError_t launch_block_place(int B, bool key_slots, const TableView &tv, const
                                const uint32_t *ends, uint32_t region, uint32_t bins, int fine_shift,
                                const PlaceBuffers &pb, bool count, cudaStream_t s);
 
+// kern_small.cu: the whole build (fill, inserts, control block) of a table that
+// fits one SM's shared memory, by one block; limit: as PlaceBuffers::limit.
+bool small_build_fits(int B, uint64_t m, uint64_t n);
+cudaError_t launch_small_build(int scheme, int B, bool key_slots, const TableView &tv, const uint32_t *k,
+                               const uint32_t *v, uint64_t n, uint32_t limit, bool count, PublishedCtrl *host,
+                               unsigned long long number, cudaStream_t s);
+
 // Copy a control block to pinned host memory, its number last (kern_other.cu).
 cudaError_t launch_publish(const Ctrl *ctrl, PublishedCtrl *host, unsigned long long number, cudaStream_t s);
 

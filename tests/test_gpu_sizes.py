@@ -119,6 +119,33 @@ def test_pool_requests_of_all_sizes(G, cfg):
     pool.close()
 
 
+# the one-block build: the smallest tables, a thread's second and last key, the
+# most that a block holds, and one key more
+@pytest.mark.parametrize("n", [1, 15, 1024, 1025, 20011, 27000, 28500, 32769])
+@pytest.mark.parametrize("scheme,lf", [("bcht", 0.96), ("p2bht", 0.75), ("iht", 0.78), ("bcht_lb", 0.9),
+                                       ("cuckoo1", 0.6), ("bcht_set", 0.96)])
+def test_one_block_build(G, scheme, lf, n):
+    st = _check(G, scheme, n, lf if n > 100 else 0.4, seed=n)
+    assert st["built"] == 1 and st["n_stored"] == n
+
+
+def test_one_block_build_reports_sentinels_and_full_tables(G):
+    for scheme in ("bcht", "p2bht", "iht", "bcht_lb", "cuckoo1"):
+        keys, vals = W.make_keys(3000, 4), W.make_values(3000, 4)
+        bad = keys.clone()
+        bad[1717] = -1
+        t = G.HashTable(scheme, 3000, 0.5, seed=1)
+        with pytest.raises(G.GhtError) as e:
+            t.build(bad.cuda(), vals.cuda())
+        assert e.value.status == "GHT_ERR_SENTINEL_KEY"
+        t.build(keys.cuda(), vals.cuda())  # the same table then builds
+        assert t.stats()["built"] == 1
+    t = G.HashTable("p2bht", 20000, 1.0, seed=1, max_attempts=2)
+    with pytest.raises(G.GhtError) as e:
+        t.build(W.make_keys(20000, 1).cuda(), W.make_values(20000, 1).cuda())
+    assert e.value.status == "GHT_ERR_BUILD_FAILED" and t.stats()["built"] == 0
+
+
 # placement by load: pairs of keys per thread, odd counts; buckets of 16 and 32, evictions at 0.99
 @pytest.mark.parametrize("scheme,b,lf,n", [("p2bht", 16, 0.8, 40001), ("p2bht", 32, 0.88, 622593), ("bcht_lb", 16, 0.99, 622592),
                                            ("bcht_lb", 32, 0.99, 70003), ("p2bht", 16, 0.82, 5000011)])
