@@ -109,13 +109,17 @@ typedef struct {
    * scratch (ght_build_scratch_bytes) and 16-byte aligned key and value
    * arrays, else the build runs in input order. */
   int32_t group_build;
-  /* Two-phase build of BCHT, BCHT_SET and IHT: every key that arrives at its
+  /* Two-phase build (tables that fit one SM's shared memory are built there in
+   * one launch instead, while group_build, ranked_build and the build shape are
+   * at their defaults). BCHT, BCHT_SET and IHT: every key that arrives at its
    * first-choice bucket while it has room (IHT: while it holds fewer than
    * threshold - 1 keys) is stored at its arrival rank without reading the
    * bucket, the rest are inserted by the scheme's insert (the same table,
    * Sec. III-A and III-C, with those keys inserted first). P2BHT and BCHT_LB:
    * keys go to the least loaded candidate by the buckets' counts of arrivals
-   * (ungrouped), the rest of BCHT_LB's by its insert. 1 = on, -1 = off, 0 =
+   * (ungrouped), the rest of BCHT_LB's by its insert. CUCKOO1: the first key
+   * to reach its first choice stays there, the rest are inserted from the
+   * second. 1 = on, -1 = off, 0 =
    * default: on where it pays (IHT: while few keys are expected beyond the
    * threshold; without grouping: tables below twice the L2). Needs scratch
    * (ght_build_scratch_bytes), else the build inserts every key. */

@@ -204,7 +204,7 @@ int resolve(int scheme, uint64_t capacity, double lf, const ght_config *user, Sh
   s->small_build = d.group_build == 0 && d.ranked_build == 0 && d.build_blocks_per_sm == 0 &&
                    !(user && user->build_tile_lanes && user->build_tile_lanes != shape0.build_tile_lanes) &&
                    !(user && user->build_keys_per_lane && user->build_keys_per_lane != shape0.build_keys_per_lane);
-  s->ranked_build = scheme == GHT_CUCKOO1 ? -1 : d.ranked_build;
+  s->ranked_build = d.ranked_build;
   s->slot_bytes = (int)slot_bytes;
   s->find_async = async_find ? 1 : 0;
   s->check_dups = d.check_duplicates > 0 ? 1 : 0;
@@ -251,21 +251,21 @@ uint64_t group_scratch_bytes(uint64_t len) {
 
 // Overflow list capacity of a two-phase build of n keys: far above the ~10 %
 // of keys that overflow their first-choice bucket at load factor 1 with
-// 16-slot buckets; a larger overflow (many keys sharing a bucket) falls back
-// to the cuckoo insert of every key.
-uint64_t place_cap(uint64_t n) { return std::min<uint64_t>(n, n / 4 + 1024); }
+// 16-slot buckets (bucket size one: 37 %); a larger overflow (many keys
+// sharing a bucket) falls back to the insert of every key.
+uint64_t place_cap(uint64_t n, int b) { return std::min<uint64_t>(n, n / (b == 1 ? 2 : 4) + 1024); }
 
 uint64_t align256(uint64_t x) { return (x + 255ull) & ~255ull; }
 
-uint64_t place_scratch_bytes(uint64_t m, uint64_t n) {
-  return align256(m * sizeof(uint32_t)) + 2 * align256(place_cap(n) * sizeof(uint32_t));
+uint64_t place_scratch_bytes(uint64_t m, uint64_t n, int b) {
+  return align256(m * sizeof(uint32_t)) + 2 * align256(place_cap(n, b) * sizeof(uint32_t));
 }
 
-ght::PlaceBuffers place_buffers(char *scr, uint64_t m, uint64_t n, uint32_t limit) {
+ght::PlaceBuffers place_buffers(char *scr, uint64_t m, uint64_t n, int b, uint32_t limit) {
   ght::PlaceBuffers pb;
   pb.limit = limit;
   pb.counters = reinterpret_cast<uint32_t *>(scr);
-  pb.cap = place_cap(n);
+  pb.cap = place_cap(n, b);
   pb.ovf_k = reinterpret_cast<uint32_t *>(scr + align256(m * sizeof(uint32_t)));
   pb.ovf_v = pb.ovf_k + align256(pb.cap * sizeof(uint32_t)) / sizeof(uint32_t);
   return pb;
@@ -466,7 +466,7 @@ uint64_t device_l2_bytes() {
 // keys that find fewer than the threshold with them (Sec. III-C); 0 for the
 // schemes that place by their candidates' loads.
 uint32_t place_limit(const Shape &s) {
-  if (s.scheme == GHT_BCHT || s.scheme == GHT_BCHT_SET) return (uint32_t)s.b;
+  if (s.scheme == GHT_BCHT || s.scheme == GHT_BCHT_SET || s.scheme == GHT_CUCKOO1) return (uint32_t)s.b;
   if (s.scheme == GHT_IHT) return (uint32_t)std::min(s.b, s.t - 1);
   return 0;
 }
@@ -532,6 +532,13 @@ bool wants_ranked(const ght_table *t, uint64_t n) {
   if (t->shape.ranked_build < 0 || n == 0 || n > 0xFFFFFFFFull) return false;
   if (places_by_load(t->shape)) return t->shape.group_build <= 0;  // in input order
   if (!limit) return false;
+  // bucket size one: only grouped (below), where the placement keeps the first
+  // exchange of the 60-75 % of keys that find their slot empty from DRAM (whole
+  // builds, us: 2^24 keys LF 0.8 1272 -> 941, LF 0.6 854 -> 684, 2^25 LF 0.5 2008 ->
+  // 1292); inside the L2 it gains nothing (2^22 LF 0.8 282 / 290, 2^23 435 / 454)
+  if (t->shape.scheme == GHT_CUCKOO1 && t->shape.ranked_build <= 0 &&
+      (t->shape.group_build < 0 || t->storage_bytes < device_l2_bytes()))
+    return false;
   if (t->shape.group_build < 0 && !places_ungrouped(t)) return false;
   return t->shape.scheme != GHT_IHT || expected_overflow(n, t->shape.m, limit) <= 0.22;
 }
@@ -546,7 +553,8 @@ bool wants_ranked(const ght_table *t, uint64_t n) {
 // of 2^24 keys, 70 MB, 372 / 437); beyond it they go to DRAM (BCHT 2^24 keys,
 // 149 MB, 534 / 411).
 bool wants_grouping(const ght_table *t, uint64_t n) {
-  if (t->shape.scheme == GHT_CUCKOO1 || n == 0 || n > 0xFFFFFFFFull) return false;
+  if (n == 0 || n > 0xFFFFFFFFull) return false;
+  if (t->shape.scheme == GHT_CUCKOO1 && !wants_ranked(t, n)) return false;
   if (t->shape.group_build != 0) return t->shape.group_build > 0;
   return wants_ranked(t, n) && !places_by_load(t->shape) && t->storage_bytes >= device_l2_bytes();
 }
@@ -607,7 +615,7 @@ uint64_t sub_scratch_bytes(const GroupPlan &g) {
 }
 
 uint64_t build_scratch_need(const ght_table *t, uint64_t n) {
-  uint64_t need = wants_ranked(t, n) ? place_scratch_bytes(t->shape.m, n) : 0;
+  uint64_t need = wants_ranked(t, n) ? place_scratch_bytes(t->shape.m, n, t->shape.b) : 0;
   if (wants_grouping(t, n)) {
     const GroupPlan g = group_plan(t, n);
     need += group_scratch_bytes(g.len) + sub_scratch_bytes(g);
@@ -918,10 +926,10 @@ int build_device(ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n,
   uint32_t *gv = gk + align256(g.len * sizeof(uint32_t)) / sizeof(uint32_t);
   char *place_scr = grouped ? scr + group_scratch_bytes(g.len) : scr;
   const ght::PlaceBuffers pb =
-      ranked ? place_buffers(place_scr, t->shape.m, n, place_limit(t->shape)) : ght::PlaceBuffers();
+      ranked ? place_buffers(place_scr, t->shape.m, n, t->shape.b, place_limit(t->shape)) : ght::PlaceBuffers();
   uint32_t *sk = nullptr, *sv = nullptr, *scur = nullptr;
   if (g.split) {
-    char *p = place_scr + place_scratch_bytes(t->shape.m, n);
+    char *p = place_scr + place_scratch_bytes(t->shape.m, n, t->shape.b);
     const uint64_t arr = align256((uint64_t)g.sub.bins * g.sub.region2 * sizeof(uint32_t));
     sk = reinterpret_cast<uint32_t *>(p);
     sv = reinterpret_cast<uint32_t *>(p + arr);
@@ -1254,9 +1262,9 @@ int ght_build_host(ght_table *t, const uint32_t *h_keys, const uint32_t *h_value
     if (rc == GHT_OK) rc = build_device(t, d_k, d_v, n, 0);
   } else {
     void *place_pool = nullptr;
-    char *scr = ranked_wanted ? build_scratch(t, place_scratch_bytes(t->shape.m, n), &place_pool) : nullptr;
+    char *scr = ranked_wanted ? build_scratch(t, place_scratch_bytes(t->shape.m, n, t->shape.b), &place_pool) : nullptr;
     const bool ranked = scr != nullptr;
-    const ght::PlaceBuffers pb = ranked ? place_buffers(scr, t->shape.m, n, place_limit(t->shape)) : ght::PlaceBuffers();
+    const ght::PlaceBuffers pb = ranked ? place_buffers(scr, t->shape.m, n, t->shape.b, place_limit(t->shape)) : ght::PlaceBuffers();
     cudaStream_t copy = nullptr;
     cudaEvent_t landed[2] = {nullptr, nullptr};
     if ((e = cudaStreamCreateWithFlags(&copy, cudaStreamNonBlocking)) != cudaSuccess ||

@@ -601,7 +601,12 @@ rank_place_kernel(TableView tv, const uint32_t *__restrict__ keys, const uint32_
 template <bool COUNT>
 __global__ void __launch_bounds__(256)
 cuckoo1_insert_kernel(TableView tv, const uint32_t *__restrict__ keys,
-                      const uint32_t *__restrict__ values, uint64_t n) {
+                      const uint32_t *__restrict__ values, uint64_t n, bool overflow) {
+  if (overflow) {  // as in bucketed_insert_kernel
+    const unsigned long long listed = tv.ctrl->reserved[0];
+    if (load_status(tv.ctrl) != 0u || listed > n) return;
+    n = listed;
+  }
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   unsigned long long probes = 0, evictions = 0, longest = 0;
   const int h = tv.h;
@@ -614,7 +619,7 @@ cuckoo1_insert_kernel(TableView tv, const uint32_t *__restrict__ keys,
       continue;
     }
     uint64_t pair = ((uint64_t)__ldg(values + i) << 32) | k0;
-    uint32_t cur = bucket_of(tv.hf, 0, k0);
+    uint32_t cur = bucket_of(tv.hf, tv.first, k0);
     uint32_t displaced = 0;
     for (;;) {
       const bool at_bound = displaced >= tv.max_chain;

@@ -57,6 +57,7 @@ cudaError_t launch_place_pairs(int B, const TableView &tv, const uint32_t *k, co
   if (n == 0) return cudaSuccess;
   if (B == 16) return place_b<16>(tv, k, v, n, pb, count, s);
   if (B == 32) return place_b<32>(tv, k, v, n, pb, count, s);
+  if (B == 1) return place_b<1>(tv, k, v, n, pb, count, s);
   return cudaErrorInvalidValue;
 }
 

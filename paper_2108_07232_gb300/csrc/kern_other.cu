@@ -220,7 +220,7 @@ cudaError_t launch_insert_other(int scheme, int B, const TableView &tv, const ui
     int blocks = 0;
     cudaError_t e = grid_for(kern, n, o.blocks_per_sm, &blocks);
     if (e != cudaSuccess) return e;
-    kern<<<blocks, kThreads, 0, s>>>(tv, k, v, n);
+    kern<<<blocks, kThreads, 0, s>>>(tv, k, v, n, o.overflow);
     return cudaGetLastError();
   }
   if (!other_shape_supported(scheme, B, o.tile_lanes)) return cudaErrorInvalidValue;

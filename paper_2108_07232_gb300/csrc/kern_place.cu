@@ -30,7 +30,9 @@ namespace {
 constexpr int kBPThreads = 512;
 constexpr int kBPBatch = 8;          // pairs a thread loads before ranking them
 constexpr int kBPStage = 2048;       // overflow pairs staged per block
-constexpr uint32_t kBPImageBytes = 65536;
+// bytes of buckets per sub-group; bucket size one: half, for 4096 counters and
+// an overflow (about 1000 of 3300 pairs) that the stage holds
+__host__ __device__ constexpr uint32_t image_bytes(int B) { return B == 1 ? 32768 : 65536; }
 
 }  // namespace
 
@@ -40,9 +42,8 @@ block_place_kernel(TableView tv, const uint32_t *__restrict__ pk, const uint32_t
                    const uint32_t *__restrict__ ends, uint32_t region, uint32_t bins, int fine_shift,
                    uint32_t *__restrict__ ovf_k, uint32_t *__restrict__ ovf_v, uint64_t cap, uint32_t limit) {
   using T = typename S::T;
-  constexpr int kMaxBuckets = (int)(kBPImageBytes / (B * sizeof(T)));
-  constexpr int kVecB = (int)(B * sizeof(T) / 16);  // 16-byte vectors per bucket
-  extern __shared__ uint4 bp_img[];                 // [kBPImageBytes / 16]
+  constexpr int kMaxBuckets = (int)(image_bytes(B) / (B * sizeof(T)));
+  extern __shared__ uint4 bp_img[];                 // [image_bytes(B) / 16]
   T *img = reinterpret_cast<T *>(bp_img);
   __shared__ uint32_t bcnt[kMaxBuckets];
   __shared__ uint32_t ok[kBPStage], ov[kBPStage];
@@ -78,7 +79,8 @@ block_place_kernel(TableView tv, const uint32_t *__restrict__ pk, const uint32_t
     const uint32_t b0 = f << fine_shift;
     const uint32_t nb = min(m - b0, 1u << fine_shift);
     const uint4 e = make_uint4(kEmptyKey, kEmptyKey, kEmptyKey, kEmptyKey);
-    for (uint32_t i = tid; i < nb * kVecB; i += kBPThreads) bp_img[i] = e;
+    const uint32_t vecs = (uint32_t)((nb * (B * sizeof(T)) + 15u) / 16u);  // (B = 1: the last may be half a vector)
+    for (uint32_t i = tid; i < vecs; i += kBPThreads) bp_img[i] = e;
     for (uint32_t i = tid; i < nb; i += kBPThreads) bcnt[i] = 0u;
     __syncthreads();
     // a sub-group's cursor passes its region's end when it overflowed (the
@@ -118,7 +120,9 @@ block_place_kernel(TableView tv, const uint32_t *__restrict__ pk, const uint32_t
     }
     __syncthreads();
     uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<T *>(tv.slots) + (uint64_t)b0 * B);
-    for (uint32_t i = tid; i < nb * kVecB; i += kBPThreads) dst[i] = bp_img[i];
+    const uint32_t whole = (uint32_t)(nb * (B * sizeof(T)) / 16u);
+    for (uint32_t i = tid; i < whole; i += kBPThreads) dst[i] = bp_img[i];
+    if (whole < vecs && tid == 0) reinterpret_cast<T *>(dst)[nb - 1u] = img[nb - 1u];  // a table of odd slots
     const uint32_t staged = s_novf;
     __syncthreads();
     if (staged > (uint32_t)(kBPStage / 2)) flush(min(staged, (uint32_t)kBPStage));
@@ -135,7 +139,7 @@ block_place_kernel(TableView tv, const uint32_t *__restrict__ pk, const uint32_t
 int block_place_fine_shift(int B, bool key_slots) {
   const uint32_t bucket_bytes = (uint32_t)B * (key_slots ? 4u : 8u);
   int shift = 0;
-  while ((1u << (shift + 1)) * bucket_bytes <= kBPImageBytes) ++shift;
+  while ((1u << (shift + 1)) * bucket_bytes <= image_bytes(B)) ++shift;
   return shift;
 }
 
@@ -162,6 +166,7 @@ cudaError_t launch_block_place(int B, bool key_slots, const TableView &tv, const
     return place_blocks<KeySlot, 32>(tv, pk, pv, ends, region, bins, fine_shift, pb, count, s);
   }
   if (B == 16) return place_blocks<PairSlot, 16>(tv, pk, pv, ends, region, bins, fine_shift, pb, count, s);
+  if (B == 1) return place_blocks<PairSlot, 1>(tv, pk, pv, ends, region, bins, fine_shift, pb, count, s);
   if (B == 32) return place_blocks<PairSlot, 32>(tv, pk, pv, ends, region, bins, fine_shift, pb, count, s);
   return cudaErrorInvalidValue;
 }

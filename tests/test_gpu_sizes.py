@@ -154,6 +154,14 @@ def test_placement_by_load(G, scheme, b, lf, n):
     assert st["last_build_ranked"] == 1 and st["last_build_grouped"] == 0
 
 
+@pytest.mark.parametrize("n,lf", [(1250003, 0.8), (1250003, 0.6), ((1 << 24) + 77, 0.8)])
+def test_cuckoo1_two_phase(G, n, lf):
+    """Grouped, one block per sub-group of 4096 slots, the overflow from H_1 (the default from the
+    L2's size on, on request below it); odd slot counts."""
+    st = _check(G, "cuckoo1", n, lf, seed=n & 0xFFF, n_queries=1 << 20, group_build=1, ranked_build=1)
+    assert st["last_build_ranked"] == 1 and st["last_build_grouped"] == 1
+
+
 def test_batch_overflow_beyond_the_list_rebuilds_the_table(G):
     """Every key of one table in one bucket under its first constants: its overflow outgrows the
     batch's list, and the table is rebuilt alone."""
