@@ -965,7 +965,9 @@ int build_device(ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n,
     bool this_ranked = ranked;
     t->place_overflow = 0;
     if (grouped) {
-      e = ght::launch_group(tv, k, v ? v : k, n, g.shift, g.groups, counts, cursors, gk, gv, t->stream, g.region);
+      ght::GroupExtras x;
+      x.keys_only = g.split && t->shape.scheme == GHT_BCHT_SET;  // (the fallbacks read both arrays)
+      e = ght::launch_group(tv, k, v ? v : k, n, g.shift, g.groups, counts, cursors, gk, gv, t->stream, g.region, x);
       if (g.split) cudaEventRecord(t->tev[9], t->stream);
       if (e == cudaSuccess && g.split) {
         ght::SubSplit ss;
@@ -976,7 +978,7 @@ int build_device(ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n,
         ss.subs_log2 = g.sub.subs_log2;
         ss.groups = g.groups;
         e = ght::launch_subgroup(tv, gk, gv, (uint64_t)g.groups * g.region, ss, g.sub.bins, scur, g.sub.region2, sk, sv,
-                                 t->stream);
+                                 t->stream, x);
       }
       if (e != cudaSuccess) { rc = cuda_fail(e, "launching grouping"); break; }
       ik = gk;
@@ -989,7 +991,8 @@ int build_device(ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n,
       // the table, whose lines fill up in L2); phase 2: its overflow
       const bool set = t->shape.scheme == GHT_BCHT_SET, count = t->shape.count_probes != 0;
       if (g.split) {
-        e = ght::launch_block_place(t->shape.b, set, tv, sk, sv, scur, g.sub.region2, g.sub.bins, g.sub.fine_shift, pb,
+        // (a set's pairs have no values: the kernel's second load finds the keys in L1)
+        e = ght::launch_block_place(t->shape.b, set, tv, sk, set ? sk : sv, scur, g.sub.region2, g.sub.bins, g.sub.fine_shift, pb,
                                     count, t->stream);
       } else {
         ght::PlaceBuffers pa = pb;

@@ -207,6 +207,7 @@ struct GroupExtras {
   const unsigned long long *d_n = nullptr;
   SpillList spill;
   bool ident = false;
+  bool keys_only = false;  // a set's build: no values are read or written
   // second level of a grouped find (sub-groups of at most 256 buckets): each
   // item's bucket within its sub-group, written beside it
   uint8_t *out_b = nullptr;

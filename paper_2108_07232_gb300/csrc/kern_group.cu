@@ -143,13 +143,16 @@ size_t group_scatter_smem(uint32_t groups) {
 // group g is sub-group (g << subs_log2) + j.
 // LB (with SUB, a grouped find's second level): each item's bucket within
 // its sub-group (< 256) is written to out_b beside it.
-template <bool POS, bool SUB, bool IDENT = false, bool LB = false>
+// KEYS: keys alone are read and written (a set's build; with the keys moved as
+// values too the two levels took 260 + 262 us for 50 M keys, now 224 + 229).
+template <bool POS, bool SUB, bool IDENT = false, bool LB = false, bool KEYS = false>
 __global__ void __launch_bounds__(kGroupThreads, 2)
 group_scatter_kernel(TableView tv, const uint32_t *__restrict__ keys, const uint32_t *__restrict__ values,
                      uint64_t n, int shift, uint32_t groups, uint32_t *__restrict__ cursors,
                      uint32_t *__restrict__ out_k, uint32_t *__restrict__ out_v, uint32_t region, SubSplit sub,
                      const unsigned long long *__restrict__ d_n, SpillList spill, uint8_t *__restrict__ out_b) {
   static_assert(!LB || (SUB && !IDENT && !POS), "bucket indexes come with a second level by hash");
+  static_assert(!KEYS || (!POS && !IDENT && !LB), "keys alone are a set's build");
   if (d_n) {
     const unsigned long long dn = *d_n;
     if (dn < n) n = dn;
@@ -197,10 +200,10 @@ group_scatter_kernel(TableView tv, const uint32_t *__restrict__ keys, const uint
     const uint32_t bytes = (tn / 4u) * 16u;
     uint32_t *dk = bufs + 2 * b * kGroupTile;
     fence_proxy_async_smem();
-    mbar_arrive_expect_tx(&bars[b], (POS ? 1u : 2u) * bytes);
+    mbar_arrive_expect_tx(&bars[b], (POS || KEYS ? 1u : 2u) * bytes);
     if (bytes) {
       bulk_g2s(dk, keys + t0, bytes, &bars[b]);
-      if (!POS) bulk_g2s(dk + kGroupTile, values + t0, bytes, &bars[b]);
+      if (!POS && !KEYS) bulk_g2s(dk + kGroupTile, values + t0, bytes, &bars[b]);
     }
   };
   uint32_t j = 0;  // this block's tile count so far
@@ -237,7 +240,7 @@ group_scatter_kernel(TableView tv, const uint32_t *__restrict__ keys, const uint
       const uint32_t i = (uint32_t)u * kGroupThreads + tid;
       if (i < tn) {
         k[u] = i < tbulk ? sk[i] : __ldg(keys + t0 + i);
-        v[u] = POS ? (uint32_t)(t0 + i) : (i < tbulk ? sv[i] : __ldg(values + t0 + i));
+        v[u] = KEYS ? 0u : POS ? (uint32_t)(t0 + i) : (i < tbulk ? sv[i] : __ldg(values + t0 + i));
         // (IDENT: positions below the batch size give groups in range; the
         // clamp keeps any other key inside the tile's counters)
         uint32_t g, lb = 0u;
@@ -297,7 +300,7 @@ group_scatter_kernel(TableView tv, const uint32_t *__restrict__ keys, const uint
         const uint32_t g = LB ? (gr[u] >> 16) & 0xFFu : gr[u] >> 16;
         const uint32_t at = pre[g] + (gr[u] & 0xFFFFu);
         sk[at] = k[u];
-        sv[at] = v[u];
+        if (!KEYS) sv[at] = v[u];
         gid[at] = (uint16_t)(LB ? g | ((gr[u] >> 24) << 8) : g);
       }
     }
@@ -324,7 +327,7 @@ group_scatter_kernel(TableView tv, const uint32_t *__restrict__ keys, const uint
         continue;
       }
       out_k[at] = sk[i];
-      out_v[at] = sv[i];
+      if (!KEYS) out_v[at] = sv[i];
       if (LB) out_b[at] = (uint8_t)(gl >> 8);
     }
     __syncthreads();
@@ -385,7 +388,9 @@ cudaError_t launch_group(const TableView &tv, const uint32_t *keys, const uint32
   }
   const uint64_t tiles = (n + kGroupTile - 1) / kGroupTile;
   const size_t smem = group_scatter_smem(groups);
-  auto kern = pos ? group_scatter_kernel<true, false>
+  if (x.keys_only && (!region || pos || x.ident || x.d_n || x.spill.count)) return cudaErrorInvalidValue;
+  auto kern = x.keys_only ? group_scatter_kernel<false, false, false, false, true>
+              : pos ? group_scatter_kernel<true, false>
                   : (x.ident ? group_scatter_kernel<false, false, true> : group_scatter_kernel<false, false>);
   e = grid_for_smem(kern, kGroupThreads, smem, tiles * kGroupThreads, 0, &blocks);
   if (e != cudaSuccess) return e;
@@ -410,7 +415,9 @@ cudaError_t launch_subgroup(const TableView &tv, const uint32_t *keys, const uin
   int blocks = 0;
   if (x.d_n) return cudaErrorInvalidValue;  // the input's extent comes from sub.ends1
   if (x.out_b && (x.ident || sub.fine_shift > 8 || sub.subs_log2 > 8)) return cudaErrorInvalidValue;
-  auto kern = x.ident   ? group_scatter_kernel<false, true, true>
+  if (x.keys_only && (x.ident || x.out_b || x.spill.count)) return cudaErrorInvalidValue;
+  auto kern = x.keys_only ? group_scatter_kernel<false, true, false, false, true>
+              : x.ident ? group_scatter_kernel<false, true, true>
               : x.out_b ? group_scatter_kernel<false, true, false, true>
                         : group_scatter_kernel<false, true>;
   e = grid_for_smem(kern, kGroupThreads, smem, tiles * kGroupThreads, 0, &blocks);
