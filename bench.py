@@ -160,12 +160,15 @@ class ClockSampler:
 # at 2^28 keys. It describes the kernel source it was captured from,
 # identified by a hash of the find kernel's headers; after any change to them
 # the traffic is reported as null.
-FIND_TRAFFIC = {"bytes_per_launch": 60460572544, "source_sha256_16": "d0a797b09e952b68",
-               "kernel": "bcht_find_async_kernel"}  # --find-async 1
+FIND_TRAFFIC = {"bytes_per_launch": 60627704320, "source_sha256_16": "d06cc11ef46881cc",
+               "kernel": "line_find_kernel"}
 
 
 def build_kernels(st: dict) -> list[str]:
-    """The library kernels one build attempt launches, from the table's stats."""
+    """The library kernels one build attempt launches, from the table's stats
+    (the one-warp kernel that publishes the status to the host aside)."""
+    if st.get("last_fill_ms") == 0.0 and not st["last_build_ranked"]:  # one launch
+        return ["small_build_kernel"]
     if st["last_build_split"]:  # two grouping levels, block placement, no fill
         return ["region_cursors_kernel", "group_scatter_kernel", "region_cursors_kernel", "group_scatter_kernel",
                 "block_place_kernel", "bucketed_insert_kernel"]
@@ -365,7 +368,7 @@ def run_ours(args, world, rank, local):
             t = tables[lf]
             t.build(keys, vals)
             st = t.stats()
-            launches[0] += len(build_kernels(st)) * st["attempts"]
+            launches[0] += (len(build_kernels(st)) + 1) * st["attempts"]  # and the status
             e0 = torch.cuda.Event(enable_timing=True)
             e1 = torch.cuda.Event(enable_timing=True)
             e2 = torch.cuda.Event(enable_timing=True)
