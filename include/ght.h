@@ -119,9 +119,9 @@ typedef struct {
    * keys go to the least loaded candidate by the buckets' counts of arrivals
    * (ungrouped), the rest of BCHT_LB's by its insert. CUCKOO1: the first key
    * to reach its first choice stays there, the rest are inserted from the
-   * second. 1 = on, -1 = off, 0 =
-   * default: on where it pays (IHT: while few keys are expected beyond the
-   * threshold; without grouping: tables below twice the L2). Needs scratch
+   * second. 1 = on, -1 = off, 0 = default: on where it pays (IHT: while few
+   * keys are expected beyond the threshold; without grouping: tables below
+   * twice the L2; CUCKOO1: tables from the L2's size on). Needs scratch
    * (ght_build_scratch_bytes), else the build inserts every key. */
   int32_t ranked_build;
   /* Finds of 128-byte buckets (16 pairs: BCHT with 4-lane tiles, P2BHT, IHT
@@ -130,9 +130,10 @@ typedef struct {
    * with asynchronous copies, keys_per_lane (2..8, default 6, of which two
    * stay in registers) query sets in flight per lane, each scheme's own
    * probe order and stop rule; -1 = off
-   * (bucket parts in registers, keys_per_lane 1..2); 0 = default: on where
-   * it applies, the table's slots take at least the device's L2 size and
-   * neither keys_per_lane 1 nor (except for BCHT's 4) tile_lanes is given.
+   * (bucket parts in registers, keys_per_lane 1..2); 0 = default: the line
+   * find, or for other shapes than it serves the staged find where that
+   * applies, the table's slots take at least the device's L2 size and neither
+   * keys_per_lane 1 nor (except for BCHT's 4) tile_lanes is given.
    * Other shapes (32-pair buckets, CUCKOO1) reject 1. */
   int32_t find_async;
   /* 1: after a successful ght_build / ght_build_host, check that no input key
@@ -259,8 +260,8 @@ int ght_find(const ght_table *t, const uint32_t *d_queries, uint32_t *d_out, uin
  * from page-locked keys and values (allocated or registered with the CUDA
  * runtime) that requests neither grouping nor the two-phase build
  * (group_build and ranked_build <= 0) copies nothing: its placement or insert
- * reads them in place, ungrouped (last_h2d_ms -1); they
- * must stay unchanged until the call returns. If the bounded wait for the
+ * reads them in place, ungrouped (last_h2d_ms -1); they must stay unchanged
+ * until the call returns. If the bounded wait for the
  * device runs out (GHT_ERR_DEVICE_TIMEOUT, see GHT_WAIT_TIMEOUT_S), copies
  * or kernels already queued may still read h_keys/h_values or write h_out
  * afterwards. */

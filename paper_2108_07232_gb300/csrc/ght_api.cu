@@ -1,8 +1,8 @@
 // ght_api.cu -- host side of the C ABI declared in include/ght.h.
 //
 // Sizing, constant derivation, the build retry loop and the host<->device
-// pipelines live here; all table arithmetic on keys runs in the kernels of
-// kern_bcht.cu / kern_other.cu.
+// pipelines live here; all table arithmetic on keys runs in the kernels of the
+// kern_*.cu files.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -52,8 +52,8 @@ struct Shape {
 
 // Launch shapes measured fastest on GB300 at 2^27-2^28 keys (insert with
 // chunk claims; load factors near each scheme's working range).
-// Finds read 16-pair buckets fastest with two queries in flight per lane
-// and 32-pair buckets with one; builds the other way round, except the
+// The register find reads 16-pair buckets fastest with two queries in flight
+// per lane and 32-pair buckets with one; builds the other way round, except the
 // keys-only set, fastest with one key per lane for both. BCHT reads a
 // 16-pair bucket with 4 lanes in its finds and 16 in its inserts; every
 // other bucketed kernel uses 8.
@@ -160,9 +160,10 @@ int resolve(int scheme, uint64_t capacity, double lf, const ght_config *user, Sh
   double want = std::ceil((double)capacity / (lf * (double)b));
   if (want < 1.0) want = 1.0;
   if (want > 4294967295.0) return fail(GHT_ERR_INVALID_ARG, "table needs more than 2^32-1 buckets");
-  // The staged find by default where it applies and the slots do not fit in
-  // the L2: there its deeper pipeline hides DRAM latency; on an L2-resident
-  // table the register find's higher occupancy wins. A given keys_per_lane of
+  // What find_async = 0 resolves to where the line find does not answer (32-pair
+  // buckets, named shapes): the staged find where it applies and the slots do
+  // not fit in the L2 -- there its deeper pipeline hides DRAM latency, inside
+  // the L2 the register find's higher occupancy wins. A given keys_per_lane of
   // 1 keeps the register find. 6 query sets in flight (3 for 256-byte
   // buckets) unless keys_per_lane is given.
   const uint64_t slot_bytes = scheme == GHT_BCHT_SET ? 4 : 8;
