@@ -199,6 +199,13 @@ bucketed_insert_kernel(TableView tv, const uint32_t *__restrict__ keys,
   }
   const ClaimPlan plan = claim_plan(n, (uint64_t)gridDim.x * (blockDim.x >> 5), ordered);
   static_assert(B % G == 0 && 32 % G == 0 && PPL >= 1 && (KPL == 1 || KPL == 2), "tile shape");
+  // Members j that have a key in no tile are passed over, except in BCHT: the
+  // inserts of P2BHT, IHT and the load-balanced BCHT get shorter (overflow of
+  // IHT at LF 0.8, 2^20 keys 53 -> 43 us, 2^24 223 -> 171), BCHT's with its 16
+  // members longer (overflow at LF 0.95, 2^24 keys 170 -> 185 us, every key 664 ->
+  // 787; set of 50 M keys 311 -> 324). kMembers: lane 0 of every tile.
+  constexpr bool kSkip = SCHEME != kBCHT;
+  constexpr unsigned kMembers = G == 4 ? 0x11111111u : G == 8 ? 0x01010101u : G == 16 ? 0x00010001u : 1u;
   const int lane = threadIdx.x & 31;
   const int r = lane & (G - 1);
   const int tbase = lane - r;
@@ -319,6 +326,7 @@ bucketed_insert_kernel(TableView tv, const uint32_t *__restrict__ keys,
       uint32_t v[G][PPL];
 #pragma unroll
       for (int j = 0; j < G; ++j) {
+        if (kSkip && (act & (kMembers << j)) == 0u) continue;  // warp-uniform
         const uint32_t bj = __shfl_sync(kFull, cur[s], tbase + j);
         if ((act >> (tbase + j)) & 1u) load_keys_rw<PPL>(slots + (uint64_t)bj * B, r, v[j]);
       }
@@ -326,6 +334,7 @@ bucketed_insert_kernel(TableView tv, const uint32_t *__restrict__ keys,
       int my_empty = 0, my_slot = -1;
 #pragma unroll
       for (int j = 0; j < G; ++j) {
+        if (kSkip && (act & (kMembers << j)) == 0u) continue;
         const bool aj = (act >> (tbase + j)) & 1u;
         int cnt = 0, slot = -1;
 #pragma unroll
