@@ -494,9 +494,9 @@ double expected_overflow(uint64_t n, uint64_t m, uint32_t limit) {
 // off, 0 always where it applies). It costs no bucket read for the keys that
 // find room at once, so it won at every size measured (whole builds, us,
 // input order -> two phases, BCHT at LF 0.9): 2^14 keys 94 -> 81, 2^17 97 ->
-// 85, 2^20 126 -> 105, 2^22 259 -> 154, 2^24 657 -> 411; IHT at LF 0.8: 2^17
-// 120 -> 94, 2^20 181 -> 125, 2^24 1157 -> 550; set at LF 0.95: 2^17 169 ->
-// 100, 50 M keys 2920 -> 1115. IHT's overflow, the keys beyond its threshold,
+// 85, 2^20 126 -> 105, 2^22 259 -> 154, 2^24 657 -> 411; IHT at LF 0.8: 2^16
+// 110 -> 72, 2^20 181 -> 96, 2^24 1157 -> 487; set at LF 0.95: 2^17 169 ->
+// 100, 50 M keys 2920 -> 968. IHT's overflow, the keys beyond its threshold,
 // has to fit the overflow list: above 0.22 of the keys it builds in input
 // order (low thresholds, or load factors where it rarely succeeds).
 // Ungrouped, the placement's stores and counters go to DRAM one sector each on
