@@ -332,9 +332,16 @@ int ght_partition(const uint32_t *d_keys, const uint32_t *d_values, uint64_t n, 
  * asynchronous on cuda_stream. */
 int ght_unpermute(const uint32_t *d_src, const uint32_t *d_pos, uint64_t n, uint32_t *d_dst, void *cuda_stream);
 
-/* Device scratch a build of n keys uses for grouping (0 if this table
- * builds without grouping). */
+/* Device scratch that a ght_build of n keys uses at most, for its grouping
+ * and its ranked placement (0 if this table builds without either): with
+ * 16-byte aligned arrays. */
 uint64_t ght_build_scratch_bytes(const ght_table *t, uint64_t n);
+
+/* The same for these arrays: what ght_build of them uses (host 0), or
+ * ght_build_host (host 1). Unaligned arrays and page-locked ones read in
+ * place build ungrouped and use far less; pageable ones use none by default. */
+uint64_t ght_build_scratch_bytes_for(const ght_table *t, const uint32_t *keys, const uint32_t *values, uint64_t n,
+                                     int host);
 
 /* Device scratch a ght_find of n device queries uses when it runs grouped
  * (config find_grouped): about 45 bytes per query; 0 if such a find runs per
@@ -345,7 +352,9 @@ uint64_t ght_find_scratch_bytes(const ght_table *t, uint64_t n);
  * by the caller) for later builds and grouped finds; NULL clears it. Without
  * it (or where it is smaller than the call needs), a table whose storage the
  * library owns takes scratch from the library's stream-ordered pool, and a
- * table on caller storage builds ungrouped and finds per query. Calls that
+ * table on caller storage builds with what fits (the placement without the
+ * grouping, on tables below twice the L2 or with ranked_build 1; else the
+ * insert of every key) and finds per query. Calls that
  * use this buffer must not overlap on the device (they share it). */
 int ght_set_build_scratch(ght_table *t, void *d_scratch, uint64_t bytes);
 

@@ -148,6 +148,7 @@ def lib():
                 "ght_find_host_noalloc": ([vp, vp, vp, u64], i32),
                 "ght_stats": ([vp, C.POINTER(GhtStats)], i32),
                 "ght_build_scratch_bytes": ([vp, u64], u64),
+                "ght_build_scratch_bytes_for": ([vp, vp, vp, u64, i32], u64),
                 "ght_find_scratch_bytes": ([vp, u64], u64),
                 "ght_set_build_scratch": ([vp, vp, u64], i32),
                 "ght_reset_counters": ([vp], i32),
@@ -284,6 +285,10 @@ def ght_build_scratch_bytes(t: int, n: int) -> int:
     return int(lib().ght_build_scratch_bytes(t, n))
 
 
+def ght_build_scratch_bytes_for(t: int, keys, values, n: int, host: bool) -> int:
+    return int(lib().ght_build_scratch_bytes_for(t, _ptr(keys), _ptr(values), n, 1 if host else 0))
+
+
 def ght_find_scratch_bytes(t: int, n: int) -> int:
     return int(lib().ght_find_scratch_bytes(t, n))
 
@@ -413,15 +418,15 @@ class HashTable:
                 raise ValueError("keys and values differ in length")
         with _device_of(self.device):
             self._stream()
-            self._ensure_scratch(k.numel())
+            self._ensure_scratch(ght_build_scratch_bytes_for(self._t, k, v, k.numel(), not k.is_cuda))
             if k.is_cuda:
                 ght_build(self._t, k, v, k.numel())
             else:
                 ght_build_host(self._t, k, v, k.numel())
 
-    def _ensure_scratch(self, n: int) -> None:
+    def _ensure_scratch(self, need: int) -> None:
         """Two-phase and grouped builds need scratch; it is a torch tensor kept with the table."""
-        self._ensure_bytes(ght_build_scratch_bytes(self._t, n))
+        self._ensure_bytes(need)
 
     def _ensure_find_scratch(self, n: int) -> None:
         """A grouped find (find_grouped = 1) needs scratch too: the same buffer, grown."""

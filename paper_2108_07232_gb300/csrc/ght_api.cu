@@ -596,12 +596,12 @@ struct GroupPlan {
   SubShape sub;
 };
 
-GroupPlan group_plan(const ght_table *t, uint64_t n) {
+GroupPlan group_plan(const ght_table *t, uint64_t n, bool ranked) {
   GroupPlan g;
   const uint64_t m = t->shape.m;
   group_shape(m, &g.shift, &g.groups);
   g.len = n;
-  if (!wants_ranked(t, n)) return g;
+  if (!ranked) return g;
   g.region = group_region(n, g.groups);
   g.split = g.region && sub_shape(t->shape, n, g.shift, g.region, &g.sub);
   if (g.region) g.len = (uint64_t)g.groups * g.region;
@@ -615,10 +615,28 @@ uint64_t sub_scratch_bytes(const GroupPlan &g) {
   return 2 * align256((uint64_t)g.sub.bins * g.sub.region2 * sizeof(uint32_t)) + align256(g.sub.bins * sizeof(uint32_t));
 }
 
-uint64_t build_scratch_need(const ght_table *t, uint64_t n) {
-  uint64_t need = wants_ranked(t, n) ? place_scratch_bytes(t->shape.m, n, t->shape.b) : 0;
-  if (wants_grouping(t, n)) {
-    const GroupPlan g = group_plan(t, n);
+// How a build from these arrays runs, scratch aside. The grouping makes bulk
+// copies of 16-byte pieces of device memory: input that is not 16-byte aligned,
+// or in host memory (host_input), builds ungrouped.
+struct BuildPath {
+  bool grouped = false, ranked = false;
+};
+
+BuildPath build_path(const ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n, bool host_input) {
+  BuildPath p;
+  p.ranked = wants_ranked(t, n);
+  p.grouped = wants_grouping(t, n);
+  if (p.grouped && (host_input || ((reinterpret_cast<uintptr_t>(k) | reinterpret_cast<uintptr_t>(v ? v : k)) & 15u))) {
+    p.grouped = false;
+    p.ranked = p.ranked && places_ungrouped(t);
+  }
+  return p;
+}
+
+uint64_t build_scratch_need(const ght_table *t, uint64_t n, const BuildPath &p) {
+  uint64_t need = p.ranked ? place_scratch_bytes(t->shape.m, n, t->shape.b) : 0;
+  if (p.grouped) {
+    const GroupPlan g = group_plan(t, n, p.ranked);
     need += group_scratch_bytes(g.len) + sub_scratch_bytes(g);
   }
   return need;
@@ -874,6 +892,12 @@ bool device_view(const void *h, const void **d) {
   return true;
 }
 
+// Whether ght_build_host reads these arrays where they are, and their device addresses.
+bool reads_in_place(const ght_table *t, const uint32_t *h_keys, const uint32_t *h_values, const void **dk,
+                    const void **dv) {
+  return t->shape.group_build <= 0 && t->shape.ranked_build <= 0 && device_view(h_keys, dk) && device_view(h_values, dv);
+}
+
 // Take over an attempt's control block (just read): GHT_OK if it built the
 // table, GHT_ERR_BUILD_FAILED if another attempt may.
 int finish_attempt(ght_table *t, uint64_t n, uint32_t attempt, bool grouped, bool split, bool ranked) {
@@ -905,21 +929,20 @@ int build_device(ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n,
   t->built = false;
   t->n_stored = 0;
   const bool small = wants_small(t, n);
-  bool ranked = wants_ranked(t, n);
-  bool grouped = wants_grouping(t, n);
-  if (grouped && (host_input || ((reinterpret_cast<uintptr_t>(k) | reinterpret_cast<uintptr_t>(v ? v : k)) & 15u))) {
-    // the grouping makes bulk copies of 16-byte pieces of device memory: other input builds ungrouped
-    grouped = false;
-    ranked = ranked && places_ungrouped(t);
-  }
+  BuildPath path = build_path(t, k, v, n, host_input);
   void *pool_buf = nullptr;
   char *scr = nullptr;
-  if (ranked || grouped) {
-    scr = build_scratch(t, build_scratch_need(t, n), &pool_buf);
-    if (!scr) ranked = grouped = false;  // no scratch: the cuckoo insert of every key in input order
+  if (path.grouped || path.ranked) {
+    scr = build_scratch(t, build_scratch_need(t, n, path), &pool_buf);
+    if (!scr && path.grouped && path.ranked && places_ungrouped(t)) {  // the placement alone takes much less
+      path.grouped = false;
+      scr = build_scratch(t, build_scratch_need(t, n, path), &pool_buf);
+    }
+    if (!scr) path = BuildPath();  // no scratch: the insert of every key in input order
   }
+  const bool grouped = path.grouped, ranked = path.ranked;
   GroupPlan g;
-  if (grouped) g = group_plan(t, n);
+  if (grouped) g = group_plan(t, n, ranked);
   // scratch layout: [grouping: counts, cursors, keys, values][ranked placement][sub-group keys, values, cursors]
   uint32_t *counts = reinterpret_cast<uint32_t *>(scr);
   uint32_t *cursors = counts + ght::kMaxGroups;
@@ -1230,8 +1253,7 @@ int ght_build_host(ght_table *t, const uint32_t *h_keys, const uint32_t *h_value
   // pipeline -- its first chunk's wait and one insert launch tail per chunk --
   // goes away). A requested grouped or two-phase build still stages the pairs.
   const void *dk_in = nullptr, *dv_in = nullptr;
-  if (t->shape.group_build <= 0 && t->shape.ranked_build <= 0 && device_view(h_keys, &dk_in) &&
-      device_view(h_values, &dv_in)) {
+  if (reads_in_place(t, h_keys, h_values, &dk_in, &dv_in)) {
     t->timed_h2d = false;  // no copies: the insert's own loads cross the host link
     int rc = build_device(t, static_cast<const uint32_t *>(dk_in), static_cast<const uint32_t *>(dv_in), n, 0, true);
     if (rc == GHT_OK) rc = check_duplicates(t, static_cast<const uint32_t *>(dk_in), n);
@@ -1450,7 +1472,25 @@ uint64_t ght_build_scratch_bytes(const ght_table *t, uint64_t n) {
     fail(GHT_ERR_INVALID_ARG, "table is NULL");
     return 0;
   }
-  return build_scratch_need(t, n);
+  return build_scratch_need(t, n, build_path(t, nullptr, nullptr, n, false));
+}
+
+uint64_t ght_build_scratch_bytes_for(const ght_table *t, const uint32_t *keys, const uint32_t *values, uint64_t n,
+                                     int host) {
+  if (!t) {
+    fail(GHT_ERR_INVALID_ARG, "table is NULL");
+    return 0;
+  }
+  if (!host) return build_scratch_need(t, n, build_path(t, keys, values, n, false));
+  const void *dk = nullptr, *dv = nullptr;
+  if (reads_in_place(t, keys, values ? values : keys, &dk, &dv))
+    return build_scratch_need(t, n, build_path(t, nullptr, nullptr, n, true));
+  // staged: grouped builds from the staged copy, two-phase ones chunk by chunk
+  if (t->shape.group_build > 0 && wants_grouping(t, n))
+    return build_scratch_need(t, n, build_path(t, nullptr, nullptr, n, false));
+  BuildPath p;
+  p.ranked = t->shape.ranked_build > 0 && wants_ranked(t, n);
+  return build_scratch_need(t, n, p);
 }
 
 uint64_t ght_find_scratch_bytes(const ght_table *t, uint64_t n) {
