@@ -243,11 +243,11 @@ uint32_t group_region(uint64_t n, uint32_t groups) {
 }
 
 // Scratch of a grouped build: counts and cursors, then the regrouped keys and
-// values (`len` entries each).
-uint64_t group_scratch_bytes(uint64_t len) {
+// values (`len` entries each; keys_only: no values).
+uint64_t group_scratch_bytes(uint64_t len, bool keys_only) {
   const uint64_t head = 2ull * ght::kMaxGroups * sizeof(uint32_t);
   const uint64_t arr = (len * sizeof(uint32_t) + 255ull) & ~255ull;
-  return head + 2 * arr;
+  return head + (keys_only ? 1 : 2) * arr;
 }
 
 // Overflow list capacity of a two-phase build of n keys: far above the ~10 %
@@ -587,12 +587,14 @@ bool sub_shape(const Shape &s, uint64_t n, int shift, uint32_t region1, SubShape
 // Grouping of a build of n keys: groups of 2^shift first-choice buckets, each
 // in a region of `region` pairs when the build places by rank (0: exact
 // offsets, `len` = n entries); split: the groups are split into sub-groups,
-// which are placed by one block each in shared memory.
+// which are placed by one block each in shared memory; keys_only: a set's
+// split, whose two levels move no values (50 M keys: 521 MB of scratch with
+// the placement's, 943 with value arrays).
 struct GroupPlan {
   int shift = 0;
   uint32_t groups = 1, region = 0;
   uint64_t len = 0;
-  bool split = false;
+  bool split = false, keys_only = false;
   SubShape sub;
 };
 
@@ -604,6 +606,7 @@ GroupPlan group_plan(const ght_table *t, uint64_t n, bool ranked) {
   if (!ranked) return g;
   g.region = group_region(n, g.groups);
   g.split = g.region && sub_shape(t->shape, n, g.shift, g.region, &g.sub);
+  g.keys_only = g.split && t->shape.scheme == GHT_BCHT_SET;
   if (g.region) g.len = (uint64_t)g.groups * g.region;
   return g;
 }
@@ -612,7 +615,8 @@ GroupPlan group_plan(const ght_table *t, uint64_t n, bool ranked) {
 // sub-group (0 where the build does not use it).
 uint64_t sub_scratch_bytes(const GroupPlan &g) {
   if (!g.split) return 0;
-  return 2 * align256((uint64_t)g.sub.bins * g.sub.region2 * sizeof(uint32_t)) + align256(g.sub.bins * sizeof(uint32_t));
+  return (g.keys_only ? 1 : 2) * align256((uint64_t)g.sub.bins * g.sub.region2 * sizeof(uint32_t)) +
+         align256(g.sub.bins * sizeof(uint32_t));
 }
 
 // How a build from these arrays runs, scratch aside. The grouping makes bulk
@@ -637,7 +641,7 @@ uint64_t build_scratch_need(const ght_table *t, uint64_t n, const BuildPath &p) 
   uint64_t need = p.ranked ? place_scratch_bytes(t->shape.m, n, t->shape.b) : 0;
   if (p.grouped) {
     const GroupPlan g = group_plan(t, n, p.ranked);
-    need += group_scratch_bytes(g.len) + sub_scratch_bytes(g);
+    need += group_scratch_bytes(g.len, g.keys_only) + sub_scratch_bytes(g);
   }
   return need;
 }
@@ -943,12 +947,13 @@ int build_device(ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n,
   const bool grouped = path.grouped, ranked = path.ranked;
   GroupPlan g;
   if (grouped) g = group_plan(t, n, ranked);
-  // scratch layout: [grouping: counts, cursors, keys, values][ranked placement][sub-group keys, values, cursors]
+  // scratch layout: [grouping: counts, cursors, keys, values][ranked placement][sub-group keys, values, cursors],
+  // a set's split without the values
   uint32_t *counts = reinterpret_cast<uint32_t *>(scr);
   uint32_t *cursors = counts + ght::kMaxGroups;
   uint32_t *gk = reinterpret_cast<uint32_t *>(scr + 2ull * ght::kMaxGroups * sizeof(uint32_t));
   uint32_t *gv = gk + align256(g.len * sizeof(uint32_t)) / sizeof(uint32_t);
-  char *place_scr = grouped ? scr + group_scratch_bytes(g.len) : scr;
+  char *place_scr = grouped ? scr + group_scratch_bytes(g.len, g.keys_only) : scr;
   const ght::PlaceBuffers pb =
       ranked ? place_buffers(place_scr, t->shape.m, n, t->shape.b, place_limit(t->shape)) : ght::PlaceBuffers();
   uint32_t *sk = nullptr, *sv = nullptr, *scur = nullptr;
@@ -956,8 +961,11 @@ int build_device(ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n,
     char *p = place_scr + place_scratch_bytes(t->shape.m, n, t->shape.b);
     const uint64_t arr = align256((uint64_t)g.sub.bins * g.sub.region2 * sizeof(uint32_t));
     sk = reinterpret_cast<uint32_t *>(p);
-    sv = reinterpret_cast<uint32_t *>(p + arr);
-    scur = reinterpret_cast<uint32_t *>(p + 2 * arr);
+    sv = g.keys_only ? sk : reinterpret_cast<uint32_t *>(p + arr);
+    scur = reinterpret_cast<uint32_t *>(p + (g.keys_only ? 1 : 2) * arr);
+    // An attempt regrouped with exact offsets does not split: its n values go
+    // where the split's keys were (bins regions of at least n / bins each).
+    if (g.keys_only) gv = sk;
   }
   int rc = fail(GHT_ERR_BUILD_FAILED, "build failed in %u attempts (chain bound or full buckets)",
                 t->shape.max_attempts);
@@ -990,7 +998,7 @@ int build_device(ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n,
     t->place_overflow = 0;
     if (grouped) {
       ght::GroupExtras x;
-      x.keys_only = g.split && t->shape.scheme == GHT_BCHT_SET;  // (the fallbacks read both arrays)
+      x.keys_only = g.split && g.keys_only;  // (the fallback reads both arrays)
       e = ght::launch_group(tv, k, v ? v : k, n, g.shift, g.groups, counts, cursors, gk, gv, t->stream, g.region, x);
       if (g.split) cudaEventRecord(t->tev[9], t->stream);
       if (e == cudaSuccess && g.split) {

@@ -1,6 +1,7 @@
 """Device memory that builds take beside the table: the scratch fits the path a
 build runs, and a build without enough of it still succeeds."""
 
+import numpy as np
 import pytest
 import torch
 
@@ -77,3 +78,40 @@ def test_scratch_of_the_placement_alone_is_used(G, offset):
     finally:
         torch.cuda.synchronize()
         G.ght_destroy(h)
+
+
+def test_a_set_takes_no_scratch_for_values(G):
+    """A keys-only build moves keys alone: the grouped arrays hold no values (two levels of about
+    4 bytes a key, the placement's counters and list; values would add as much again as the levels)."""
+    n = 50_000_000
+    t = G.HashTable("bcht_set", n, 0.95, seed=1)
+    m = t.stats()["num_buckets"]
+    assert G.ght_build_scratch_bytes(t._t, n) < _placement_bytes(n, m) + 2 * 1.1 * 4 * n
+
+
+def test_a_set_whose_sub_group_outgrows_its_region(G):
+    """1300 keys more than average in one 512-bucket sub-group of a set: the attempt is redone with
+    exact offsets, which read and write values, in the scratch of a build without them."""
+    n, lf, seed = 1 << 22, 0.99, 43
+    m = O.num_buckets(n, lf, 32)
+    a, c = O.derive_constants(seed, 0, 3)
+    cand = np.arange(1, 1 << 24, dtype=np.uint64)
+    h0 = ((np.uint64(a[0]) * cand + np.uint64(c[0])) % np.uint64(O.PRIME)) % np.uint64(m)
+    crowd = cand[h0 < 512][:1300].astype(np.uint32)
+    rest = W.make_keys(n + 4096, 102).numpy().view(np.uint32)
+    rest = rest[~np.isin(rest, crowd)][: n - crowd.size]
+    keys = torch.from_numpy(np.concatenate([rest, crowd]).view(np.int32).copy())
+    t = G.HashTable("bcht_set", n, lf, seed=seed, group_build=1)
+    for values in (None, W.make_values(n, 3).cuda()):  # a set ignores values
+        t.build(keys.cuda(), values)
+        st = t.stats()
+        assert (st["attempts"], st["last_build_grouped"], st["last_build_split"]) == (1, 1, 0)
+        q = W.make_queries(keys, 1 << 20, 0.5, seed=9)
+        want = O.lookup(keys, keys, q) != O.EMPTY
+        assert (O._u32(t.find(q.cuda()).cpu()) == want.astype(np.uint32)).all()
+    T = O.Table(O.BCHT, n, lf, b=32, m=m)
+    T.set_constants(st["hash_a"], st["hash_c"])
+    raw = t.export()
+    zeros = torch.zeros(n, dtype=torch.int32)
+    ok, msg = T.validate(keys, zeros, slots=np.where(raw == O.EMPTY, np.uint64(O.EMPTY_PAIR), raw.astype(np.uint64)))
+    assert ok, msg
