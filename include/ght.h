@@ -490,7 +490,9 @@ void ght_batch_destroy(ght_batch *b);
  * arrive while others run join the next launch. A build worker admits build
  * requests in arrival order once the table fits in the budget (storage from
  * the library's stream-ordered pool) and builds on its own stream, overlapping
- * the finds. Each answer is exactly what a single-table find returns.
+ * the finds; scratch for the build comes out of what the budget has left then
+ * (used_bytes counts it until the build is done; without room for it every key
+ * is inserted, with the same table). Each answer is exactly what a single-table find returns.
  * Device arrays passed to submit calls must stay valid until the request
  * completes.
  * ------------------------------------------------------------------------- */

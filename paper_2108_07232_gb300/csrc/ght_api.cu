@@ -637,6 +637,14 @@ BuildPath build_path(const ght_table *t, const uint32_t *k, const uint32_t *v, u
   return p;
 }
 
+// What runs where p's scratch is not to be had: the placement without the
+// grouping, which takes much less, else the insert of every key in input order.
+BuildPath smaller_path(const ght_table *t, const BuildPath &p) {
+  BuildPath q;
+  q.ranked = p.grouped && p.ranked && places_ungrouped(t);
+  return q;
+}
+
 uint64_t build_scratch_need(const ght_table *t, uint64_t n, const BuildPath &p) {
   uint64_t need = p.ranked ? place_scratch_bytes(t->shape.m, n, t->shape.b) : 0;
   if (p.grouped) {
@@ -936,13 +944,9 @@ int build_device(ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n,
   BuildPath path = build_path(t, k, v, n, host_input);
   void *pool_buf = nullptr;
   char *scr = nullptr;
-  if (path.grouped || path.ranked) {
+  while (!scr && (path.grouped || path.ranked)) {
     scr = build_scratch(t, build_scratch_need(t, n, path), &pool_buf);
-    if (!scr && path.grouped && path.ranked && places_ungrouped(t)) {  // the placement alone takes much less
-      path.grouped = false;
-      scr = build_scratch(t, build_scratch_need(t, n, path), &pool_buf);
-    }
-    if (!scr) path = BuildPath();  // no scratch: the insert of every key in input order
+    if (!scr) path = smaller_path(t, path);
   }
   const bool grouped = path.grouped, ranked = path.ranked;
   GroupPlan g;
@@ -1135,6 +1139,14 @@ bool ght::table_descriptor(const ght_table *t, ght::BatchTable *out) {
     out->c[i] = t->c[i];
   }
   return true;
+}
+
+uint64_t ght::build_scratch_within(const ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n,
+                                   uint64_t most) {
+  BuildPath p = build_path(t, k, v, n, false);
+  uint64_t need;
+  while ((need = build_scratch_need(t, n, p)) > most) p = smaller_path(t, p);
+  return need;
 }
 
 extern "C" {

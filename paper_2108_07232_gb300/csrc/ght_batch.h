@@ -48,6 +48,9 @@ bool batch_find_shape_supported(int tile_lanes, int keys_per_lane);
 // Describe a built single BCHT table (b = 16) as a batch descriptor (ght_api.cu).
 // Returns false if the table is not a built 16-pair BCHT table.
 bool table_descriptor(const struct ::ght_table *t, BatchTable *out);
+// Scratch of the fastest build of these device arrays that takes at most `most` bytes (ght_api.cu).
+uint64_t build_scratch_within(const struct ::ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n,
+                              uint64_t most);
 
 // Copy n items from per-segment sources into one array and back
 // (kern_batch.cu): dst[i] = src[s][i - offs[s]] for offs[s] <= i < offs[s+1].

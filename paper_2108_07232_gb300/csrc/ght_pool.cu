@@ -11,8 +11,9 @@
 //     of the queries before it, a scatter after it). Requests that arrive
 //     while launches run join the next launch (continuous batching).
 //   * the build worker admits build requests in arrival order when the table
-//     fits in the HBM budget, allocates its storage from the library pool and
-//     builds it on its own stream, so builds overlap finds on the device.
+//     fits in the HBM budget, allocates its storage and, within what the budget
+//     has left, the build's scratch from the library pool and builds it on its
+//     own stream, so builds overlap finds on the device.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -336,9 +337,14 @@ void ght_pool::build_loop() {
       if (!t) rc = GHT_ERR_INVALID_ARG;
     }
     if (rc == GHT_OK) rc = ght_set_stream(t, build_stream);
-    // scratch of a two-phase build, for this build only (without it the build inserts every key)
+    // scratch of a two-phase build, for this build only and from what the budget has left
     void *scratch = nullptr;
-    const uint64_t need = rc == GHT_OK ? ght_build_scratch_bytes(t, r.n) : 0;
+    uint64_t need = 0;
+    if (rc == GHT_OK) {
+      std::lock_guard<std::mutex> lock(mu);
+      need = ght::build_scratch_within(t, r.values ? r.in : nullptr, r.values, r.n, budget - used);
+      used += need;
+    }
     if (need && ght::host::pool_alloc(&scratch, need, build_stream) != cudaSuccess) {
       cudaGetLastError();
       scratch = nullptr;
@@ -350,6 +356,7 @@ void ght_pool::build_loop() {
       cudaFreeAsync(scratch, build_stream);
     }
     std::lock_guard<std::mutex> lock(mu);
+    used -= need;
     pt.t = t;
     pt.storage = storage;
     if (rc == GHT_OK && ght::table_descriptor(t, &pt.desc)) {
