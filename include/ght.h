@@ -485,9 +485,11 @@ void ght_batch_destroy(ght_batch *b);
  *
  * Continuous batching: a scheduler thread keeps up to two batched find
  * launches in flight; each new launch takes every pending find whose table is
- * built (oldest first, at most 2^22 queries and 4096 requests), gathers their
- * queries, finds them in one launch and scatters the answers, so requests that
- * arrive while others run join the next launch. A build worker admits build
+ * built (oldest first, at most 2^22 queries and 4096 requests) and finds them
+ * in one launch, so requests that arrive while others run join the next launch.
+ * Answers may be written over queries of the same request, in place or at an
+ * offset, and of others in the launch: such a launch gathers all its queries
+ * before its find and scatters the answers after it. A build worker admits build
  * requests in arrival order once the table fits in the budget (storage from
  * the library's stream-ordered pool) and builds on its own stream, overlapping
  * the finds; scratch for the build comes out of what the budget has left then

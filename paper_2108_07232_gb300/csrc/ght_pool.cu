@@ -7,8 +7,9 @@
 //     one completes it packs every pending find request whose table is ready
 //     (oldest first, up to a query cap) into the next launch: one upload of
 //     per-request descriptors and one batched find that reads and answers each
-//     request in its own arrays (find shapes other than the line find: a gather
-//     of the queries before it, a scatter after it). Requests that arrive
+//     request in its own arrays (find shapes other than the line find, and
+//     answers that go over queries: a gather of the queries before it, a scatter
+//     after it). Requests that arrive
 //     while launches run join the next launch (continuous batching).
 //   * the build worker admits build requests in arrival order when the table
 //     fits in the HBM budget, allocates its storage and, within what the budget
@@ -131,7 +132,42 @@ struct ght_pool {
   void find_loop();
   void build_loop();
   int launch_finds(Slot &sl, std::vector<uint64_t> &batch);
+  std::vector<uintptr_t> starts, ends;  // the find thread's, for answers_over_queries
+  bool answers_over_queries(const uint32_t *const *src, uint32_t *const *dst, const uint64_t *offs, uint32_t R);
 };
+
+// Whether answers of these requests go where queries of theirs are, other than
+// those of a request answered exactly in place (whose every query the same warp
+// reads before it writes that place): then all queries have to be read before
+// any answer is written. With the ranges of all queries sorted by start and by
+// end, those that a range of answers meets are the ones that start before its
+// end less the ones that end before its start.
+bool ght_pool::answers_over_queries(const uint32_t *const *src, uint32_t *const *dst, const uint64_t *offs,
+                                    uint32_t R) {
+  auto at = [](const void *p) { return reinterpret_cast<uintptr_t>(p); };
+  uintptr_t s_lo = ~(uintptr_t)0, s_hi = 0, d_lo = ~(uintptr_t)0, d_hi = 0;
+  starts.clear();
+  ends.clear();
+  for (uint32_t i = 0; i < R; ++i) {
+    const uint64_t bytes = (offs[i + 1] - offs[i]) * sizeof(uint32_t);
+    starts.push_back(at(src[i]));
+    ends.push_back(at(src[i]) + bytes);
+    s_lo = std::min(s_lo, starts[i]);
+    s_hi = std::max(s_hi, ends[i]);
+    d_lo = std::min(d_lo, at(dst[i]));
+    d_hi = std::max(d_hi, at(dst[i]) + bytes);
+  }
+  if (d_hi <= s_lo || s_hi <= d_lo) return false;
+  std::sort(starts.begin(), starts.end());
+  std::sort(ends.begin(), ends.end());
+  for (uint32_t i = 0; i < R; ++i) {
+    const uintptr_t lo = at(dst[i]), hi = lo + (offs[i + 1] - offs[i]) * sizeof(uint32_t);
+    const auto met = (std::lower_bound(starts.begin(), starts.end(), hi) - starts.begin()) -
+                     (std::upper_bound(ends.begin(), ends.end(), lo) - ends.begin());
+    if (met > (dst[i] == src[i] ? 1 : 0)) return true;
+  }
+  return false;
+}
 
 int ght_pool::launch_finds(Slot &sl, std::vector<uint64_t> &batch) {
   const uint32_t R = (uint32_t)batch.size();
@@ -161,8 +197,10 @@ int ght_pool::launch_finds(Slot &sl, std::vector<uint64_t> &batch) {
   const uint32_t *const *d_src = reinterpret_cast<const uint32_t *const *>(d_offs + R + 1);
   uint32_t *const *d_dst = reinterpret_cast<uint32_t *const *>(d_offs + R + 1 + R);
   // The line find reads and answers each request in its own arrays; the other
-  // find shapes take one array, gathered and scattered around them.
-  const bool direct = find_o.tile_lanes == 4 && find_o.keys_per_lane == 1 && total <= ght::kLineFindMost;
+  // find shapes take one array, gathered and scattered around them, and so do
+  // requests whose answers go over queries.
+  const bool direct = find_o.tile_lanes == 4 && find_o.keys_per_lane == 1 && total <= ght::kLineFindMost &&
+                      !answers_over_queries(src, dst, offs, R);
   const uint64_t need = direct ? 0 : 2ull * total * sizeof(uint32_t) + 512;
   if (sl.staging_bytes < need) {
     if (sl.staging) cudaFreeAsync(sl.staging, find_stream);

@@ -51,3 +51,57 @@ def test_pool_build_scratch_comes_out_of_the_budget(G):
         pool.wait(pool.submit_find(tid, d, out))
         assert (O._u32(out.cpu()) == want).all()
         pool.close()
+
+
+def _tables(G, pool, count, n=40000):
+    sets, ids = [], []
+    for s in range(count):
+        k, v = W.make_keys(n, 10 + s), W.make_values(n, 10 + s)
+        ticket, tid = pool.submit_build(n, 0.95, s, k.cuda(), v.cuda())
+        assert pool.wait(ticket)["status"] == 0
+        sets.append((k, v))
+        ids.append(tid)
+    return sets, ids
+
+
+@pytest.mark.parametrize("shift", [-4097, -33, -1, 0, 1, 31, 32, 4096])
+def test_pool_answers_over_the_queries_of_the_request(G, shift):
+    """One request whose answers start `shift` words from its queries, in the same buffer."""
+    pool = G.Pool(1 << 28)
+    sets, ids = _tables(G, pool, 1)
+    n = 300007
+    q = W.make_queries(sets[0][0], n, 0.6, seed=8)
+    buf = torch.zeros(n + 2 * 5000, dtype=torch.int32, device="cuda")
+    ins, out = buf[5000:5000 + n], buf[5000 + shift:5000 + shift + n]
+    ins.copy_(q)
+    torch.cuda.synchronize()
+    assert pool.wait(pool.submit_find(ids[0], ins, out))["status"] == 0
+    assert (O._u32(out.cpu()) == O.lookup(*sets[0], q)).all()
+    pool.close()
+
+
+def test_pool_answers_over_the_queries_of_others(G):
+    """Requests packed into one launch behind others that keep the pool busy: one is answered over
+    the queries of two others, one in place while another asks the same queries."""
+    pool = G.Pool(1 << 28)
+    sets, ids = _tables(G, pool, 2)
+    n = 100003
+    qa, qb, qc = (W.make_queries(sets[i & 1][0], n, 0.6, seed=20 + i) for i in range(3))
+    a, b, c = (x.cuda() for x in (qa, qb, qc))
+    both = torch.cat([a, b])
+    out_a, out_b, out_c = (torch.empty_like(a) for _ in range(3))
+    busy_q = W.make_queries(sets[0][0], 1 << 22, 0.5, seed=30).cuda()
+    busy_out = torch.empty_like(busy_q)
+    torch.cuda.synchronize()
+    busy = [pool.submit_find(ids[0], busy_q, busy_out) for _ in range(40)]
+    half = n // 2
+    over = both[half:half + n]  # the end of a's queries and the start of b's
+    tickets = [pool.submit_find(ids[0], both[:n], out_a), pool.submit_find(ids[1], both[n:], out_b),
+               pool.submit_find(ids[0], c, over), pool.submit_find(ids[1], c, out_c), pool.submit_find(ids[0], c, c)]
+    packed = [pool.wait(t)["launch_requests"] for t in tickets]
+    for t in busy:
+        pool.wait(t)
+    assert packed == [len(tickets)] * len(tickets)
+    for got, table, q in ((out_a, 0, qa), (out_b, 1, qb), (over, 0, qc), (out_c, 1, qc), (c, 0, qc)):
+        assert (O._u32(got.cpu()) == O.lookup(*sets[table], q)).all()
+    pool.close()
