@@ -441,17 +441,20 @@ int ght_batch_set_stream(ght_batch *b, void *cuda_stream);
  * at 0; table t's key count may not exceed its capacity. Synchronous upload. */
 int ght_batch_set_layout(ght_batch *b, const uint64_t *h_key_offsets, const uint64_t *h_query_offsets);
 
-/* Build every table from the concatenated device arrays with one fill and
- * one insert launch for the whole batch; reads the tables' status words
- * once, then rebuilds each failed table alone with its next constants (up to
- * max_attempts). GHT_ERR_BUILD_FAILED if any table stays unbuilt. */
+/* Build every table from the concatenated device arrays with one fill, one
+ * ranked placement and one insert of its overflow for the whole batch (insert
+ * shapes other than the default, or no memory for the placement's scratch: one
+ * fill and one insert of every key); reads the tables' status words once, then
+ * rebuilds each failed table alone: with the same constants where its keys
+ * found the overflow list full, else with its next ones (up to max_attempts).
+ * GHT_ERR_BUILD_FAILED if any table stays unbuilt. */
 int ght_batch_build(ght_batch *b, const uint32_t *d_keys, const uint32_t *d_values);
 
 /* Find every table's queries with one launch (asynchronous). */
 int ght_batch_find(const ght_batch *b, const uint32_t *d_queries, uint32_t *d_out);
 
-/* Build and find in one CUDA-graph launch (fill, insert, find, status read
- * back), captured on the first call and re-captured when the arrays or the
+/* Build and find in one CUDA-graph launch (the build's launches, find, status
+ * read back), captured on the first call and re-captured when the arrays or the
  * launch shapes change; waits once. Tables whose build failed are rebuilt
  * alone and their queries answered again before returning. The graph is
  * launched on the batch's stream, which must not be capturing. */

@@ -30,6 +30,10 @@ struct BatchView {
 
 constexpr uint64_t kLineFindMost = 0xFFFF0000ull;  // queries of one batched line find (32-bit places)
 
+// Status of a table with keys that found the overflow list of the batch's
+// placement full: not inserted, whatever its constants.
+constexpr uint32_t kStatusListFull = 64u;
+
 // Scratch of a batch's ranked placement: an arrival counter per bucket of the
 // whole slot array, and the overflow list.
 struct BatchPlace {

@@ -132,29 +132,36 @@ int launch_find(const ght_batch *b, uint32_t lo, uint32_t hi, const uint32_t *q,
   return e == cudaSuccess ? GHT_OK : cuda_fail(e, "launching batch find");
 }
 
-// After the mirror holds fresh status words: rebuild each failed table alone
-// with its next constants; optionally answer its queries again.
+// After the mirror holds fresh status words: rebuild each failed table alone,
+// with the same constants where only the placement's list failed it, else with
+// its next ones; optionally answer its queries again.
 int repair(ght_batch *b, const uint32_t *k, const uint32_t *v, const uint32_t *q, uint32_t *out) {
   b->tables_failed = 0;
   for (uint32_t t = 0; t < b->T; ++t) {
-    uint32_t st = b->h_tables[t].status;
+    bool rebuilt = false;
+    auto build_alone = [&]() {
+      rebuilt = true;
+      int rc = upload_tables(b, t, t + 1);
+      if (!rc) rc = launch_build(b, t, t + 1, k, v, true);
+      return rc ? rc : download_tables(b, t, t + 1);
+    };
+    const uint32_t &st = b->h_tables[t].status;
+    if ((st & ght::kStatusListFull) && !(st & ght::kStatusSentinel)) {
+      if (const int rc = build_alone()) return rc;
+    }
     if (st & ght::kStatusSentinel) return fail(GHT_ERR_SENTINEL_KEY, "table %u: an input key is the sentinel", t);
     if (st & ght::kStatusTimeout) return fail(GHT_ERR_DEVICE_TIMEOUT, "table %u: a key exceeded the step bound", t);
     if (st & ght::kStatusCorrupt) return fail(GHT_ERR_CUDA, "table %u: corrupt", t);
     while (st != 0u && b->attempt[t] + 1 < b->max_attempts) {
       b->set_constants(t, b->attempt[t] + 1);
       b->rebuilds++;
-      int rc = upload_tables(b, t, t + 1);
-      if (!rc) rc = launch_build(b, t, t + 1, k, v, true);
-      if (!rc) rc = download_tables(b, t, t + 1);
-      if (rc) return rc;
-      st = b->h_tables[t].status;
+      if (const int rc = build_alone()) return rc;
     }
     if (st != 0u) {
       b->tables_failed++;
       continue;
     }
-    if (q && b->rebuilds && b->attempt[t] > 0) {
+    if (q && rebuilt) {
       const int rc = launch_find(b, t, t + 1, q, out);
       if (rc) return rc;
     }

@@ -190,8 +190,10 @@ batch_fill_kernel(BatchView bv, uint4 *__restrict__ slots16, uint64_t n16, uint3
 // rank_place_kernel for one table): a key's arrival number at its bucket H_0
 // comes from the bucket's counter (bl.counters, one per bucket in slot order),
 // numbers below 16 are stored in that slot, the other keys go to the overflow
-// list with their table. A key that no longer fits the list fails its table's
-// attempt (the table is then rebuilt alone). The warps take the chunks of 32
+// list with their table. A key that no longer fits the list marks its table
+// (kStatusListFull), which is then built alone, with the same constants and the
+// insert of every key: the keys that crowd the list may be another table's. The
+// warps take the chunks of 32
 // pairs in turn, so the stores and counters in flight stay in the few tables
 // that the chunks are in. Build of 512 tables of 2^10..2^20 keys at LF
 // 0.8..0.99 (85 M keys): 3.75 ms with the insert of every key, 2.54 now; 64
@@ -222,7 +224,7 @@ batch_place_kernel(BatchView bv, BatchPlace bl, const uint32_t *__restrict__ key
         bl.v[at] = over[1][waiting + lane];
         bl.table[at] = over[2][waiting + lane];
       } else {
-        atomicOr(&bv.tables[over[2][waiting + lane]].status, kStatusBuildFailed);
+        atomicOr(&bv.tables[over[2][waiting + lane]].status, kStatusListFull);
       }
     }
     __syncwarp();

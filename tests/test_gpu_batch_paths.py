@@ -1,0 +1,55 @@
+"""Batched tables on the paths beside the default one: a crowded table beside
+others, every find shape, and the memory a batch takes."""
+
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def G():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2108_07232_gb300 import build
+    build.build()
+    import paper_2108_07232_gb300 as G
+    return G
+
+
+@pytest.mark.parametrize("run", [True, False])
+def test_a_crowded_table_costs_no_table_its_attempt(G, run):
+    """All keys of one table share their first bucket, so they fill the batch's overflow list and
+    other tables' keys find it full; every table's first constants build it (the oracle's insert of
+    the crowded one too), so a batch with a single attempt must build them all."""
+    n, others, seed = 6000, 40, 29
+    m = O.num_buckets(n, 0.5, 16)
+    a, c = O.derive_constants(seed, 0, 3)
+    cand = np.arange(1, 1 << 24, dtype=np.uint64)
+    h0 = ((np.uint64(a[0]) * cand + np.uint64(c[0])) % np.uint64(O.PRIME)) % np.uint64(m)
+    crowd = cand[h0 == h0[0]][:n].astype(np.uint32)
+    alone = O.Table(O.BCHT, n, 0.5)
+    alone.set_constants(a, c)
+    rest = W.make_keys(2 * others * 300, 3).numpy().view(np.uint32)
+    rest = rest[~np.isin(rest, crowd)][: others * 300]
+    keys = torch.from_numpy(np.concatenate([crowd, rest]).view(np.int32).copy())
+    vals = W.make_values(keys.numel(), 8)
+    assert alone.build(keys[:n], vals[:n]) == 1
+    b = G.Batch([n] + [300] * others, [0.5] + [0.95] * others, seed=seed, max_attempts=1)
+    offs = np.concatenate([[0], n + 300 * np.arange(others + 1)]).astype(np.uint64)
+    b.set_layout(offs, offs)
+    dk, dv = keys.cuda(), vals.cuda()
+    for _ in range(3):
+        if run:
+            out = b.run(dk, dv, dk)
+        else:
+            b.build(dk, dv)
+            out = b.find(dk)
+        assert torch.equal(out, dv)
+        st = b.stats()
+        assert st["tables_failed"] == 0 and st["rebuilds"] == 0
+        assert all(b.table_stats(t)["attempts"] == 1 for t in range(others + 1))
