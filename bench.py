@@ -715,7 +715,7 @@ def batched_measure(dev, seed, num_tables, log2_max, steps, warmup):
                    "input_seed": seed},
         "graph_ms": graph_ms, "autotuned": {kk: tuned[kk] for kk in ("tile_lanes", "keys_per_lane", "blocks_per_sm",
                                                                      "build_tile_lanes", "build_keys_per_lane",
-                                                                     "build_blocks_per_sm") if kk in tuned},
+                                                                     "build_blocks_per_sm", "find_line") if kk in tuned},
         "rebuilds": st["rebuilds"],
         "plain_back_to_back": {"value": round(items * steps / (ms_plain / 1e3) / 1e9, 3), "unit": "Gkeys/s",
                                "ms_per_step": round(ms_plain / steps, 3),

@@ -94,8 +94,9 @@ typedef struct {
    * find_async 0 and tile_lanes and keys_per_lane 0 or as
    * ght_default_config gives them, 128-byte buckets are read by the line find
    * (32-byte loads, one query per lane, queries that need another bucket
-   * refill the warp), which is faster at every size; other values select the
-   * register or staged find. Build: the same three for the insert kernel. */
+   * refill the warp); other values, or find_async -1, select the register or
+   * staged find. Tables, batches and pools alike. Build: the same three for the
+   * insert kernel. */
   int32_t tile_lanes;
   int32_t blocks_per_sm;
   int32_t keys_per_lane;
@@ -426,6 +427,7 @@ typedef struct {
   uint64_t graph_launches;
   int32_t blocks_per_sm;       /* find grid: resident blocks per SM (0 = as many as fit) */
   int32_t build_blocks_per_sm; /* insert grid, likewise */
+  int32_t find_line;           /* 1: the line find answers, whatever the find shape above */
 } ght_batch_stats_t;
 
 /* Create num_tables empty tables, table t sized for h_capacities[t] keys at
@@ -463,8 +465,8 @@ int ght_batch_run(ght_batch *b, const uint32_t *d_keys, const uint32_t *d_values
 
 /* Choose the insert and find launch shapes by timing each candidate on
  * these arrays: first the tile shape (lanes per bucket tile, keys per lane;
- * for finds 4 lanes and one query per lane is the line find, the default, and
- * 4-lane tiles with 6 query sets per lane the staged find
+ * for finds the line find, the default, comes before them, and 4-lane tiles
+ * with 6 query sets per lane are the staged find
  * whose bucket parts wait in shared memory), then the grid (1-4 resident
  * blocks per SM, or as many as fit) of the best shape; keeps the fastest.
  * The tables are rebuilt as a side effect. */

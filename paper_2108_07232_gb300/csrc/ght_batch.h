@@ -22,7 +22,7 @@ struct BatchView {
   const uint64_t *query_offs;  // num_tables + 1 prefix offsets into the query/result arrays
   Ctrl *ctrl;                  // batch-wide probe counters
   const uint32_t *const *src;  // finds, if set: each segment's queries and answers in arrays of its own
-  uint32_t *const *dst;        // (the line find alone reads them: 4 lanes, one query per lane)
+  uint32_t *const *dst;        // (the line find alone reads them)
   uint32_t t_lo, t_hi;         // tables this launch covers
   int32_t h;
   uint32_t max_chain, max_steps, rng_seed;
@@ -44,10 +44,12 @@ struct BatchPlace {
 };
 
 bool batch_shape_supported(int tile_lanes, int keys_per_lane);
-// Find shapes: the above, of which 4-lane tiles with one query per lane are the
-// line find (32-byte loads, the default), and 4-lane tiles with 6 query sets
-// per lane (the staged find: bucket parts in shared memory).
+// Find shapes: the above, and 4-lane tiles with 6 query sets per lane (the
+// staged find: bucket parts in shared memory).
 bool batch_find_shape_supported(int tile_lanes, int keys_per_lane);
+// A config's find: its shape, or the line find (32-byte loads) where it names
+// no other than ght_default_config gives, as for one table.
+void batch_find_shape(const ght_config *cfg, LaunchOpts *o);
 
 // Describe a built single BCHT table (b = 16) as a batch descriptor (ght_api.cu).
 // Returns false if the table is not a built 16-pair BCHT table.

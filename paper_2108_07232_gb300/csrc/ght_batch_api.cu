@@ -72,8 +72,8 @@ struct ght_batch {
   }
 
   int shape_sig() const {
-    return ((build_o.blocks_per_sm * 64 + find_o.blocks_per_sm) * 100 + build_o.tile_lanes) * 1000 +
-           build_o.keys_per_lane * 100 + find_o.tile_lanes * 10 + find_o.keys_per_lane;
+    return (((build_o.blocks_per_sm * 64 + find_o.blocks_per_sm) * 100 + build_o.tile_lanes) * 1000 +
+            build_o.keys_per_lane * 100 + find_o.tile_lanes * 10 + find_o.keys_per_lane) * 2 + find_o.line_find;
   }
 
   void drop_graph() {
@@ -199,8 +199,7 @@ ght_batch *ght_batch_create(uint32_t num_tables, const uint64_t *h_capacities, c
   }
   b->T = num_tables;
   b->seed = seed;
-  b->find_o.tile_lanes = 4;
-  b->find_o.keys_per_lane = 1;  // the line find
+  ght::batch_find_shape(cfg, &b->find_o);
   b->build_o.tile_lanes = 16;
   b->build_o.keys_per_lane = 1;
   if (cfg) {
@@ -216,8 +215,6 @@ ght_batch *ght_batch_create(uint32_t num_tables, const uint64_t *h_capacities, c
     }
     if (cfg->max_chain) b->max_chain = cfg->max_chain;
     if (cfg->max_attempts) b->max_attempts = cfg->max_attempts;
-    if (cfg->tile_lanes) b->find_o.tile_lanes = cfg->tile_lanes;
-    if (cfg->keys_per_lane) b->find_o.keys_per_lane = cfg->keys_per_lane;
     if (cfg->build_tile_lanes) b->build_o.tile_lanes = cfg->build_tile_lanes;
     if (cfg->build_keys_per_lane) b->build_o.keys_per_lane = cfg->build_keys_per_lane;
     b->find_o.blocks_per_sm = cfg->blocks_per_sm;
@@ -429,7 +426,8 @@ int ght_batch_autotune(ght_batch *b, const uint32_t *d_keys, const uint32_t *d_v
   // tile shapes (lanes per bucket, keys per lane), then the grid (resident
   // blocks per SM; 0 = as many as fit) of the chosen shape
   static const int kBuild[][2] = {{16, 1}, {8, 1}, {8, 2}, {4, 2}};
-  static const int kFind[][2] = {{4, 1}, {4, 2}, {8, 2}, {8, 1}, {16, 1}, {4, 6}};  // the line find first; {4, 6}: staged
+  static const int kFind[][3] = {{4, 2, 1}, {4, 2, 0}, {4, 1, 0}, {8, 2, 0}, {8, 1, 0},
+                                 {16, 1, 0}, {4, 6, 0}};  // the line find first; {4, 6}: staged
   static const int kGrid[] = {0, 1, 2, 3, 4};
   if (b->build_o.blocks_per_sm < 0 || b->find_o.blocks_per_sm < 0) return fail(GHT_ERR_INVALID_ARG, "negative grid");
   auto time_between = [&](float *out_ms) -> int {
@@ -491,6 +489,7 @@ int ght_batch_autotune(ght_batch *b, const uint32_t *d_keys, const uint32_t *d_v
   for (const auto &c : kFind) {
     b->find_o.tile_lanes = c[0];
     b->find_o.keys_per_lane = c[1];
+    b->find_o.line_find = c[2] != 0;
     if ((rc = time_find(&total))) return rc;
     if (total < best) {
       best = total;
@@ -532,6 +531,7 @@ int ght_batch_stats(const ght_batch *b, ght_batch_stats_t *out) {
   out->graph_launches = b->graph_launches;
   out->blocks_per_sm = b->find_o.blocks_per_sm;
   out->build_blocks_per_sm = b->build_o.blocks_per_sm;
+  out->find_line = b->find_o.line_find ? 1 : 0;
   return GHT_OK;
 }
 

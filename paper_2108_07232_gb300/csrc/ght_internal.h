@@ -21,6 +21,7 @@ struct LaunchOpts {
   bool ordered = false;  // insert: the warps advance through the input together
   bool overflow = false;  // insert: the pairs are a placement's overflow, counted in the control block
   bool async_find = false;  // find: bucket parts staged in shared memory (BCHT, b = 16, 4-lane tiles)
+  bool line_find = false;   // find of a batch or pool: the line find, whatever the tile shape
 };
 
 constexpr uint32_t kMaxGroups = 4096;

@@ -199,8 +199,8 @@ int ght_pool::launch_finds(Slot &sl, std::vector<uint64_t> &batch) {
   // The line find reads and answers each request in its own arrays; the other
   // find shapes take one array, gathered and scattered around them, and so do
   // requests whose answers go over queries.
-  const bool direct = find_o.tile_lanes == 4 && find_o.keys_per_lane == 1 && total <= ght::kLineFindMost &&
-                      !answers_over_queries(src, dst, offs, R);
+  const bool direct =
+      find_o.line_find && total <= ght::kLineFindMost && !answers_over_queries(src, dst, offs, R);
   const uint64_t need = direct ? 0 : 2ull * total * sizeof(uint32_t) + 512;
   if (sl.staging_bytes < need) {
     if (sl.staging) cudaFreeAsync(sl.staging, find_stream);
@@ -436,10 +436,7 @@ ght_pool *ght_pool_create(uint64_t hbm_budget_bytes, const ght_config *cfg) {
     if (cfg->tile_lanes) p->cfg.tile_lanes = cfg->tile_lanes;
     if (cfg->keys_per_lane) p->cfg.keys_per_lane = cfg->keys_per_lane;
   }
-  p->find_o.tile_lanes = p->cfg.tile_lanes;
-  p->find_o.keys_per_lane = p->cfg.keys_per_lane;
-  // a config that names no other find shape than the default: the line find
-  if (p->find_o.tile_lanes == 4 && p->find_o.keys_per_lane == 2) p->find_o.keys_per_lane = 1;
+  ght::batch_find_shape(cfg, &p->find_o);
   if (!ght::batch_find_shape_supported(p->find_o.tile_lanes, p->find_o.keys_per_lane)) {
     fail(GHT_ERR_INVALID_ARG, "unsupported find shape");
     delete p;

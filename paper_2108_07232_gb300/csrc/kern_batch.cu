@@ -966,6 +966,12 @@ bool batch_shape_supported(int G, int kpl) {
 
 bool batch_find_shape_supported(int G, int kpl) { return batch_shape_supported(G, kpl) || (G == 4 && kpl == 6); }
 
+void batch_find_shape(const ght_config *cfg, LaunchOpts *o) {
+  o->tile_lanes = cfg && cfg->tile_lanes ? cfg->tile_lanes : 4;
+  o->keys_per_lane = cfg && cfg->keys_per_lane ? cfg->keys_per_lane : 2;
+  o->line_find = o->tile_lanes == 4 && o->keys_per_lane == 2 && !(cfg && cfg->find_async < 0);
+}
+
 // staged find: 6 query sets per lane, 2-warp blocks (24 KB of shared memory per warp)
 static cudaError_t find_staged(const BatchView &bv, const uint32_t *q, uint32_t *out, uint64_t items,
                                const LaunchOpts &o, cudaStream_t s) {
@@ -1023,11 +1029,12 @@ cudaError_t launch_batch_find(const BatchView &bv, const uint32_t *q, uint32_t *
                               const LaunchOpts &o, cudaStream_t s) {
   if (items == 0) return cudaSuccess;
   const int g = o.tile_lanes, kpl = o.keys_per_lane;
-  if (bv.src && !(g == 4 && kpl == 1 && items <= kLineFindMost)) return cudaErrorInvalidValue;
+  if (bv.src && !(o.line_find && items <= kLineFindMost)) return cudaErrorInvalidValue;
+  if (o.line_find) return find_lines(bv, q, out, items, o, s);
   if (g == 16) return kpl == 1 ? find_cfg<16, 1>(bv, q, out, items, o, s) : find_cfg<16, 2>(bv, q, out, items, o, s);
   if (g == 8) return kpl == 1 ? find_cfg<8, 1>(bv, q, out, items, o, s) : find_cfg<8, 2>(bv, q, out, items, o, s);
   if (g == 4 && kpl == 6) return find_staged(bv, q, out, items, o, s);
-  if (g == 4) return kpl == 1 ? find_lines(bv, q, out, items, o, s) : find_cfg<4, 2>(bv, q, out, items, o, s);
+  if (g == 4) return kpl == 1 ? find_cfg<4, 1>(bv, q, out, items, o, s) : find_cfg<4, 2>(bv, q, out, items, o, s);
   return cudaErrorInvalidValue;
 }
 

@@ -53,3 +53,46 @@ def test_a_crowded_table_costs_no_table_its_attempt(G, run):
         st = b.stats()
         assert st["tables_failed"] == 0 and st["rebuilds"] == 0
         assert all(b.table_stats(t)["attempts"] == 1 for t in range(others + 1))
+
+
+def _uneven(seed):
+    return W.make_batch(60, 3, 13, 0.8, 0.99, 2.0, 0.6, seed=seed)
+
+
+@pytest.mark.parametrize("cfg,shape", [
+    ({}, (4, 2, 1)), ({"tile_lanes": 4, "keys_per_lane": 2}, (4, 2, 1)), ({"find_async": -1}, (4, 2, 0)),
+    ({"tile_lanes": 8}, (8, 2, 0)), ({"tile_lanes": 16}, (16, 2, 0)), ({"keys_per_lane": 1}, (4, 1, 0)),
+    ({"tile_lanes": 8, "keys_per_lane": 1}, (8, 1, 0)), ({"tile_lanes": 16, "keys_per_lane": 1}, (16, 1, 0)),
+    ({"tile_lanes": 4, "keys_per_lane": 6}, (4, 6, 0))])
+def test_every_batch_find_shape(G, cfg, shape):
+    """A config's shape is the one that runs (a missing half is the default's), the default and the
+    values of the default config are the line find, and all answer alike; sentinel queries too."""
+    w = _uneven(5)
+    b = G.Batch(w["capacities"], w["load_factors"], seed=2, **cfg)
+    st = b.stats()
+    assert (st["tile_lanes"], st["keys_per_lane"], st["find_line"]) == shape
+    b.set_layout(w["key_offsets"], w["query_offsets"])
+    q = w["queries"].clone()
+    q[5::37] = -1
+    b.build(w["keys"].cuda(), w["values"].cuda())
+    got = O._u32(b.find(q.cuda()).cpu())
+    ko, qo = w["key_offsets"], w["query_offsets"]
+    for t in range(b.num_tables):
+        want = O.lookup(w["keys"][ko[t]:ko[t + 1]], w["values"][ko[t]:ko[t + 1]], q[qo[t]:qo[t + 1]])
+        assert (got[qo[t]:qo[t + 1]] == want).all(), t
+
+
+@pytest.mark.parametrize("cfg", [{"keys_per_lane": 1}, {"find_async": -1}, {"tile_lanes": 16}, {"tile_lanes": 4, "keys_per_lane": 2}])
+def test_pool_find_shapes_answer_alike(G, cfg):
+    pool = G.Pool(1 << 28, **cfg)
+    k, v = W.make_keys(30000, 1), W.make_values(30000, 1)
+    ticket, tid = pool.submit_build(30000, 0.95, 1, k.cuda(), v.cuda())
+    assert pool.wait(ticket)["status"] == 0
+    for n in (1, 33, 70001):
+        q = W.make_queries(k, n, 0.6, seed=n)
+        d = q.cuda()
+        out = torch.empty_like(d)
+        torch.cuda.synchronize()
+        assert pool.wait(pool.submit_find(tid, d, out))["status"] == 0
+        assert (O._u32(out.cpu()) == O.lookup(k, v, q)).all()
+    pool.close()
