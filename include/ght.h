@@ -445,8 +445,9 @@ int ght_batch_set_layout(ght_batch *b, const uint64_t *h_key_offsets, const uint
 
 /* Build every table from the concatenated device arrays with one fill, one
  * ranked placement and one insert of its overflow for the whole batch (insert
- * shapes other than the default, or no memory for the placement's scratch: one
- * fill and one insert of every key); reads the tables' status words once, then
+ * shapes other than the default, or no memory for the placement's scratch of
+ * about 3 bytes a key, which the batch keeps: one fill and one insert of every
+ * key); reads the tables' status words once, then
  * rebuilds each failed table alone: with the same constants where its keys
  * found the overflow list full, else with its next ones (up to max_attempts).
  * GHT_ERR_BUILD_FAILED if any table stays unbuilt. */

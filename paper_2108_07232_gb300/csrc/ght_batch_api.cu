@@ -108,13 +108,40 @@ int download_tables(ght_batch *b, uint32_t lo, uint32_t hi) {
 // Overflow list of a two-phase batch build of n keys, as for one table.
 uint64_t place_cap(uint64_t n) { return std::min<uint64_t>(n, n / 4 + 1024); }
 
+// The insert shape that builds in two phases.
+bool two_phase_shape(const ght_batch *b) { return b->build_o.tile_lanes == 16 && b->build_o.keys_per_lane == 1; }
+
+// Take the scratch of the two-phase build where the insert shape runs it, give
+// it back where it does not. Without it (no memory) builds insert every key.
+void fit_place_scratch(ght_batch *b) {
+  if (two_phase_shape(b) == (b->place_mem != nullptr)) return;
+  if (b->place_mem) {
+    cudaStreamSynchronize(b->stream);
+    cudaFree(b->place_mem);
+    b->place_mem = nullptr;
+    b->place = ght::BatchPlace();
+    return;
+  }
+  uint64_t keys_most = 0;
+  for (uint64_t c : b->caps) keys_most += c;
+  const uint64_t cap = place_cap(keys_most), counters = b->total_slots / 16;
+  if (keys_most > 0 && cudaMalloc(&b->place_mem, (counters + 3 * cap) * sizeof(uint32_t)) == cudaSuccess) {
+    b->place.slots = static_cast<uint64_t *>(b->slots_mem);
+    b->place.counters = static_cast<uint32_t *>(b->place_mem);
+    b->place.k = b->place.counters + counters;
+    b->place.v = b->place.k + cap;
+    b->place.table = b->place.v + cap;
+    b->place.cap = cap;
+  }
+  cudaGetLastError();
+}
+
 // Fill + insert of tables [lo, hi) (no wait): in two phases with the default
 // insert shape, unless `plain` (a rebuild, whatever made the first attempt fail).
 int launch_build(ght_batch *b, uint32_t lo, uint32_t hi, const uint32_t *k, const uint32_t *v, bool plain = false) {
   const ght::BatchView bv = b->view(lo, hi);
   const uint64_t items = b->key_offs[hi] - b->key_offs[lo];
-  const bool two = !plain && b->place.cap > 0 && b->build_o.tile_lanes == 16 && b->build_o.keys_per_lane == 1 &&
-                   items <= 0xFFFF0000ull;
+  const bool two = !plain && b->place.cap > 0 && two_phase_shape(b) && items <= 0xFFFF0000ull;
   uint64_t *slots = static_cast<uint64_t *>(b->slots_mem) + b->slot_off[lo];
   const uint64_t nslots = b->slot_off[hi] - b->slot_off[lo];
   cudaError_t e = ght::launch_batch_fill(bv, slots, nslots, two ? b->place.counters + b->slot_off[lo] / 16 : nullptr,
@@ -265,19 +292,7 @@ ght_batch *ght_batch_create(uint32_t num_tables, const uint64_t *h_capacities, c
     ght_batch_destroy(b);
     return nullptr;
   }
-  // scratch of the two-phase build; without it (no memory) builds insert every key
-  uint64_t keys_most = 0;
-  for (uint32_t t = 0; t < num_tables; ++t) keys_most += h_capacities[t];
-  const uint64_t cap = place_cap(keys_most), counters = b->total_slots / 16;
-  if (keys_most > 0 && cudaMalloc(&b->place_mem, (counters + 3 * cap) * sizeof(uint32_t)) == cudaSuccess) {
-    b->place.slots = static_cast<uint64_t *>(b->slots_mem);
-    b->place.counters = static_cast<uint32_t *>(b->place_mem);
-    b->place.k = b->place.counters + counters;
-    b->place.v = b->place.k + cap;
-    b->place.table = b->place.v + cap;
-    b->place.cap = cap;
-  }
-  cudaGetLastError();
+  fit_place_scratch(b);
   char *p = static_cast<char *>(b->meta_mem);
   b->d_tables = reinterpret_cast<ght::BatchTable *>(p);
   p += num_tables * sizeof(ght::BatchTable);
@@ -465,6 +480,7 @@ int ght_batch_autotune(ght_batch *b, const uint32_t *d_keys, const uint32_t *d_v
   for (const auto &c : kBuild) {
     b->build_o.tile_lanes = c[0];
     b->build_o.keys_per_lane = c[1];
+    if (two_phase_shape(b)) fit_place_scratch(b);
     if ((rc = time_build(&total))) return rc;
     if (total < best) {
       best = total;
@@ -508,7 +524,8 @@ int ght_batch_autotune(ght_batch *b, const uint32_t *d_keys, const uint32_t *d_v
   }
   b->find_o = best_o;
   b->tuned = 1;
-  b->drop_graph();
+  b->drop_graph();  // (it may hold the placement's launches)
+  fit_place_scratch(b);
   return GHT_OK;
 }
 

@@ -96,3 +96,34 @@ def test_pool_find_shapes_answer_alike(G, cfg):
         assert pool.wait(pool.submit_find(tid, d, out))["status"] == 0
         assert (O._u32(out.cpu()) == O.lookup(k, v, q)).all()
     pool.close()
+
+
+def test_a_batch_takes_placement_scratch_only_where_it_places(G):
+    """An insert shape without the placement keeps no scratch for it; the autotuner takes it to
+    time the default shape and keeps it only if that wins."""
+    n = 1 << 24
+    slots = O.num_buckets(n, 0.9, 16) * 128
+    scratch = (slots // 128 + 3 * (n // 4)) * 4  # 55 MB
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+
+    def taken():
+        torch.cuda.synchronize()
+        return before - torch.cuda.mem_get_info()[0] - slots
+
+    b = G.Batch([n], [0.9], seed=1, build_tile_lanes=8)
+    assert taken() < scratch // 2
+    b.close()
+    b = G.Batch([n], [0.9], seed=1)
+    assert taken() > scratch // 2
+    b.close()
+    assert taken() + slots < scratch // 2
+
+    w = _uneven(9)
+    k, v, q = w["keys"].cuda(), w["values"].cuda(), w["queries"].cuda()
+    for cfg in ({"build_tile_lanes": 8}, {}):
+        b = G.Batch(w["capacities"], w["load_factors"], seed=4, **cfg)
+        b.set_layout(w["key_offsets"], w["query_offsets"])
+        first = b.run(k, v, q)
+        b.autotune(k, v, q)
+        assert torch.equal(b.run(k, v, q), first)
