@@ -514,10 +514,10 @@ bool places_ungrouped(const ght_table *t) {
 // 64 / 85; set LF 0.95 4000 34 / 79, 27,000 60 / 86; P2BHT LF 0.75 4000 34 / 64,
 // 20,000 60 / 63; load-balanced LF 0.9 20,000 72 / 81, 24,000 92 / 83; bucket size
 // one (its insert in place of two phases) LF 0.8 1000 51 / 65, 2000 68 / 68, 4000
-// 78 / 67.
-bool wants_small(const ght_table *t, uint64_t n) {
+// 78 / 67. host_input: from page-locked arrays read in place.
+bool wants_small(const ght_table *t, uint64_t n, bool host_input = false) {
   const Shape &s = t->shape;
-  if (!s.small_build || !ght::small_build_fits(s.b, s.m, n)) return false;
+  if (!s.small_build || !ght::small_build_fits(s.b, s.scheme == GHT_BCHT_SET, s.m, n, host_input)) return false;
   switch (s.scheme) {
     case GHT_BCHT: return n <= (t->lf <= 0.96 ? 18432u : 8192u);
     case GHT_CUCKOO1: return n <= 2048u;
@@ -527,8 +527,8 @@ bool wants_small(const ght_table *t, uint64_t n) {
   }
 }
 
-bool wants_ranked(const ght_table *t, uint64_t n) {
-  if (wants_small(t, n)) return false;
+bool wants_ranked(const ght_table *t, uint64_t n, bool host_input = false) {
+  if (wants_small(t, n, host_input)) return false;
   const uint32_t limit = place_limit(t->shape);
   if (t->shape.ranked_build < 0 || n == 0 || n > 0xFFFFFFFFull) return false;
   if (places_by_load(t->shape)) return t->shape.group_build <= 0;  // in input order
@@ -628,7 +628,7 @@ struct BuildPath {
 
 BuildPath build_path(const ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n, bool host_input) {
   BuildPath p;
-  p.ranked = wants_ranked(t, n);
+  p.ranked = wants_ranked(t, n, host_input);
   p.grouped = wants_grouping(t, n);
   if (p.grouped && (host_input || ((reinterpret_cast<uintptr_t>(k) | reinterpret_cast<uintptr_t>(v ? v : k)) & 15u))) {
     p.grouped = false;
@@ -940,7 +940,7 @@ int build_device(ght_table *t, const uint32_t *k, const uint32_t *v, uint64_t n,
                  bool host_input = false) {
   t->built = false;
   t->n_stored = 0;
-  const bool small = wants_small(t, n);
+  const bool small = wants_small(t, n, host_input);
   BuildPath path = build_path(t, k, v, n, host_input);
   void *pool_buf = nullptr;
   char *scr = nullptr;

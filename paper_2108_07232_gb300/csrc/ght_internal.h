@@ -239,7 +239,8 @@ cudaError_t launch_block_place(int B, bool key_slots, const TableView &tv, const
 
 // kern_small.cu: the whole build (fill, inserts, control block) of a table that
 // fits one SM's shared memory, by one block; limit: as PlaceBuffers::limit.
-bool small_build_fits(int B, uint64_t m, uint64_t n);
+// far_values: the values are in host memory.
+bool small_build_fits(int B, bool key_slots, uint64_t m, uint64_t n, bool far_values);
 cudaError_t launch_small_build(int scheme, int B, bool key_slots, const TableView &tv, const uint32_t *k,
                                const uint32_t *v, uint64_t n, uint32_t limit, bool count, PublishedCtrl *host,
                                unsigned long long number, cudaStream_t s);

@@ -305,14 +305,22 @@ static cudaError_t launch_small(const TableView &tv, const uint32_t *k, const ui
   return cudaGetLastError();
 }
 
-bool small_build_fits(int B, uint64_t m, uint64_t n) {
-  return n <= (uint64_t)kSmallThreads * kSmallKeys && small_build_smem(B, m, n) <= kSmallSmem;
+// Values that do not fit beside the keys are gathered 4 bytes at a time when the
+// table is written. From host memory that takes L1, which the lines fetched over
+// the link stay in: none is left beside more than 195 KB. Builds from page-locked
+// arrays, us, this / two phases: IHT LF 0.78 21,000 keys (198 KB) 65 / 71, 22,000
+// (208 KB) 121 / 72; LF 0.6 18,000 (199 KB) 55 / 60, 19,000 (210 KB) 104 / 59;
+// P2BHT LF 0.6 18,000 61 / 60, 19,000 109 / 59.
+bool small_build_fits(int B, bool key_slots, uint64_t m, uint64_t n, bool far_values) {
+  const uint64_t smem = small_build_smem(B, m, n);
+  if (n > (uint64_t)kSmallThreads * kSmallKeys || smem > kSmallSmem) return false;
+  return !far_values || key_slots || smem <= 195u * 1024u || smem + 4u * n <= kSmallSmem;
 }
 
 cudaError_t launch_small_build(int scheme, int B, bool key_slots, const TableView &tv, const uint32_t *k,
                                const uint32_t *v, uint64_t n, uint32_t limit, bool count, PublishedCtrl *host,
                                unsigned long long number, cudaStream_t s) {
-  if (!small_build_fits(B, tv.m, n)) return cudaErrorInvalidValue;
+  if (!small_build_fits(B, key_slots, tv.m, n, false)) return cudaErrorInvalidValue;
   if (key_slots) return launch_small<kBCHT, 32, KeySlot>(tv, k, v, n, limit, count, host, number, s);
   if (scheme == kCuckoo1) return launch_small<kCuckoo1, 1, PairSlot>(tv, k, v, n, limit, count, host, number, s);
   if (B == 16) {
