@@ -501,9 +501,12 @@ double expected_overflow(uint64_t n, uint64_t m, uint32_t limit) {
 // order (low thresholds, or load factors where it rarely succeeds).
 // Ungrouped, the placement's stores and counters go to DRAM one sector each on
 // tables beyond the L2: above twice its size (where 2^28 keys took 17.6 ms
-// against 16.8 in input order) only on request.
+// against 16.8 in input order) only on request, and so for bucket size one,
+// where every key has a sector of its own (whole builds, us, ungrouped / input
+// order: 13 M keys LF 0.8 961 / 817, 2^24 LF 0.8 1475 / 1286, LF 0.6 1291 / 876).
 bool places_ungrouped(const ght_table *t) {
-  return t->shape.ranked_build > 0 || t->storage_bytes < 2ull * device_l2_bytes();
+  return t->shape.ranked_build > 0 ||
+         (t->shape.scheme != GHT_CUCKOO1 && t->storage_bytes < 2ull * device_l2_bytes());
 }
 
 // Whether a build of n keys runs in one block (kern_small.cu): where the table

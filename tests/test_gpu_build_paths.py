@@ -53,3 +53,17 @@ def test_one_block_builds_from_page_locked_arrays(G, scheme, lf, n, ranked):
         t.build(place(keys), None if scheme == "bcht_set" else place(vals))
         st = _check(G, t, scheme, keys, vals)
         assert st["last_build_ranked"] == two_phase and (st["last_fill_ms"] == 0.0) == (not two_phase)
+
+
+def test_bucket_size_one_is_placed_ungrouped_only_on_request(G):
+    """Between the L2's size and twice it: arrays off a 16-byte boundary and page-locked ones, which
+    build ungrouped, are inserted in input order; the ungrouped placement on request."""
+    n, lf = (1 << 24) + 3, 0.8  # 168 MB of slots
+    keys, vals = W.make_keys(n + 1, 6), W.make_values(n + 1, 6)
+    dk, dv = keys.cuda(), vals.cuda()
+    for cfg, k, v, ranked in (({}, dk[1:], dv[1:], 0), ({"ranked_build": 1}, dk[1:], dv[1:], 1),
+                              ({}, keys[:n].pin_memory(), vals[:n].pin_memory(), 0)):
+        t = G.HashTable("cuckoo1", n, lf, seed=2, **cfg)
+        t.build(k, v)
+        st = _check(G, t, "cuckoo1", k.cpu(), v.cpu())
+        assert (st["last_build_ranked"], st["last_build_grouped"]) == (ranked, 0)
