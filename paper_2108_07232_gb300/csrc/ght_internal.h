@@ -104,6 +104,24 @@ inline cudaError_t grid_for_smem(K kernel, int threads, size_t smem, uint64_t n,
   return cudaSuccess;
 }
 
+// Raise a kernel's dynamic shared-memory limit on the current device to `smem`
+// where it is below, once per device and kernel: for launches whose grid does not
+// depend on the occupancy, whatever share of `smem` each of them takes.
+template <typename K>
+inline cudaError_t allow_smem(K kernel, size_t smem) {
+  static std::mutex mu;
+  static std::unordered_map<int, std::unordered_map<const void *, size_t>> limit;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lock(mu);
+  size_t &now = limit[dev][(const void *)kernel];
+  if (now >= smem) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess) now = smem;
+  return e;
+}
+
 // Warps of a grid share the input in contiguous slices of this many items.
 inline uint64_t per_warp_of(uint64_t n, int blocks) {
   const uint64_t warps = (uint64_t)blocks * (kThreads / 32);

@@ -298,8 +298,7 @@ static cudaError_t launch_small(const TableView &tv, const uint32_t *k, const ui
   uint64_t smem = small_build_smem(B, tv.m, n);
   const bool keep_values = sizeof(typename S::T) == 8 && smem + 4u * n <= kSmallSmem;
   if (keep_values) smem += 4u * n;
-  int blocks = 0;
-  const cudaError_t e = grid_for_smem(kern, kSmallThreads, smem, 1, 1, &blocks);  // sets the kernel's memory limit
+  const cudaError_t e = allow_smem(kern, kSmallSmem);
   if (e != cudaSuccess) return e;
   kern<<<1, kSmallThreads, smem, s>>>(tv, k, v, (uint32_t)n, limit, keep_values, host, number);
   return cudaGetLastError();

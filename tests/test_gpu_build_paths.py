@@ -67,3 +67,22 @@ def test_bucket_size_one_is_placed_ungrouped_only_on_request(G):
         t.build(k, v)
         st = _check(G, t, "cuckoo1", k.cpu(), v.cpu())
         assert (st["last_build_ranked"], st["last_build_grouped"]) == (ranked, 0)
+
+
+def test_one_block_builds_of_many_sizes_keep_nothing_per_size(G):
+    """Builds of 4000 different key counts leave nothing behind on the host heap."""
+    class Info(ctypes.Structure):
+        _fields_ = [(f, ctypes.c_size_t) for f in ("arena", "ordblks", "smblks", "hblks", "hblkhd", "usmblks",
+                                                   "fsmblks", "uordblks", "fordblks", "keepcost")]
+    libc = ctypes.CDLL("libc.so.6")
+    libc.mallinfo2.restype = Info
+    n = 4400
+    keys, vals = W.make_keys(n, 7).cuda(), W.make_values(n, 7).cuda()
+    t = G.HashTable("bcht", n, 0.9, seed=1)
+    for i in range(1, 401):
+        t.build(keys[:i], vals[:i])
+    before = libc.mallinfo2().uordblks
+    for i in range(401, n + 1):
+        t.build(keys[:i], vals[:i])
+    # 4000 cached sizes of a hash map took over 128 KB
+    assert libc.mallinfo2().uordblks - before < 64 << 10
