@@ -167,7 +167,7 @@ FIND_TRAFFIC = {"bytes_per_launch": 60627704320, "source_sha256_16": "d06cc11ef4
 def build_kernels(st: dict) -> list[str]:
     """The library kernels one build attempt launches, from the table's stats
     (the one-warp kernel that publishes the status to the host aside)."""
-    if st.get("last_fill_ms") == 0.0 and not st["last_build_ranked"]:  # one launch
+    if st.get("last_build_small"):  # one launch
         return ["small_build_kernel"]
     if st["last_build_split"]:  # two grouping levels, block placement, no fill
         return ["region_cursors_kernel", "group_scatter_kernel", "region_cursors_kernel", "group_scatter_kernel",
@@ -181,15 +181,14 @@ def build_kernels(st: dict) -> list[str]:
     return ks + ["bucketed_insert_kernel"]
 
 
-def find_kernels(st: dict, line: bool = False) -> list[str]:
-    """The library kernels one find launches, from the table's stats; line: the
-    table's config names no find shape (tile_lanes, keys_per_lane, find_async)."""
+def find_kernels(st: dict) -> list[str]:
+    """The library kernels one find launches, from the table's stats."""
     if st["last_find_grouped"]:  # per round: two groupings and the lookup; then the return to query order
         rnd = ["region_cursors_kernel", "group_scatter_kernel", "region_cursors_kernel", "group_scatter_kernel",
                "grouped_lookup_kernel"]
         return rnd * st["num_hashes"] + ["grouped_spill_kernel"] + ["region_cursors_kernel", "group_scatter_kernel"] * 2 \
             + ["window_write_kernel"]
-    if line:
+    if st.get("find_line"):
         return ["line_find_kernel"]
     return ["bcht_find_async_kernel" if st["find_staged"] else "bucketed_find_kernel"]
 
@@ -360,9 +359,6 @@ def run_ours(args, world, rank, local):
     phase_ms = {f"{op}@{lf}": [] for lf in LFS
                 for op in ("fill", "group", "split", "place", "insert", "find_pos", "find_neg")}
 
-    # the config names no other find shape than BCHT's default
-    line_find = not args.find_async and args.tile_lanes in (0, 4) and args.keys_per_lane in (0, 2)
-
     def step(record: bool):
         for lf in LFS:
             t = tables[lf]
@@ -377,7 +373,7 @@ def run_ours(args, world, rank, local):
             e1.record()
             t.find(neg, out)
             e2.record()
-            launches[0] += 2 * len(find_kernels(t.stats(), line_find))
+            launches[0] += 2 * len(find_kernels(t.stats()))
             if record:
                 phase_ms[f"fill@{lf}"].append(st["last_fill_ms"])
                 phase_ms[f"group@{lf}"].append(max(st["last_group_ms"], 0.0))
@@ -498,7 +494,7 @@ def run_ours(args, world, rank, local):
     st0 = st_dev
     bks = build_kernels(st0)
     has_fill = "fill_kernel" in bks  # else the placement writes every line: no fill to rate
-    find_name = "+".join(dict.fromkeys(find_kernels(st0, line_find)))
+    find_name = "+".join(dict.fromkeys(find_kernels(st0)))
     for lf in LFS:
         # a build's work after the fill: the grouping (one or two levels) and
         # the ranked placement (when the build does them) and the cuckoo

@@ -176,7 +176,9 @@ typedef struct {
   uint32_t attempts;           /* attempts used by the last build */
   uint32_t max_chain;
   uint32_t hash_a[4], hash_c[4];
-  uint64_t insert_probes;      /* bucket reads by inserts, CAS retries excluded (needs count_probes) */
+  uint64_t insert_probes;      /* bucket visits by inserts, CAS retries excluded (needs count_probes): a
+                                  candidate whose slots were read, or, in a placement or a one-block build,
+                                  its count of keys; victim looks are counted apart */
   uint64_t insert_retries;     /* bucket re-reads after a failed CAS */
   uint64_t insert_evictions;   /* cuckoo exchanges */
   uint64_t longest_chain;      /* most exchanges one insert made (needs count_probes) */
@@ -196,7 +198,7 @@ typedef struct {
   double last_place_ms;        /* device time of its ranked placement (-1 if not two-phase) */
   uint64_t place_overflow;     /* keys the ranked placement left to the cuckoo insert */
   int32_t find_staged;         /* find_async as resolved: 1 if tile_lanes and keys_per_lane are the staged find's
-                                  (which runs where the config names them, the line find where it does not) */
+                                  (which runs unless find_line is 1) */
   int32_t last_build_split;    /* 1 if the last build split its groups into 64 KB sub-groups and placed
                                   each whole in shared memory (block placement, no table fill) */
   /* host-to-device copies of the last ght_build_host / ght_find_host call:
@@ -210,6 +212,12 @@ typedef struct {
    * 64 KB sub-groups of a block placement; -1 if none); last_group_ms is
    * then the first level alone */
   double last_split_ms;
+  int32_t find_line;           /* 1: finds that do not run grouped are the line find, whatever the shape above */
+  int32_t last_build_small;    /* 1: the last build was one launch of one block (last_fill_ms 0, last_insert_ms
+                                  the whole build) */
+  /* full buckets a long eviction chain looked through for a victim that can
+   * move on, each reading up to one sector per slot (needs count_probes) */
+  uint64_t victim_looks;
 } ght_stats_t;
 
 /* Library version string; never NULL. */

@@ -57,6 +57,7 @@ class GhtStats(C.Structure):
         ("find_staged", C.c_int32), ("last_build_split", C.c_int32),
         ("last_h2d_ms", C.c_double), ("last_h2d_bytes", C.c_uint64),
         ("find_grouped", C.c_int32), ("last_find_grouped", C.c_int32), ("last_split_ms", C.c_double),
+        ("find_line", C.c_int32), ("last_build_small", C.c_int32), ("victim_looks", C.c_uint64),
     ]
 
     def as_dict(self) -> dict:

@@ -355,7 +355,7 @@ struct ght_table {
   void *scratch = nullptr;  // caller-owned build scratch (ght_set_build_scratch)
   uint64_t scratch_bytes = 0;
   mutable bool timed_find = false;
-  mutable uint64_t insert_probes = 0, insert_retries = 0, insert_evictions = 0, longest_chain = 0;
+  mutable uint64_t insert_probes = 0, insert_retries = 0, insert_evictions = 0, longest_chain = 0, victim_looks = 0;
 
   void derive(uint32_t attempt) {
     ght::host::derive_constants(seed, attempt, shape.h, a, c);
@@ -925,6 +925,7 @@ int finish_attempt(ght_table *t, uint64_t n, uint32_t attempt, bool grouped, boo
   t->insert_retries = t->h_ctrl->ctrl.insert_retries;
   t->insert_evictions = t->h_ctrl->ctrl.insert_evictions;
   t->longest_chain = t->h_ctrl->ctrl.longest_chain;
+  t->victim_looks = t->h_ctrl->ctrl.victim_looks;
   if (st == 0u) {
     t->built = true;
     t->n_stored = n;
@@ -1384,6 +1385,7 @@ int ght_build_host(ght_table *t, const uint32_t *h_keys, const uint32_t *h_value
         t->insert_retries = t->h_ctrl->ctrl.insert_retries;
         t->insert_evictions = t->h_ctrl->ctrl.insert_evictions;
         t->longest_chain = t->h_ctrl->ctrl.longest_chain;
+        t->victim_looks = t->h_ctrl->ctrl.victim_looks;
         if (st == 0u) {
           t->built = true;
           t->n_stored = n;
@@ -1561,6 +1563,9 @@ int ght_stats(const ght_table *t, ght_stats_t *out) {
   out->insert_retries = t->insert_retries;
   out->insert_evictions = t->insert_evictions;
   out->longest_chain = t->longest_chain;
+  out->victim_looks = t->victim_looks;
+  out->find_line = t->shape.find_line;
+  out->last_build_small = t->timed_build && t->last_small ? 1 : 0;
   out->last_fill_ms = out->last_insert_ms = out->last_find_ms = -1.0;
   float ms = 0.f;
   out->last_group_ms = -1.0;

@@ -573,6 +573,7 @@ int ght_batch_table_stats(const ght_batch *b, uint32_t table, ght_stats_t *out) 
   out->built = b->h_tables[table].status == 0u ? 1 : 0;
   out->tile_lanes = b->find_o.tile_lanes;
   out->keys_per_lane = b->find_o.keys_per_lane;
+  out->find_line = b->find_o.line_find ? 1 : 0;
   out->build_tile_lanes = b->build_o.tile_lanes;
   out->build_keys_per_lane = b->build_o.keys_per_lane;
   out->last_fill_ms = out->last_insert_ms = out->last_find_ms = out->last_group_ms = -1.0;

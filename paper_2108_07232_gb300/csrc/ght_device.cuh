@@ -34,7 +34,8 @@ struct Ctrl {
   unsigned long long find_queries;
   unsigned long long longest_chain;
   unsigned long long work_cursor;  // next input index claimed by an insert
-  unsigned long long reserved[24];
+  unsigned long long reserved[23];
+  unsigned long long victim_looks;  // full buckets whose keys' next buckets were looked at (choose_victims)
 };
 static_assert(sizeof(Ctrl) == 256, "control block is 256 bytes");
 

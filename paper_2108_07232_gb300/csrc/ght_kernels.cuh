@@ -241,7 +241,7 @@ bucketed_insert_kernel(TableView tv, const uint32_t *__restrict__ keys,
     b_a[s] = 0;
     b_b[s] = 0xFFFFFFFFu;
   }
-  unsigned long long probes = 0, retries = 0, evictions = 0, longest = 0;
+  unsigned long long probes = 0, retries = 0, evictions = 0, longest = 0, looks = 0;
   uint32_t round = 0;
 
   for (;;) {
@@ -352,6 +352,7 @@ bucketed_insert_kernel(TableView tv, const uint32_t *__restrict__ keys,
       int victim = -1;
       if (SCHEME == kBCHT) {
         const unsigned look = __ballot_sync(kFull, active[s] && my_empty == 0 && chain[s] >= tv.look && chain[s] < tv.max_chain);
+        if (COUNT) looks += (look >> lane) & 1u;
         if (look != 0u) {
           xorshift32(rng);
           victim = choose_victims<B, G, S>(tv, look, cur[s], tbase, tmask, r, lane, rng);
@@ -465,12 +466,14 @@ bucketed_insert_kernel(TableView tv, const uint32_t *__restrict__ keys,
     probes = warp_sum(probes);
     retries = warp_sum(retries);
     evictions = warp_sum(evictions);
+    looks = warp_sum(looks);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       const unsigned long long other = __shfl_xor_sync(kFull, longest, o);
       longest = other > longest ? other : longest;
     }
     if (lane == 0) {
+      if (looks) atomicAdd(&tv.ctrl->victim_looks, looks);
       atomicAdd(&tv.ctrl->insert_probes, probes);
       atomicAdd(&tv.ctrl->insert_retries, retries);
       atomicAdd(&tv.ctrl->insert_evictions, evictions);

@@ -86,3 +86,56 @@ def test_one_block_builds_of_many_sizes_keep_nothing_per_size(G):
         t.build(keys[:i], vals[:i])
     # 4000 cached sizes of a hash map took over 128 KB
     assert libc.mallinfo2().uordblks - before < 64 << 10
+
+
+# the most keys a scheme builds in one block, and one more
+@pytest.mark.parametrize("scheme,lf,most", [("bcht", 0.96, 18432), ("bcht", 0.97, 8192), ("bcht", 0.99, 8192),
+                                            ("cuckoo1", 0.6, 2048), ("p2bht", 0.75, 20480), ("bcht_lb", 0.9, 20480)])
+@pytest.mark.parametrize("more", [0, 1])
+def test_the_most_keys_of_a_one_block_build(G, scheme, lf, most, more):
+    n = most + more
+    keys, vals = W.make_keys(n, n & 0xFF), W.make_values(n, 9)
+    t = G.HashTable(scheme, n, lf, seed=n)
+    t.build(keys.cuda(), vals.cuda())
+    st = _check(G, t, scheme, keys, vals)
+    assert st["last_build_small"] == 1 - more and st["built"] == 1
+
+
+# the most that fits 226 KB: keys, one index a slot, one count a bucket
+@pytest.mark.parametrize("scheme,lf,b", [("iht", 0.78, 16), ("iht", 0.8, 32), ("bcht_set", 0.95, 32)])
+def test_the_largest_one_block_build(G, scheme, lf, b):
+    def fits(n):
+        return 4 * (n + O.num_buckets(n, lf, b) * (b + 1)) <= 226 * 1024
+
+    most = max(n for n in range(20000, 32769) if fits(n))
+    for n in (most, most + 1):
+        keys, vals = W.make_keys(n, 4), W.make_values(n, 4)
+        t = G.HashTable(scheme, n, lf, seed=7, bucket_size=b)
+        t.build(keys.cuda(), None if scheme == "bcht_set" else vals.cuda())
+        assert _check(G, t, scheme, keys, vals)["last_build_small"] == int(n == most)
+
+
+def test_stats_say_which_kernels_ran(G):
+    """The find that answers, for default and named shapes; the one-block build; and the looks for
+    a victim of long chains, which are no bucket visits: counted where there are any."""
+    n = 3000
+    keys, vals = W.make_keys(n, 1).cuda(), W.make_values(n, 1).cuda()
+    for scheme, cfg, line in (("bcht", {}, 1), ("bcht", {"tile_lanes": 4, "keys_per_lane": 2}, 1),
+                              ("bcht", {"keys_per_lane": 1}, 0), ("bcht", {"tile_lanes": 8}, 0),
+                              ("bcht", {"find_async": -1}, 0), ("bcht", {"find_async": 1}, 0),
+                              ("bcht", {"bucket_size": 32}, 0), ("p2bht", {}, 1), ("iht", {}, 1), ("bcht_lb", {}, 1),
+                              ("cuckoo1", {}, 0), ("bcht_set", {}, 1)):
+        t = G.HashTable(scheme, n, 0.6, seed=2, **cfg)
+        t.build(keys, vals)
+        assert t.stats()["find_line"] == line and t.stats()["last_build_small"] == (scheme != "cuckoo1")
+        t.build(keys[:100], vals[:100])
+    b = G.Batch([n], [0.9], seed=1, tile_lanes=8)
+    assert b.table_stats(0)["find_line"] == 0
+    n = 1 << 20
+    keys, vals = W.make_keys(n, 2).cuda(), W.make_values(n, 2).cuda()
+    for lf, some in ((0.99, True), (0.5, False)):
+        t = G.HashTable("bcht", n, lf, seed=3, count_probes=1)
+        t.build(keys, vals)
+        st = t.stats()
+        assert (st["victim_looks"] > 0) == some
+        assert st["victim_looks"] <= st["insert_evictions"] and st["last_build_small"] == 0
