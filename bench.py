@@ -203,7 +203,7 @@ def kernel_source_hash() -> str:
 
 
 def bytes_per_key(op: str, p: float, lf: float) -> float:
-    """Algorithmic bytes per key (query/result or pair, 128 B per bucket probe,
+    """Algorithmic bytes per key (query/result or pair, 128 B per bucket line read,
     plus one write-back of the table for inserts)."""
     if op == "find":
         return 4 + 4 + 128 * p
@@ -212,6 +212,15 @@ def bytes_per_key(op: str, p: float, lf: float) -> float:
     if op == "fill":
         return 8 / lf
     raise ValueError(op)
+
+
+def build_line_reads(st: dict, n: int) -> float:
+    """Bucket lines a build of n keys reads per key, from a counted build's stats: the visits of its
+    insert. A ranked placement counts one visit for every key but reads no bucket (it counts
+    arrivals), and a one-block build reads none from the table."""
+    if st.get("last_build_small"):
+        return 0.0
+    return st["insert_probes"] / n - (1.0 if st["last_build_ranked"] else 0.0)
 
 
 PROBE_MODES = {0: "random_line_read", 1: "line_read_then_cas", 2: "line_read_then_cas_waited", 3: "atomic_add_only",
@@ -486,7 +495,8 @@ def run_ours(args, world, rank, local):
         tc.find(neg, out)
         p_neg = tc.stats()["find_probes"] / n
         probes[lf] = {"insert": p_ins, "find_pos": p_pos, "find_neg": p_neg,
-                      "insert_retries": st["insert_retries"] / n}
+                      "insert_retries": st["insert_retries"] / n, "insert_line_reads": build_line_reads(st, n),
+                      "victim_looks": st["victim_looks"] / n}
         del tc
 
     peak, peak_src = peaks()
@@ -503,7 +513,7 @@ def run_ours(args, world, rank, local):
                                    zip(phase_ms[f"group@{lf}"], phase_ms[f"split@{lf}"], phase_ms[f"place@{lf}"],
                                        phase_ms[f"insert@{lf}"])]
         for op, key, pp in ((("fill", "fill", 0.0),) if has_fill else ()) + (
-                ("insert", "build", probes[lf]["insert"]), ("find", "find_pos", probes[lf]["find_pos"]),
+                ("insert", "build", probes[lf]["insert_line_reads"]), ("find", "find_pos", probes[lf]["find_pos"]),
                 ("find", "find_neg", probes[lf]["find_neg"])):
             t_ms = statistics.median(phase_ms[f"{key}@{lf}"])
             bpk = bytes_per_key(op, pp, lf)
@@ -540,7 +550,9 @@ def run_ours(args, world, rank, local):
     ceilings = None
     if not args.no_ceilings:
         ceilings = measure_ceilings(tables[LFS[0]].stats()["num_buckets"], n, dev)
-        ins_lines = sum(probes[lf]["insert"] * n for lf in LFS) / sum(kernels[f"build@{lf}"]["ms"] / 1e3 for lf in LFS)
+        # the lines that the insert reads, over its own time (a build's other phases read none)
+        ins_lines = (sum(probes[lf]["insert_line_reads"] * n for lf in LFS)
+                     / sum(statistics.median(phase_ms[f"insert@{lf}"]) / 1e3 for lf in LFS))
         find_lines = (sum((probes[lf]["find_pos"] + probes[lf]["find_neg"]) * n for lf in LFS)
                       / sum((kernels[f"find_pos@{lf}"]["ms"] + kernels[f"find_neg@{lf}"]["ms"]) / 1e3 for lf in LFS))
         ceilings["kernels_glines_s"] = {"find": round(find_lines / 1e9, 2), "insert": round(ins_lines / 1e9, 2)}
