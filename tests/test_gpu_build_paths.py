@@ -30,7 +30,8 @@ def _check(G, t, scheme, keys, vals, b=None):
     got = O._u32(t.find(q.cuda()).cpu())
     want = O.lookup(keys, vals, q)
     assert (got == ((want != O.EMPTY).astype(want.dtype) if sets else want)).all()
-    T = O.Table(O.BCHT if sets else G.SCHEMES[scheme], keys.numel(), 0.5, b=st["bucket_size"], m=st["num_buckets"])
+    T = O.Table(O.BCHT if sets else G.SCHEMES[scheme], keys.numel(), 0.5, b=st["bucket_size"],
+                t=st["threshold"] or None, m=st["num_buckets"])
     T.set_constants(st["hash_a"], st["hash_c"])
     slots = t.export()
     if sets:
@@ -139,3 +140,88 @@ def test_stats_say_which_kernels_ran(G):
         st = t.stats()
         assert (st["victim_looks"] > 0) == some
         assert st["victim_looks"] <= st["insert_evictions"] and st["last_build_small"] == 0
+
+
+# 3648 warps of three blocks, 2432 of two on 152 SMs: around one chunk of 32 keys a warp, around
+# 32, and past it, where the last quarter is claimed
+@pytest.mark.parametrize("n", [33, 116737, 3735553, 5000011])
+@pytest.mark.parametrize("scheme,lf", [("bcht", 0.95), ("p2bht", 0.75), ("iht", 0.8), ("bcht_lb", 0.9), ("bcht_set", 0.95)])
+def test_insert_of_every_key(G, scheme, lf, n):
+    """The insert in input order, which serves builds without scratch."""
+    keys, vals = W.make_keys(n, n & 0xFFF), W.make_values(n, 3)
+    t = G.HashTable(scheme, n, lf, seed=n, group_build=-1, ranked_build=-1)
+    t.build(keys.cuda(), None if scheme == "bcht_set" else vals.cuda())
+    st = _check(G, t, scheme, keys, vals)
+    assert (st["last_build_ranked"], st["last_build_grouped"], st["last_build_small"]) == (0, 0, 0)
+
+
+@pytest.mark.parametrize("scheme,lf", [("p2bht", 0.78), ("iht", 0.8), ("bcht_lb", 0.95), ("cuckoo1", 0.7), ("bcht", 0.95)])
+def test_two_phase_build_from_pageable_arrays(G, scheme, lf):
+    """On request, pageable arrays are placed chunk by chunk as they arrive."""
+    n = 300007
+    keys, vals = W.make_keys(n, 8), W.make_values(n, 8)
+    t = G.HashTable(scheme, n, lf, seed=6, ranked_build=1)
+    t.build(keys, vals)
+    st = _check(G, t, scheme, keys, vals)
+    assert (st["last_build_ranked"], st["last_build_grouped"]) == (1, 0) and st["last_h2d_bytes"] == 8 * n
+
+
+@pytest.mark.parametrize("scheme,lf", [("p2bht", 0.75), ("iht", 0.75), ("bcht_lb", 0.9), ("cuckoo1", 0.7)])
+def test_two_phase_build_from_pageable_arrays_of_two_chunks(G, scheme, lf):
+    n = (1 << 25) + 1001
+    keys, vals = W.make_keys(n, 9), W.make_values(n, 9)
+    t = G.HashTable(scheme, n, lf, seed=6, ranked_build=1)
+    t.build(keys, vals)
+    assert t.stats()["last_build_ranked"] == 1 and t.stats()["n_stored"] == n
+    assert torch.equal(t.find(keys.cuda()), vals.cuda())
+    absent = W.make_negatives(n, 1 << 20, 9).cuda()
+    assert (t.find(absent) == -1).all()
+
+
+@pytest.mark.parametrize("scheme,n,ranked", [("p2bht", 40001, 0), ("p2bht", 700001, 0), ("p2bht", 40001, -1), ("iht", 40001, -1),
+                                             ("iht", 40001, 0)])
+def test_schemes_without_evictions_fail_full_tables(G, scheme, n, ranked):
+    """At load factor 1 some key finds all its candidates full, in the placement by load as in the
+    inserts: every attempt is made, the call says so, and the same table then builds fewer keys."""
+    keys, vals = W.make_keys(n, 2), W.make_values(n, 2)
+    t = G.HashTable(scheme, n, 1.0, seed=4, max_attempts=3, ranked_build=ranked, group_build=-1 if ranked else 0)
+    with pytest.raises(G.GhtError) as e:
+        t.build(keys.cuda(), vals.cuda())
+    assert e.value.status == "GHT_ERR_BUILD_FAILED"
+    assert t.stats()["attempts"] == 3 and t.stats()["built"] == 0
+    most = n // 2
+    t.build(keys[:most].cuda(), vals[:most].cuda())
+    st = _check(G, t, scheme, keys[:most], vals[:most])
+    assert st["last_build_ranked"] == (1 if ranked == 0 else 0) and st["attempts"] == 1
+
+
+def test_load_balanced_overflow_beyond_the_list(G):
+    """Keys whose candidates all lie in an eighth of the buckets under the first constants: the
+    placement by load overflows its list, the attempt is redone with the insert of every key, which
+    cannot hold them either, and the next constants build the table."""
+    n, lf, seed = 40000, 0.8, 13
+    m = O.num_buckets(n, lf, 16)
+    a, c = O.derive_constants(seed, 0, 3)
+    cand = np.arange(1, 1 << 25, dtype=np.uint64)
+    for i in range(3):
+        h = ((np.uint64(a[i]) * cand + np.uint64(c[i])) % np.uint64(O.PRIME)) % np.uint64(m)
+        cand = cand[h < m // 8]
+    crowd = cand[:n].astype(np.uint32)
+    assert crowd.size == n
+    keys, vals = torch.from_numpy(crowd.view(np.int32).copy()), W.make_values(n, 5)
+    t = G.HashTable("bcht_lb", n, lf, seed=seed)
+    t.build(keys.cuda(), vals.cuda())
+    st = _check(G, t, "bcht_lb", keys, vals)
+    assert st["attempts"] == 2 and st["last_build_ranked"] == 1
+
+
+@pytest.mark.parametrize("n", [3000, 60001])
+@pytest.mark.parametrize("threshold", [1, 2, 16, 17])
+def test_iht_thresholds_at_the_ends(G, threshold, n):
+    """From a primary that takes no key at first to one that takes a full bucket, in one block and
+    over the whole device."""
+    keys, vals = W.make_keys(n, 3), W.make_values(n, 3)
+    t = G.HashTable("iht", n, 0.5, seed=2, threshold=threshold)
+    t.build(keys.cuda(), vals.cuda())
+    st = _check(G, t, "iht", keys, vals)
+    assert st["last_build_small"] == (n == 3000) and st["threshold"] == threshold
