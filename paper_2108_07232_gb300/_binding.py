@@ -663,9 +663,10 @@ class Pool:
         return tk
 
     def wait(self, ticket: int, timeout: float = 60.0) -> dict:
-        r = GhtPoolResult()
+        r = GhtPoolResult(status=-1)
         rc = lib().ght_pool_wait(self._p, int(ticket), float(timeout), C.byref(r))
-        self._keep.pop(ticket, None)
+        if r.status >= 0:  # done; a request still pending at the timeout keeps its tensors
+            self._keep.pop(ticket, None)
         if rc != 0:
             raise GhtError(rc, ght_last_error())
         return r.as_dict()

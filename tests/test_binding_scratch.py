@@ -50,3 +50,30 @@ def test_a_grouped_find_without_room_still_fails(table):
     table.room = 1000
     with pytest.raises(torch.OutOfMemoryError):
         table._ensure_find_scratch(10)
+
+
+def test_a_pool_request_keeps_its_tensors_past_a_timeout(monkeypatch):
+    """A wait that runs out leaves the request pending, and the device may still use its arrays."""
+    answers = [(7, None), (0, 0), (7, None), (1, 1)]  # (return code, status written or none)
+
+    class Lib:
+        def ght_pool_submit_find(self, p, t, q, o, n):
+            return 5
+
+        def ght_pool_wait(self, p, ticket, timeout, ref):
+            rc, status = answers.pop(0)
+            if status is not None:
+                ref._obj.status = status
+            return rc
+
+    monkeypatch.setattr(B, "lib", lambda: Lib())
+    monkeypatch.setattr(B, "ght_last_error", lambda: "")
+    pool = B.Pool.__new__(B.Pool)
+    pool._p, pool._keep = None, {}
+    for done in (lambda: pool.wait(5), lambda: pytest.raises(B.GhtError, pool.wait, 5)):
+        ticket = pool.submit_find(0, torch.zeros(3, dtype=torch.int32), torch.zeros(3, dtype=torch.int32))
+        with pytest.raises(B.GhtError):
+            pool.wait(ticket)
+        assert ticket in pool._keep
+        done()
+        assert ticket not in pool._keep
