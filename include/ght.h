@@ -108,7 +108,7 @@ typedef struct {
    * a few MB of the table at a time. 1 = on, -1 = off, 0 = default: on for
    * two-phase builds of tables of at least the device's L2 size. Needs
    * scratch (ght_build_scratch_bytes) and 16-byte aligned key and value
-   * arrays, else the build runs in input order. */
+   * arrays in device memory, else the build runs ungrouped. */
   int32_t group_build;
   /* Two-phase build (tables that fit one SM's shared memory are built there in
    * one launch instead, while group_build, ranked_build and the build shape are
@@ -121,8 +121,8 @@ typedef struct {
    * (ungrouped), the rest of BCHT_LB's by its insert. CUCKOO1: the first key
    * to reach its first choice stays there, the rest are inserted from the
    * second. 1 = on, -1 = off, 0 = default: on where it pays (IHT: while few
-   * keys are expected beyond the threshold; without grouping: tables below
-   * twice the L2; CUCKOO1: tables from the L2's size on). Needs scratch
+   * keys are expected beyond the threshold; ungrouped: tables below twice the
+   * L2; CUCKOO1: grouped, from the L2's size on). Needs scratch
    * (ght_build_scratch_bytes), else the build inserts every key. */
   int32_t ranked_build;
   /* Finds of 128-byte buckets (16 pairs: BCHT with 4-lane tiles, P2BHT, IHT

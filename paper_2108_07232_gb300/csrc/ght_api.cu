@@ -489,21 +489,14 @@ double expected_overflow(uint64_t n, uint64_t m, uint32_t limit) {
   return mean > 0.0 ? (mean - below - limit * (1.0 - cdf)) / mean : 0.0;
 }
 
-// Whether a build of n keys runs in two phases (ranked first-choice
-// placement, then the insert of the overflow; config ranked_build: 1 on, -1
-// off, 0 always where it applies). It costs no bucket read for the keys that
-// find room at once, so it won at every size measured (whole builds, us,
-// input order -> two phases, BCHT at LF 0.9): 2^14 keys 94 -> 81, 2^17 97 ->
-// 85, 2^20 126 -> 105, 2^22 259 -> 154, 2^24 657 -> 411; IHT at LF 0.8: 2^16
-// 110 -> 72, 2^20 181 -> 96, 2^24 1157 -> 487; set at LF 0.95: 2^17 169 ->
-// 100, 50 M keys 2920 -> 968. IHT's overflow, the keys beyond its threshold,
-// has to fit the overflow list: above 0.22 of the keys it builds in input
-// order (low thresholds, or load factors where it rarely succeeds).
-// Ungrouped, the placement's stores and counters go to DRAM one sector each on
-// tables beyond the L2: above twice its size (where 2^28 keys took 17.6 ms
-// against 16.8 in input order) only on request, and so for bucket size one,
-// where every key has a sector of its own (whole builds, us, ungrouped / input
-// order: 13 M keys LF 0.8 961 / 817, 2^24 LF 0.8 1475 / 1286, LF 0.6 1291 / 876).
+// Whether keys are also placed without the grouping (unaligned or host input,
+// no scratch for it, group_build -1). The placement's stores and counters then
+// go to DRAM one sector each on tables beyond the L2. Up to twice its size that
+// still beats the insert (whole builds, us, ungrouped / input order: BCHT 2^24
+// LF 0.95 580 / 721, 25 M keys 928 / 1117; IHT 23 M keys LF 0.8 862 / 1196; set of
+// 50 M keys 1648 / 2884); above only on request (2^28 keys 17.6 ms against
+// 16.8), and so for bucket size one, where every key has a sector of its own (13
+// M keys LF 0.8 961 / 817, 2^24 LF 0.8 1475 / 1286, LF 0.6 1291 / 876).
 bool places_ungrouped(const ght_table *t) {
   return t->shape.ranked_build > 0 ||
          (t->shape.scheme != GHT_CUCKOO1 && t->storage_bytes < 2ull * device_l2_bytes());
@@ -530,6 +523,16 @@ bool wants_small(const ght_table *t, uint64_t n, bool host_input = false) {
   }
 }
 
+// Whether a build of n keys runs in two phases (ranked first-choice
+// placement, then the insert of the overflow; config ranked_build: 1 on, -1
+// off, 0 always where it applies). It costs no bucket read for the keys that
+// find room at once, so it won at every size measured (whole builds, us,
+// input order -> two phases, BCHT at LF 0.9): 2^14 keys 94 -> 81, 2^17 97 ->
+// 85, 2^20 126 -> 105, 2^22 259 -> 154, 2^24 657 -> 411; IHT at LF 0.8: 2^16
+// 110 -> 72, 2^20 181 -> 96, 2^24 1157 -> 487; set at LF 0.95: 2^17 169 ->
+// 100, 50 M keys 2920 -> 968. IHT's overflow, the keys beyond its threshold,
+// has to fit the overflow list: above 0.22 of the keys it builds in input
+// order (low thresholds, or load factors where it rarely succeeds).
 bool wants_ranked(const ght_table *t, uint64_t n, bool host_input = false) {
   if (wants_small(t, n, host_input)) return false;
   const uint32_t limit = place_limit(t->shape);
@@ -1297,7 +1300,7 @@ int ght_build_host(ght_table *t, const uint32_t *h_keys, const uint32_t *h_value
   }
   uint32_t *d_k = static_cast<uint32_t *>(buf), *d_v = d_k + arr / sizeof(uint32_t);
   int rc = GHT_OK;
-  // From host buffers the input-order build overlaps the copies with the
+  // From pageable buffers the input-order build overlaps the copies with the
   // inserts chunk by chunk, which a grouped build cannot (the grouping needs
   // every pair); so here grouping and ranked placement run only on request.
   const bool ranked_wanted = t->shape.ranked_build > 0 && wants_ranked(t, n);

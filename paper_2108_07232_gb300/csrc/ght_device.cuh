@@ -124,7 +124,10 @@ struct ClaimPlan {
 //  * Beyond: three quarters shared evenly, the rest in about eight runs a warp
 //    (each claim is one atomic on one address, ~3 ns apart): 2^24 keys 747 ->
 //    712 us for BCHT at LF 0.95, 1191 -> 1091 for P2BHT and 1073 -> 922 for IHT
-//    at LF 0.8. (Half shared evenly and four runs: 817, 1165, 1040.)
+//    at LF 0.8. (Half shared evenly and four runs: 817, 1165, 1040.) With the
+//    inserts as they are now, this / claims only: BCHT 2^24 664 / 718, 2^26 LF 0.9
+//    2920 / 2983, 2^28 LF 0.99 16855 / 16886; set 2^26 3723 / 3720; P2BHT 2^26 4085
+//    / 4115, IHT 3383 / 3474, load-balanced 5525 / 5552.
 //  * ordered: the input order is a locality order (a grouped input, or a batch
 //    whose tables follow one another), so beyond 8 chunks a warp (0.9 M pairs,
 //    whose buckets the L2 holds in any order) all warps advance together:

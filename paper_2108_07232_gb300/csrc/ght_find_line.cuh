@@ -6,7 +6,7 @@
 // (one instruction, each line once in the L1's pipeline), a warp probes 32
 // queries at a time, one per lane, and a query that needs another bucket waits
 // in shared memory until 32 such queries fill a warp again. So all lanes work
-// in every step and a step is short: about 190 warp instructions for 32
+// in every step and a step is short: 178-181 warp instructions for 32
 // probes, against 415 in the register find (bucketed_find_kernel) and 392 in
 // the staged find (bcht_find_async_kernel), and with 64 registers a thread 32
 // warps fit on an SM instead of 16 and 12. That hides the latency of 1024
