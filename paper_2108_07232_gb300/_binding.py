@@ -351,6 +351,8 @@ class HashTable:
     """One static table whose storage is a torch tensor on the current CUDA
     device. Work follows torch's current stream at each call."""
 
+    _scratch_bytes = 0  # of the scratch that builds have taken so far
+
     def __init__(self, scheme, capacity: int, load_factor: float, seed: int = 0, device=None,
                  **config):
         import torch
@@ -419,11 +421,16 @@ class HashTable:
                 raise ValueError("keys and values differ in length")
         with _device_of(self.device):
             self._stream()
-            self._ensure_scratch(ght_build_scratch_bytes_for(self._t, k, v, k.numel(), not k.is_cuda))
+            n = k.numel()
+            need = ght_build_scratch_bytes(self._t, n)  # at most, whatever the arrays
+            if need > self._scratch_bytes:
+                need = ght_build_scratch_bytes_for(self._t, k, v, n, not k.is_cuda)
+                if need > self._scratch_bytes:
+                    self._ensure_scratch(need)
             if k.is_cuda:
-                ght_build(self._t, k, v, k.numel())
+                ght_build(self._t, k, v, n)
             else:
-                ght_build_host(self._t, k, v, k.numel())
+                ght_build_host(self._t, k, v, n)
 
     def _ensure_scratch(self, need: int) -> None:
         """Two-phase and grouped builds need scratch; it is a torch tensor kept with the table.
@@ -440,8 +447,7 @@ class HashTable:
 
     def _ensure_bytes(self, need: int) -> None:
         import torch
-        have = getattr(self, "_scratch_bytes", 0)
-        if need and need > have:
+        if need > self._scratch_bytes:
             self._scratch = torch.empty(need + 256, dtype=torch.uint8, device=self.device)
             base = self._scratch.data_ptr()
             ght_set_build_scratch(self._t, (base + 255) & ~255, need)
@@ -449,7 +455,7 @@ class HashTable:
 
     def release_scratch(self) -> None:
         """Drop the build scratch (later builds insert every key with the cuckoo insert until re-set)."""
-        if getattr(self, "_scratch_bytes", 0):
+        if self._scratch_bytes:
             ght_set_build_scratch(self._t, None, 0)
             self._scratch = None
             self._scratch_bytes = 0
