@@ -669,9 +669,9 @@ class Pool:
         return tk
 
     def wait(self, ticket: int, timeout: float = 60.0) -> dict:
-        r = GhtPoolResult(status=-1)
+        r = GhtPoolResult()
         rc = lib().ght_pool_wait(self._p, int(ticket), float(timeout), C.byref(r))
-        if r.status >= 0:  # done; a request still pending at the timeout keeps its tensors
+        if rc == 0 or r.status != 0:  # done; a request still pending at the timeout keeps its tensors
             self._keep.pop(ticket, None)
         if rc != 0:
             raise GhtError(rc, ght_last_error())

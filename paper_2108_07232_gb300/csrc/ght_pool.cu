@@ -146,18 +146,20 @@ bool ght_pool::answers_over_queries(const uint32_t *const *src, uint32_t *const 
                                     uint32_t R) {
   auto at = [](const void *p) { return reinterpret_cast<uintptr_t>(p); };
   uintptr_t s_lo = ~(uintptr_t)0, s_hi = 0, d_lo = ~(uintptr_t)0, d_hi = 0;
-  starts.clear();
-  ends.clear();
   for (uint32_t i = 0; i < R; ++i) {
     const uint64_t bytes = (offs[i + 1] - offs[i]) * sizeof(uint32_t);
-    starts.push_back(at(src[i]));
-    ends.push_back(at(src[i]) + bytes);
-    s_lo = std::min(s_lo, starts[i]);
-    s_hi = std::max(s_hi, ends[i]);
+    s_lo = std::min(s_lo, at(src[i]));
+    s_hi = std::max(s_hi, at(src[i]) + bytes);
     d_lo = std::min(d_lo, at(dst[i]));
     d_hi = std::max(d_hi, at(dst[i]) + bytes);
   }
   if (d_hi <= s_lo || s_hi <= d_lo) return false;
+  starts.clear();
+  ends.clear();
+  for (uint32_t i = 0; i < R; ++i) {
+    starts.push_back(at(src[i]));
+    ends.push_back(at(src[i]) + (offs[i + 1] - offs[i]) * sizeof(uint32_t));
+  }
   std::sort(starts.begin(), starts.end());
   std::sort(ends.begin(), ends.end());
   for (uint32_t i = 0; i < R; ++i) {
