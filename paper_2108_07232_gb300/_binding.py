@@ -422,8 +422,8 @@ class HashTable:
         with _device_of(self.device):
             self._stream()
             n = k.numel()
-            need = ght_build_scratch_bytes(self._t, n)  # at most, whatever the arrays
-            if need > self._scratch_bytes:
+            need = ght_build_scratch_bytes(self._t, n) if k.is_cuda else None  # at most, for device arrays
+            if need is None or need > self._scratch_bytes:
                 need = ght_build_scratch_bytes_for(self._t, k, v, n, not k.is_cuda)
                 if need > self._scratch_bytes:
                     self._ensure_scratch(need)

@@ -594,7 +594,7 @@ bool sub_shape(const Shape &s, uint64_t n, int shift, uint32_t region1, SubShape
 // in a region of `region` pairs when the build places by rank (0: exact
 // offsets, `len` = n entries); split: the groups are split into sub-groups,
 // which are placed by one block each in shared memory; keys_only: a set's
-// split, whose two levels move no values (50 M keys: 521 MB of scratch with
+// split, whose two levels move no values (50 M keys: 525 MB of scratch with
 // the placement's, 943 with value arrays).
 struct GroupPlan {
   int shift = 0;

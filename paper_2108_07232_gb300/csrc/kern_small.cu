@@ -307,8 +307,8 @@ static cudaError_t launch_small(const TableView &tv, const uint32_t *k, const ui
 // Values that do not fit beside the keys are gathered 4 bytes at a time when the
 // table is written. From host memory that takes L1, which the lines fetched over
 // the link stay in: none is left beside more than 195 KB. Builds from page-locked
-// arrays, us, this / two phases: IHT LF 0.78 21,000 keys (198 KB) 65 / 71, 22,000
-// (208 KB) 121 / 72; LF 0.6 18,000 (199 KB) 55 / 60, 19,000 (210 KB) 104 / 59;
+// arrays, us, this / two phases: IHT LF 0.78 21,000 keys (194 KB) 65 / 71, 22,000
+// (203 KB) 121 / 72; LF 0.6 18,000 (195 KB) 55 / 60, 19,000 (206 KB) 104 / 59;
 // P2BHT LF 0.6 18,000 61 / 60, 19,000 109 / 59.
 bool small_build_fits(int B, bool key_slots, uint64_t m, uint64_t n, bool far_values) {
   const uint64_t smem = small_build_smem(B, m, n);

@@ -77,3 +77,11 @@ def test_a_pool_request_keeps_its_tensors_past_a_timeout(monkeypatch):
         assert ticket in pool._keep
         done()
         assert ticket not in pool._keep
+
+
+def test_host_arrays_are_asked_for_by_what_they_are(table, monkeypatch):
+    """A build that needs no scratch from device arrays may need some from page-locked ones."""
+    monkeypatch.setattr(B, "ght_build_scratch_bytes", lambda *a: 0)
+    keys = torch.arange(10, dtype=torch.int32)
+    table.build(keys, keys)
+    assert table.calls == [("scratch", 1 << 20), ("build", 10)]
