@@ -122,8 +122,10 @@ typedef struct {
    * to reach its first choice stays there, the rest are inserted from the
    * second. 1 = on, -1 = off, 0 = default: on where it pays (IHT: while few
    * keys are expected beyond the threshold; ungrouped: tables below twice the
-   * L2; CUCKOO1: grouped, from the L2's size on). Needs scratch
-   * (ght_build_scratch_bytes), else the build inserts every key. */
+   * L2; CUCKOO1: grouped, from the L2's size and 6 M keys on, where builds are
+   * 20-45 % shorter and finds of present keys 2-10 % longer than after an insert
+   * in input order). Needs scratch (ght_build_scratch_bytes), else the build
+   * inserts every key. */
   int32_t ranked_build;
   /* Finds of 128-byte buckets (16 pairs: BCHT with 4-lane tiles, P2BHT, IHT
    * and the load-balanced BCHT, whose find tiles then have 4 lanes; the

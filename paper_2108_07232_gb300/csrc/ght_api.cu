@@ -542,9 +542,16 @@ bool wants_ranked(const ght_table *t, uint64_t n, bool host_input = false) {
   // bucket size one: only grouped (below), where the placement keeps the first
   // exchange of the 60-75 % of keys that find their slot empty from DRAM (whole
   // builds, us: 2^24 keys LF 0.8 1272 -> 941, LF 0.6 854 -> 684, 2^25 LF 0.5 2008 ->
-  // 1292); inside the L2 it gains nothing (2^22 LF 0.8 282 / 290, 2^23 435 / 454)
+  // 1292); inside the L2 it gains nothing (2^22 LF 0.8 282 / 290, 2^23 435 / 454),
+  // and a large table with few keys costs the passes over all of it (tables for
+  // 16.8 M keys, input order -> two phases: 2.1 M keys 128 -> 178, 4 M 183 -> 203, 6 M
+  // 247 -> 247, 8 M 323 -> 304; for 67 M: 2.1 M 229 -> 350, 4 M 308 -> 367, 6 M 396 ->
+  // 395, 8 M 482 -> 424). Finds of present keys pay some of it back: the overflow
+  // starts at H_1, so fewer keys stay at H_0 (LF 0.8 1.86 probes, 1.79 in input
+  // order; 2^24 keys 380 us against 373, 2^26 2790 / 2590; with the overflow started
+  // at H_0 2730, and builds of 2^24 keys 1155 us instead of 947).
   if (t->shape.scheme == GHT_CUCKOO1 && t->shape.ranked_build <= 0 &&
-      (t->shape.group_build < 0 || t->storage_bytes < device_l2_bytes()))
+      (t->shape.group_build < 0 || t->storage_bytes < device_l2_bytes() || n < 6000000u))
     return false;
   if (t->shape.group_build < 0 && !places_ungrouped(t)) return false;
   return t->shape.scheme != GHT_IHT || expected_overflow(n, t->shape.m, limit) <= 0.22;

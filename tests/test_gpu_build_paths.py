@@ -225,3 +225,14 @@ def test_iht_thresholds_at_the_ends(G, threshold, n):
     t.build(keys.cuda(), vals.cuda())
     st = _check(G, t, "iht", keys, vals)
     assert st["last_build_small"] == (n == 3000) and st["threshold"] == threshold
+
+
+@pytest.mark.parametrize("n,two_phase", [(6000000, 1), (5999999, 0), (1000, 0)])
+def test_few_keys_in_a_large_table_of_bucket_size_one(G, n, two_phase):
+    keys, vals = W.make_keys(n, 4), W.make_values(n, 4)
+    t = G.HashTable("cuckoo1", 1 << 24, 0.8, seed=2)
+    t.build(keys.cuda(), vals.cuda())
+    st = t.stats()
+    assert (st["last_build_ranked"], st["last_build_grouped"], st["n_stored"]) == (two_phase, two_phase, n)
+    q = W.make_queries(keys, 1 << 20, 0.5, seed=3)
+    assert (O._u32(t.find(q.cuda()).cpu()) == O.lookup(keys, vals, q)).all()
